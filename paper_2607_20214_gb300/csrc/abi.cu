@@ -681,7 +681,8 @@ int forward_impl(const elsaa_params *params, const void *q, const void *k,
                                    return launch_topk(
                                        sg, P, q, k, pq, pk,
                                        (float *)(ws + P.off_sums), cand,
-                                       selmask, status, st);
+                                       selmask, (float *)keyrank, status,
+                                       st);  // keyrank is spent by now
                                }),
                                kStage[sg]);
         const size_t pb = (size_t)P.BH * P.N * sizeof(int32_t);

@@ -106,12 +106,20 @@ struct GateFusion {
 
 // Per-query top-k selector (topk.cu).
 bool topk_supported(const Plan &P, const char **msg);
-// stage 0: block sums; 1: candidate blocks; 2: per-query selection
+// stage 0: block sums; 1: candidate blocks; 2: per-query selection. norms:
+// 2 B H N floats of scratch from stage 0 to stage 2.
 cudaError_t launch_topk(int stage, const Plan &P, const void *q,
                         const void *k, const int32_t *perm_q,
                         const int32_t *perm_k, float *sums, int32_t *cand,
-                        uint32_t *selmask, DeviceStatus *status,
+                        uint32_t *selmask, float *norms, DeviceStatus *status,
                         cudaStream_t st);
+// The selection on the tensor cores (topk_tc.cu).
+bool topk_tc_supported(const Plan &P);
+cudaError_t launch_topk_select_tc(const Plan &P, const void *q, const void *k,
+                                  const int32_t *perm_q,
+                                  const int32_t *perm_k, const int32_t *cand,
+                                  const float *norms, uint32_t *selmask,
+                                  DeviceStatus *status, cudaStream_t st);
 cudaError_t launch_topk_export(const Plan &P, const int32_t *perm_q,
                                const int32_t *perm_k, const int32_t *cand,
                                const uint32_t *selmask, int32_t *out,

@@ -36,116 +36,166 @@ __device__ __forceinline__ uint32_t ordered_key(float f) {
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
-// Grid (T, BH, 2), d threads: sums[w][bh][t][e] over the sorted positions
-// [t b, (t + 1) b) of queries (w = 0) or keys (w = 1).
-template <typename X>
-__global__ void k_topk_sums(const X *__restrict__ qx, const X *__restrict__ kx,
-                            const int32_t *__restrict__ perm_q,
-                            const int32_t *__restrict__ perm_k, int N, int d,
-                            int b, float *__restrict__ sums,
-                            DeviceStatus *status) {
-    const int t = blockIdx.x, bh = blockIdx.y, w = blockIdx.z;
-    const int T = gridDim.x, BH = gridDim.y, e = threadIdx.x;
-    const X *x = (w ? kx : qx) + (size_t)bh * N * d;
+// Reads d / 32 consecutive values of a row (one load of 2 to 16 bytes).
+template <typename X, int CPL>
+struct __align__(sizeof(X) * CPL) RowPiece {
+    X v[CPL];
+};
+
+// One warp per (block t, head, Q|K): sums[w][bh][t][e] over the sorted
+// positions [t b, (t + 1) b) of queries (w = 0) or keys (w = 1), each lane
+// holding d / 32 columns, and norms[w][bh][p] = |x|^2 of every row (used as
+// an error bound by the tensor-core selection; NULL: not wanted). Rows are
+// loaded whole, kU at a time; the additions stay in sorted order. The row
+// norms of 32 rows are reduced together (one shuffle per row). Bound by the
+// read of Q and K: one thread per column and two-byte loads took 132 us at
+// B2 H16 N16384 d128, this kernel 85 us (beside the RACE key side in both).
+template <typename X, int CPL>
+__global__ void __launch_bounds__(kSelThreads)
+    k_topk_sums(const X *__restrict__ qx, const X *__restrict__ kx,
+                const int32_t *__restrict__ perm_q,
+                const int32_t *__restrict__ perm_k, int N, int b,
+                float *__restrict__ sums, float *__restrict__ norms,
+                DeviceStatus *status) {
+    constexpr int d = 32 * CPL, kU = 16;
+    const int lane = threadIdx.x & 31, T = N / b;
+    const int t = blockIdx.x * kSelWarps + (threadIdx.x >> 5);
+    const int bh = blockIdx.y, BH = gridDim.y, w = blockIdx.z;
+    if (t >= T) return;  // whole warps
+    const X *x = (w ? kx : qx) + (size_t)bh * N * d + lane * CPL;
     const int32_t *pm = (w ? perm_k : perm_q) + (size_t)bh * N;
-    // rows 16 at a time: the loads are issued together, the additions stay
-    // in sorted order
-    constexpr int kU = 16;
-    float acc = 0.0f;
-    for (int p0 = t * b; p0 < (t + 1) * b; p0 += kU) {
-        float v[kU];
+    float acc[CPL];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) {
-            int i = pm[p0 + u];
-            if (i < 0 || i >= N) {
-                if (e == 0) report(status, kDevPermRange, 20, bh, i);
-                i = 0;
-            }
-            v[u] = to_f32<X>(x[(size_t)i * d + e]);
+    for (int e = 0; e < CPL; ++e) acc[e] = 0.0f;
+    int ahead = pm[t * b + lane];
+    for (int p0 = t * b; p0 < (t + 1) * b; p0 += 32) {
+        int i = ahead;
+        if (p0 + 32 < (t + 1) * b) ahead = pm[p0 + 32 + lane];
+        if (i < 0 || i >= N) {
+            report(status, kDevPermRange, 20, bh, i);
+            i = 0;
         }
+        float sq[32];
 #pragma unroll
-        for (int u = 0; u < kU; ++u) acc = __fadd_rn(acc, v[u]);
+        for (int h = 0; h < 32; h += kU) {
+            RowPiece<X, CPL> v[kU];
+#pragma unroll
+            for (int u = 0; u < kU; ++u)
+                v[u] = *reinterpret_cast<const RowPiece<X, CPL> *>(
+                    x + (size_t)__shfl_sync(0xffffffffu, i, h + u) * d);
+#pragma unroll
+            for (int u = 0; u < kU; ++u) {
+                float s = 0.0f;
+#pragma unroll
+                for (int e = 0; e < CPL; ++e) {
+                    const float f = to_f32<X>(v[u].v[e]);
+                    acc[e] = __fadd_rn(acc[e], f);
+                    s = fmaf(f, f, s);
+                }
+                sq[h + u] = s;
+            }
+        }
+        if (norms) {
+            // lane l ends with the sum over lanes of sq[l]
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int u = 0; u < o; ++u) {
+                    const bool up = lane & o;
+                    const float give = up ? sq[u] : sq[u + o];
+                    sq[u] = (up ? sq[u + o] : sq[u]) +
+                            __shfl_xor_sync(0xffffffffu, give, o);
+                }
+            norms[((size_t)w * BH + bh) * N + p0 + lane] = sq[0];
+        }
     }
-    sums[(((size_t)w * BH + bh) * T + t) * d + e] = acc;
+    float *out = sums + (((size_t)w * BH + bh) * T + t) * d + lane * CPL;
+#pragma unroll
+    for (int e = 0; e < CPL; ++e) out[e] = acc[e];
 }
 
-// Grid (T, BH), kSelThreads threads; dynamic shared memory: T scores, T
-// flags, the block's query sum. cand[bh][t][0 .. c) = t, then the c - 1
-// blocks u != t of largest score in order (equal scores: lower u).
+// Grid (ceil(T / G), BH), kSelThreads threads: G query blocks per CTA, so
+// every block sum of the keys that is read feeds G chains (one block per
+// CTA had taken 72 us at T = 128, BH = 32: the strided reads of the sums
+// bound it; this kernel 20 us). Dynamic shared memory: the G query sums,
+// G x T scores, G x T flags. cand[bh][t][0 .. c) = t, then the c - 1 blocks
+// u != t of largest score in order (equal scores: lower u).
+template <int G>
 __global__ void __launch_bounds__(kSelThreads)
-    k_topk_cand(const float *__restrict__ sums, int d, int c,
+    k_topk_cand(const float *__restrict__ sums, int T, int d, int c,
                 int32_t *__restrict__ cand) {
-    extern __shared__ float csm[];
-    const int t = blockIdx.x, bh = blockIdx.y;
-    const int T = gridDim.x, BH = gridDim.y;
+    extern __shared__ __align__(16) float csm[];
+    const int t0 = blockIdx.x * G, bh = blockIdx.y, BH = gridDim.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    float *qs = csm;                     // [d]
-    float *sc = qs + d;                  // [T]
-    int *taken = reinterpret_cast<int *>(sc + T);  // [T]
-    __shared__ float bs[kSelWarps];
-    __shared__ int bu[kSelWarps];
-    const float *qsum = sums + ((size_t)bh * T + t) * d;
+    const int ng = min(G, T - t0);
+    float *qs = csm;         // [G][d]
+    float *sc = qs + G * d;  // [G][T]
+    unsigned char *taken = reinterpret_cast<unsigned char *>(sc + G * T);
+    const float *qsum = sums + ((size_t)bh * T + t0) * d;
     const float *ksum = sums + ((size_t)(BH + bh) * T) * d;
-    for (int e = tid; e < d; e += kSelThreads) qs[e] = qsum[e];
+    for (int e = tid; e < G * d; e += kSelThreads)
+        qs[e] = e < ng * d ? qsum[e] : 0.0f;
     __syncthreads();
     for (int u = tid; u < T; u += kSelThreads) {
         const float4 *kr = reinterpret_cast<const float4 *>(ksum +
                                                              (size_t)u * d);
-        float acc = 0.0f;
+        float acc[G];
+#pragma unroll
+        for (int g = 0; g < G; ++g) acc[g] = 0.0f;
         for (int e = 0; e < d; e += 16) {
             float4 kv[4];
 #pragma unroll
             for (int x = 0; x < 4; ++x) kv[x] = kr[e / 4 + x];
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-                acc = fmaf(qs[e + 4 * x], kv[x].x, acc);
-                acc = fmaf(qs[e + 4 * x + 1], kv[x].y, acc);
-                acc = fmaf(qs[e + 4 * x + 2], kv[x].z, acc);
-                acc = fmaf(qs[e + 4 * x + 3], kv[x].w, acc);
-            }
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const float4 qv = *reinterpret_cast<const float4 *>(
+                        qs + g * d + e + 4 * x);
+                    acc[g] = fmaf(qv.x, kv[x].x, acc[g]);
+                    acc[g] = fmaf(qv.y, kv[x].y, acc[g]);
+                    acc[g] = fmaf(qv.z, kv[x].z, acc[g]);
+                    acc[g] = fmaf(qv.w, kv[x].w, acc[g]);
+                }
         }
-        sc[u] = acc;
-        taken[u] = u == t;
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            sc[g * T + u] = acc[g];
+            taken[g * T + u] = u == t0 + g;
+        }
     }
     __syncthreads();
-    int32_t *out = cand + ((size_t)bh * T + t) * c;
-    if (tid == 0) out[0] = t;
-    for (int m = 1; m < c; ++m) {
-        // (score, u) lexicographic best: larger score, then lower u
-        float best = 0.0f;
-        int bu_ = -1;
-        for (int u = tid; u < T; u += kSelThreads)
-            if (!taken[u] && (bu_ < 0 || sc[u] > best)) {
-                best = sc[u];
-                bu_ = u;
-            }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-            const int ou = __shfl_xor_sync(0xffffffffu, bu_, o);
-            if (ou >= 0 && (bu_ < 0 || ob > best || (ob == best && ou < bu_))) {
-                best = ob;
-                bu_ = ou;
-            }
-        }
-        if (lane == 0) {
-            bs[warp] = best;
-            bu[warp] = bu_;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            float b0 = 0.0f;
-            int u0 = -1;
-            for (int w = 0; w < kSelWarps; ++w)
-                if (bu[w] >= 0 &&
-                    (u0 < 0 || bs[w] > b0 || (bs[w] == b0 && bu[w] < u0))) {
-                    b0 = bs[w];
-                    u0 = bu[w];
+    for (int g = warp; g < ng; g += kSelWarps) {
+        int32_t *out = cand + ((size_t)bh * T + t0 + g) * c;
+        const float *s = sc + g * T;
+        unsigned char *tk = taken + g * T;
+        if (lane == 0) out[0] = t0 + g;
+        for (int m = 1; m < c; ++m) {
+            // (score, u) lexicographic best: larger score, then lower u
+            float best = 0.0f;
+            int bu = -1;
+            for (int u = lane; u < T; u += 32)
+                if (!tk[u] && (bu < 0 || s[u] > best)) {
+                    best = s[u];
+                    bu = u;
                 }
-            out[m] = u0;
-            if (u0 >= 0) taken[u0] = 1;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int ou = __shfl_xor_sync(0xffffffffu, bu, o);
+                if (ou >= 0 &&
+                    (bu < 0 || ob > best || (ob == best && ou < bu))) {
+                    best = ob;
+                    bu = ou;
+                }
+            }
+            bu = __shfl_sync(0xffffffffu, bu, 0);
+            if (lane == 0) {
+                out[m] = bu;
+                if (bu >= 0) tk[bu] = 1;
+            }
+            __syncwarp();
         }
-        __syncthreads();
     }
 }
 
@@ -505,31 +555,48 @@ bool topk_supported(const Plan &P, const char **msg) {
 cudaError_t launch_topk(int stage, const Plan &P, const void *q,
                         const void *k, const int32_t *perm_q,
                         const int32_t *perm_k, float *sums, int32_t *cand,
-                        uint32_t *selmask, DeviceStatus *status,
+                        uint32_t *selmask, float *norms, DeviceStatus *status,
                         cudaStream_t st) {
     const int T = P.N / P.b;
     if (stage == 0) {
-    dim3 gs(T, P.BH, 2);
-    if (P.dtype == ELSAA_FP32)
-        k_topk_sums<float><<<gs, P.d, 0, st>>>(
-            (const float *)q, (const float *)k, perm_q, perm_k, P.N, P.d, P.b,
-            sums, status);
-    else
-        k_topk_sums<__nv_bfloat16><<<gs, P.d, 0, st>>>(
-            (const __nv_bfloat16 *)q, (const __nv_bfloat16 *)k, perm_q,
-            perm_k, P.N, P.d, P.b, sums, status);
-        return cudaGetLastError();
+        dim3 gs((T + kSelWarps - 1) / kSelWarps, P.BH, 2);
+        auto run = [&](auto kern, auto *qp, auto *kp) {
+            kern<<<gs, kSelThreads, 0, st>>>(
+                qp, kp, perm_q, perm_k, P.N, P.b, sums,
+                topk_tc_supported(P) ? norms : nullptr, status);
+            return cudaGetLastError();
+        };
+        auto *qf = (const float *)q, *kf = (const float *)k;
+        auto *qb = (const __nv_bfloat16 *)q, *kb = (const __nv_bfloat16 *)k;
+        const bool f32 = P.dtype == ELSAA_FP32;
+        switch (P.d) {
+            case 32:
+                return f32 ? run(k_topk_sums<float, 1>, qf, kf)
+                           : run(k_topk_sums<__nv_bfloat16, 1>, qb, kb);
+            case 64:
+                return f32 ? run(k_topk_sums<float, 2>, qf, kf)
+                           : run(k_topk_sums<__nv_bfloat16, 2>, qb, kb);
+            default:
+                return f32 ? run(k_topk_sums<float, 4>, qf, kf)
+                           : run(k_topk_sums<__nv_bfloat16, 4>, qb, kb);
+        }
     }
     if (stage == 1) {
-        const size_t csm = (size_t)P.d * 4 + (size_t)T * 8;
-        if (csm > 48 * 1024)
-            cudaFuncSetAttribute(k_topk_cand,
+        // eight query blocks per CTA while their scores fit 83 KB
+        auto run = [&](auto kern, int G) {
+            const size_t csm = (size_t)G * P.d * 4 + (size_t)G * T * 5;
+            cudaFuncSetAttribute(kern,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)csm);
-        k_topk_cand<<<dim3(T, P.BH), kSelThreads, csm, st>>>(sums, P.d,
-                                                             P.tk_c, cand);
-        return cudaGetLastError();
+            kern<<<dim3((T + G - 1) / G, P.BH), kSelThreads, csm, st>>>(
+                sums, T, P.d, P.tk_c, cand);
+            return cudaGetLastError();
+        };
+        return T <= 2048 ? run(k_topk_cand<8>, 8) : run(k_topk_cand<2>, 2);
     }
+    if (topk_tc_supported(P))
+        return launch_topk_select_tc(P, q, k, perm_q, perm_k, cand, norms,
+                                     selmask, status, st);
     const size_t smem = select_smem(P);
     auto run = [&](auto kern, auto *qp, auto *kp) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
