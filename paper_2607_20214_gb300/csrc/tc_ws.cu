@@ -30,6 +30,8 @@
 #include "tc_common.cuh"
 #include "tc_race.cuh"
 
+#include <type_traits>
+
 namespace elsaa {
 
 namespace {
@@ -47,10 +49,11 @@ constexpr int kWsNK = 128;        // keys per query tile
 // [0, 128) go to quarters 1 and 3, buckets [128, 256) to quarters 0 and 2
 // once the P V product is done.
 
+template <int QS, int VS>
 struct WsBars {
-    uint64_t qk_full, wb_full, head_done;
+    uint64_t qk_full[QS], wb_full, head_done;
     uint64_t idx_full[2], idx_empty[2];
-    uint64_t v_full[2], v_empty[2], pv0_done[2];
+    uint64_t v_full[VS], v_empty[VS], pv0_done[2];
     uint64_t s_full[2], p_full[2], pv_done[2], p2_full[2], o_full[2];
     uint64_t tmem_empty[2];
 };
@@ -64,7 +67,15 @@ struct WsBars {
 // (cand, tk_c per query block), each key masked unless the row's bit in
 // selmask is set. The checks of the other modes are compiled out. O32: O
 // is written as fp32 (out_fp32), each thread storing its half row directly.
-template <int G, int NPASS, int KM, bool O32 = false>
+// QS: buffers of the Q and key tiles (one pass per tile when > 1), so that
+// the rows of tile t + QS are copied while tiles t + 1 .. t + QS - 1 wait
+// for their scores, with as many value buffers (d = 64; O then leaves from
+// registers, and a value buffer is free as soon as its product is done).
+// KB: b when it is 32 or 64 (0: any b). The 32 rows of a warp then share one
+// key block of KB scores, half for each of the row's two threads, kept in
+// registers between the maximum and the exponentials; the general path
+// takes all 128 columns with a mask.
+template <int G, int NPASS, int KM, bool O32 = false, int QS = 1, int KB = 0>
 __global__ void __launch_bounds__(kWsThreads, 1)
     k_block_attn_ws(const uint16_t *__restrict__ qx,
                     const uint16_t *__restrict__ kx,
@@ -86,10 +97,14 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                     const int32_t *__restrict__ cand,
                     const uint32_t *__restrict__ selmask, int tk_c) {
     constexpr bool WIN = KM == 1, SEL = KM == 2;
+    constexpr int VS = QS > 2 ? QS : 2;  // value buffers
+    static_assert((QS == 1 && KB == 0) || (NPASS == 1 && KM == 0),
+                  "one pass per tile");
+    constexpr bool DIRECT = QS > 1 && !O32;  // O stored from registers
     constexpr int R = 1 << G;
     constexpr int nk = kWsNK;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ WsBars bars;
+    __shared__ WsBars<QS, VS> bars;
     __shared__ uint32_t tbase;
     __shared__ int abort_flag;
     __shared__ float xmax[2][2][128], xsum[2][2][128], xden[2][2][128];
@@ -112,23 +127,27 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     // TMEM columns [0, 128) and [128, 128 + Lg_pad)
     const int NR = nk + Lg_pad;
     const uint32_t sQ = base;
-    const uint32_t sKW = sQ + tileB;
-    const uint32_t sV0 = sKW + align1k((uint32_t)NR * d * 2u);
-    const uint32_t sB = sV0 + 2 * tileB;
+    const uint32_t sKW = sQ + QS * tileB;
+    const uint32_t tileKW = align1k((uint32_t)NR * d * 2u);
+    const uint32_t sV0 = sKW + QS * tileKW;
+    const uint32_t sB = sV0 + VS * tileB;
     const uint32_t sA = sB + align1k(r * d * 2);  // fp32 [r]
     const float *Asm = reinterpret_cast<const float *>(smem_raw + (sA - smem_u32(smem_raw)));
 
     if (warp == kWsMmaWarp) tmem_alloc(&tbase, 512);
     if (tid == 0) {
-        mbar_init(&bars.qk_full, 256);  // the issuing slot's threads
+        // the issuing slot's threads
+        for (int s = 0; s < QS; ++s) mbar_init(&bars.qk_full[s], 256);
+        for (int s = 0; s < VS; ++s) {
+            mbar_init(&bars.v_full[s], kWsLoaders);
+            mbar_init(&bars.v_empty[s], 1);
+        }
         mbar_init(&bars.wb_full, 1);
         mbar_init(&bars.head_done, 1);
         for (int s = 0; s < 2; ++s) {
             mbar_init(&bars.idx_full[s], kWsLoaders);
             mbar_init(&bars.idx_empty[s], 256 * NPASS);
             mbar_init(&bars.pv0_done[s], 1);
-            mbar_init(&bars.v_full[s], kWsLoaders);
-            mbar_init(&bars.v_empty[s], 1);
             mbar_init(&bars.s_full[s], 1);
             mbar_init(&bars.p_full[s], 256);
             mbar_init(&bars.pv_done[s], 1);
@@ -246,10 +265,14 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 if (i > 0 && !lwait(&bars.head_done, (hc - 1) & 1, 31)) break;
                 if (lt == 0) {  // TMA: planes under the key rows, B, A
                     mbar_expect_tx(&bars.wb_full,
-                                   (uint32_t)(Lg_pad + r) * d * 2u + r * 4u);
+                                   (uint32_t)(QS * Lg_pad + r) * d * 2u +
+                                       r * 4u);
                     for (int p = 0; p < (d >> 6); ++p) {
-                        tma_load_2d(sKW + p * NR * 128 + nk * 128, &tmW,
-                                    64 * p, (bh % H) * Lg_pad, &bars.wb_full);
+                        for (int q = 0; q < QS; ++q)
+                            tma_load_2d(
+                                sKW + q * tileKW + p * NR * 128 + nk * 128,
+                                &tmW, 64 * p, (bh % H) * Lg_pad,
+                                &bars.wb_full);
                         tma_load_2d(sB + p * r * 128, &tmB, 64 * p, bh * r,
                                     &bars.wb_full);
                     }
@@ -272,21 +295,21 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                         rows4(perm_k + (size_t)bh * N,
                               key_pos(bh, p0, ps) + 4 * lt, bh * N);
                     __syncwarp();
-                    // buffer i & 1 serves the passes of tiles i, i + 2, ...
+                    // buffer i mod VS serves the passes of tiles i, i + VS ..
                     // in turn; a pass's V goes in once the previous user is
                     // done (its P V product, or the epilogue of the last
                     // pass, which stages O there)
-                    const int ub = (i >> 1) * NPASS + ps;
+                    const int ub = i / VS * NPASS + ps;
                     if (ub >= 1 &&
-                        !lwait(&bars.v_empty[i & 1], (ub - 1) & 1, 33)) {
+                        !lwait(&bars.v_empty[i % VS], (ub - 1) & 1, 33)) {
                         go = false;
                         break;
                     }
-                    const uint32_t sV = sV0 + (i & 1) * tileB;
+                    const uint32_t sV = sV0 + (i % VS) * tileB;
                     for (int row = lrow; row < nk; row += rpi)
                         cp_async16(sV + panel_offset(row, lc, nk),
                                    vx + (size_t)vrow[row] * d + lc * 8);
-                    cp_async_mbar_arrive(&bars.v_full[i & 1]);
+                    cp_async_mbar_arrive(&bars.v_full[i % VS]);
                 }
             }
             cp_async_wait<0>();
@@ -343,11 +366,13 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                     const int s = t & 1;
                     const int su = (t >> 1) * NPASS + pass;  // unit in slot
                     const uint32_t so = tm + 256u * s;
+                    const int vb = t % VS;
                     if (mbar_test(&bars.p_full[s], su & 1) &&
-                        mbar_test(&bars.v_full[s], su & 1)) {
+                        mbar_test(&bars.v_full[vb],
+                                  (t / VS * NPASS + pass) & 1)) {
                         fence_proxy_async_smem();  // cp.async data -> MMA
                         tc_fence_after();
-                        const uint32_t sV = sV0 + s * tileB;
+                        const uint32_t sV = sV0 + vb * tileB;
                         for (int kk = 0; kk < nk / 16; ++kk)  // O (+)= P V
                             mma_ts(so + nk, so + quarter_col(kk, 0),
                                    smem_desc(sV + kk * 2048, (uint32_t)nk * 128,
@@ -355,13 +380,15 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                                    id_o, pass > 0 || kk > 0);
                         if (pass < NPASS - 1) {
                             mma_commit(&bars.pv0_done[s]);
-                            mma_commit(&bars.v_empty[s]);
+                            mma_commit(&bars.v_empty[vb]);
                         } else {
                             for (int kk = 0; kk < r0 / 16; ++kk)  // + Phi' B
                                 mma_ts(so + nk, so + quarter_col(kk, 32),
                                        smem_desc(sB + kk * 2048,
                                                  (uint32_t)r * 128, 1024),
                                        id_o, 1);
+                            if constexpr (DIRECT)
+                                mma_commit(&bars.v_empty[vb]);
                             if (two_parts) {
                                 mma_commit(&bars.pv_done[s]);
                             } else {
@@ -385,7 +412,8 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                     !(nh && ts > 0 && (two_parts ? i2 : tiles_pv) < ts)) {
                     const int s = ts & 1;
                     const uint32_t so = tm + 256u * s;
-                    bool ready = mbar_test(&bars.qk_full, us & 1);
+                    const int qb = us % QS;
+                    bool ready = mbar_test(&bars.qk_full[qb], us / QS & 1);
                     if (ready && spass == 0)
                         ready = (ts < 2 || mbar_test(&bars.tmem_empty[s],
                                                      ((ts >> 1) - 1) & 1)) &&
@@ -403,8 +431,10 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                             uint32_t okw = (kk >> 2) * NR * 128 + (kk & 3) * 32;
                             // pass 0: scores and projections (N = NR);
                             // later passes: scores only
-                            mma_ss(so, smem_desc(sQ + oq, 16, 1024),
-                                   smem_desc(sKW + okw, 16, 1024),
+                            mma_ss(so,
+                                   smem_desc(sQ + qb * tileB + oq, 16, 1024),
+                                   smem_desc(sKW + qb * tileKW + okw, 16,
+                                             1024),
                                    spass == 0 ? id_sp : id_s, kk > 0);
                         }
                         mma_commit(&bars.s_full[s]);
@@ -451,9 +481,8 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             const bool ok = mbar_wait_or_abort(bar, par, abort, status, site);
             return named_sync_and(1 + g, 256, ok);
         };
-        // The Q, K copies of tile t are issued by the other slot (the one
-        // of tile t - 1) as soon as the scores of tile t - 1 free the Q, K
-        // buffer: 256 threads, whole rows per warp instruction; completion
+        // The Q, K copies of tile t are issued by the slot of tile t - QS as
+        // soon as the scores of that tile free the Q, K buffer: 256 threads, whole rows per warp instruction; completion
         // reaches qk_full through cp.async's own mbarrier arrivals.
         const int ct = (cw & 7) * 32 + lane_id;  // 0..255 within the slot
         auto issue_qk = [&](int t) -> bool {
@@ -461,13 +490,15 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             const int cpr = d >> 3, rpp = 256 / cpr;
             const int crow = ct / cpr, cc = ct - crow * cpr;
             const int *qr = qkrow[t & 1][0], *kr = qkrow[t & 1][1];
+            const uint32_t dQ = sQ + (t % QS) * tileB;
+            const uint32_t dK = sKW + (t % QS) * tileKW;
             for (int rr = crow; rr < nk; rr += rpp) {
-                cp_async16(sQ + panel_offset(rr, cc, nk),
+                cp_async16(dQ + panel_offset(rr, cc, nk),
                            qx + (size_t)qr[rr] * d + cc * 8);
-                cp_async16(sKW + panel_offset(rr, cc, NR),
+                cp_async16(dK + panel_offset(rr, cc, NR),
                            kx + (size_t)kr[rr] * d + cc * 8);
             }
-            cp_async_mbar_arrive(&bars.qk_full);
+            cp_async_mbar_arrive(&bars.qk_full[t % QS]);
             mbar_arrive(&bars.idx_empty[t & 1]);
             return true;
         };
@@ -481,12 +512,14 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             for (int rr = crow; rr < nk; rr += rpp)
                 cp_async16(sKW + panel_offset(rr, cc, NR),
                            kx + (size_t)kr[rr] * d + cc * 8);
-            cp_async_mbar_arrive(&bars.qk_full);
+            cp_async_mbar_arrive(&bars.qk_full[0]);
             mbar_arrive(&bars.idx_empty[t & 1]);
             return true;
         };
         bool started = true;
-        if (g == 1 && ntiles > 0) started = issue_qk(0);
+        if (g == 1)
+            for (int t = 0; t < QS && t < ntiles && started; ++t)
+                started = issue_qk(t);
         for (int j = g; started && j < ntiles; j += 2) {
             const int k = j >> 1;
             const uint32_t so = tm + 256u * g + lane;
@@ -504,7 +537,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             if constexpr (NPASS > 1) {
                 if (!issue_k(j, 1)) break;
             } else {
-                if (j + 1 < ntiles && !issue_qk(j + 1)) break;
+                if (j + QS < ntiles && !issue_qk(j + QS)) break;
             }
             // per-bit factors of this half's tables (sp[0, 16): chunk half,
             // up to 32 when the chunk has more projection columns and no
@@ -551,8 +584,20 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                        ((unsigned long long)w[1] << 32);
             };
             const unsigned long long sb0 = selbits(0);
+            // KB: the block of this warp's rows and this half's share of it
+            constexpr int KN = KB > 0 ? KB / 2 : 16;
+            uint32_t sv[KN];
+            const int kl = KB > 0 ? (warp & 3) * 32 / KN / 2 * KB : 0;
+            if constexpr (KB == 64) tmem_ld32(so + kl + half * KN, sv);
+            if constexpr (KB == 32) tmem_ld16(so + kl + half * KN, sv);
+            if constexpr (KB > 0) {
+                tmem_wait_ld();
 #pragma unroll
-            for (int c = 0; c < nk / 2; c += 16) {
+                for (int jj = 0; jj < KN; ++jj)
+                    mxa[jj & 3] = fmaxf(mxa[jj & 3], __uint_as_float(sv[jj]));
+            }
+#pragma unroll
+            for (int c = 0; KB == 0 && c < nk / 2; c += 16) {
                 uint32_t v[16];
                 tmem_ld16(so + kbeg + c, v);
                 tmem_wait_ld();
@@ -574,8 +619,35 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 (xden[g][0][row] + xden[g][1][row]) * (1.0f / (float)L);
             float M2 = mx * sl2e;
             float ls[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            if constexpr (KB > 0) {
+                // P of the block over the first columns of its quarter, and
+                // zeros for the tile's other keys
+                const int q = kl & 64, w = (kl & 63) / 2;
+                uint32_t pw[KN / 2], zero[16];
 #pragma unroll
-            for (int c = 0; c < nk / 2; c += 32) {
+                for (int jj = 0; jj < KN; jj += 2) {
+                    const float a0 = ex2_approx(
+                        fmaf(__uint_as_float(sv[jj]), sl2e, -M2));
+                    const float a1 = ex2_approx(
+                        fmaf(__uint_as_float(sv[jj + 1]), sl2e, -M2));
+                    ls[(jj >> 1) & 3] += a0 + a1;
+                    pw[jj >> 1] = pack_bf16x2(a0, a1);
+                }
+#pragma unroll
+                for (int jj = 0; jj < 16; ++jj) zero[jj] = 0u;
+                if constexpr (KB == 64) {
+                    tmem_st16(so + q + half * 16, pw);
+                } else {
+                    uint32_t z8[8];
+#pragma unroll
+                    for (int jj = 0; jj < 8; ++jj) z8[jj] = 0u;
+                    tmem_st8(so + q + w + half * 8, pw);
+                    tmem_st8(so + q + (w ^ 16) + half * 8, z8);
+                }
+                tmem_st16(so + (q ^ 64) + half * 16, zero);
+            }
+#pragma unroll
+            for (int c = 0; KB == 0 && c < nk / 2; c += 32) {
                 uint32_t pk16[16];
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
@@ -757,8 +829,41 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             // the swizzled panel layout, then copied out by the slot's 256
             // threads in whole rows (coalesced 16-byte stores). With an
             // fp32 output (o32) each thread stores its half row directly.
-            const uint32_t sVg = sV0 + g * tileB;
+            const uint32_t sVg = sV0 + (j % VS) * tileB;
             constexpr int kMaxHalf = 64;  // d / 2 for d = 128
+            if constexpr (DIRECT) {  // d = 64: 64 bytes per thread
+                uint32_t v[32];
+                tmem_ld32(so + nk + half * 32, v);
+                tmem_wait_ld();
+                tc_fence_before();
+                mbar_arrive(&bars.tmem_empty[g]);
+                if (qvalid) {
+                    uint16_t *dst = ox + tok * 64 + half * 32;
+                    const bool a32 = ((uintptr_t)ox & 31u) == 0;
+#pragma unroll
+                    for (int c = 0; c < 32; c += 16) {
+                        uint32_t ob[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            ob[q] = pack_bf16x2(
+                                c1e * __uint_as_float(v[c + 2 * q]),
+                                c1e * __uint_as_float(v[c + 2 * q + 1]));
+                        if (a32) {
+                            st_global_v8(dst + c, ob);
+                        } else {
+                            uint4 *p = reinterpret_cast<uint4 *>(dst + c);
+                            p[0] = make_uint4(ob[0], ob[1], ob[2], ob[3]);
+                            p[1] = make_uint4(ob[4], ob[5], ob[6], ob[7]);
+                        }
+                    }
+                    if (half == 0) {
+                        if (log_ds_out) log_ds_out[tok] = log_ds;
+                        if (dlr_out) dlr_out[tok] = denf;
+                        if (m_out) m_out[tok] = msp;
+                    }
+                }
+                continue;
+            }
 #pragma unroll
             for (int c = 0; c < kMaxHalf; c += 16) {
                 if (c < (d >> 1)) {
@@ -816,7 +921,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 }
             }
             named_sync(1 + g, 256);  // the staging buffer is read
-            if (cw == 8 * g && lane_id == 0) mbar_arrive(&bars.v_empty[g]);
+            if (cw == 8 * g && lane_id == 0) mbar_arrive(&bars.v_empty[j % VS]);
         }
         cp_async_wait<0>();
     }
@@ -863,10 +968,13 @@ cudaError_t launch_block_attn_ws(
     const int32_t *cand, const uint32_t *selmask) {
     const int lg_pad = (P.L * P.gamma + 15) / 16 * 16;
     const size_t tileB = (size_t)kWsNK * P.d * 2;
-    const size_t smem = 1024 + 4 * tileB + ((size_t)lg_pad * P.d * 2 + 1023) /
-                                               1024 * 1024 +
-                        ((size_t)P.r * P.d * 2 + 1023) / 1024 * 1024 +
-                        (size_t)P.r * 4;
+    auto smem_for = [&](int qs) {
+        const int vs = qs > 2 ? qs : 2;
+        return 1024 + (2 * qs + vs) * tileB +
+               qs * (((size_t)lg_pad * P.d * 2 + 1023) / 1024 * 1024) +
+               ((size_t)P.r * P.d * 2 + 1023) / 1024 * 1024 +
+               (size_t)P.r * 4;
+    };
     const int tiles_per_head = (P.N + 127) / 128;
     const long total = (long)tiles_per_head * P.BH;
     int dev = 0, sms = 148;
@@ -881,7 +989,8 @@ cudaError_t launch_block_attn_ws(
         e = make_tma_map_bf16(&tmB, Bh, (uint64_t)P.BH * P.r, P.d,
                               (uint32_t)P.r);
     if (e != cudaSuccess) return e;
-    auto launch = [&](auto kern) {
+    auto launch = [&](auto kern, int qs = 1) {
+        const size_t smem = smem_for(qs);
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
         kern<<<grid, kWsThreads, smem, st>>>(
@@ -894,6 +1003,27 @@ cudaError_t launch_block_attn_ws(
         return cudaGetLastError();
     };
     const int passes = ws_passes(P);
+    // d = 64 leaves shared memory for three Q/K and value buffers (172 KB at
+    // r = 128); at d = 128 one fits. Key blocks of 32 and 64 take half and a
+    // quarter of the softmax work of the masked path. Both together, B4 H12
+    // N4096 d64 b64 r128: 63 -> 45 us; B8 H12 N8192: 215 -> 138 us; B3 H5
+    // N4800 d128 b64 (KB alone): 35 -> 27 us.
+    if (P.gamma == 4 && P.sel == 0 && passes == 1) {
+        auto pick = [&](auto o32) {
+            constexpr bool F = decltype(o32)::value;
+            if (P.d == 64 && smem_for(3) <= 216 * 1024) {
+                if (P.b == 32)
+                    return launch(k_block_attn_ws<4, 1, 0, F, 3, 32>, 3);
+                if (P.b == 64)
+                    return launch(k_block_attn_ws<4, 1, 0, F, 3, 64>, 3);
+                return launch(k_block_attn_ws<4, 1, 0, F, 3>, 3);
+            }
+            if (P.b == 32) return launch(k_block_attn_ws<4, 1, 0, F, 1, 32>);
+            if (P.b == 64) return launch(k_block_attn_ws<4, 1, 0, F, 1, 64>);
+            return launch(k_block_attn_ws<4, 1, 0, F>);
+        };
+        return P.o32 ? pick(std::true_type{}) : pick(std::false_type{});
+    }
     if (P.o32) {  // fp32 output: gamma = 4 (ws_supported)
         if (P.sel) {
             switch (passes) {
@@ -907,8 +1037,7 @@ cudaError_t launch_block_attn_ws(
         if (passes == 3) return launch(k_block_attn_ws<4, 3, 1, true>);
         if (passes == 6) return launch(k_block_attn_ws<4, 6, 1, true>);
         if (P.gamma != 4) return cudaErrorInvalidValue;
-        return P.b > 128 ? launch(k_block_attn_ws<4, 2, 0, true>)
-                         : launch(k_block_attn_ws<4, 1, 0, true>);
+        return launch(k_block_attn_ws<4, 2, 0, true>);
     }
     if (P.sel) {
         switch (passes) {
@@ -925,7 +1054,7 @@ cudaError_t launch_block_attn_ws(
         case 1: return P.b > 128 ? launch(k_block_attn_ws<1, 2, 0>) : launch(k_block_attn_ws<1, 1, 0>);
         case 2: return P.b > 128 ? launch(k_block_attn_ws<2, 2, 0>) : launch(k_block_attn_ws<2, 1, 0>);
         case 3: return P.b > 128 ? launch(k_block_attn_ws<3, 2, 0>) : launch(k_block_attn_ws<3, 1, 0>);
-        case 4: return P.b > 128 ? launch(k_block_attn_ws<4, 2, 0>) : launch(k_block_attn_ws<4, 1, 0>);
+        case 4: return launch(k_block_attn_ws<4, 2, 0>);
         case 5: return P.b > 128 ? launch(k_block_attn_ws<5, 2, 0>) : launch(k_block_attn_ws<5, 1, 0>);
         case 6: return P.b > 128 ? launch(k_block_attn_ws<6, 2, 0>) : launch(k_block_attn_ws<6, 1, 0>);
         default: return cudaErrorInvalidValue;
