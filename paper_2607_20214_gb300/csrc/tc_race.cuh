@@ -83,6 +83,22 @@ __device__ __forceinline__ void race_factors16(const uint32_t *pr, int ncols,
     }
 }
 
+// The per-bit factors of n projections already loaded from TMEM (fp32 bits
+// in pr), entries past `ncols` set to 1/2.
+template <int n>
+__device__ __forceinline__ void race_factors(const uint32_t *pr, int ncols,
+                                             float beta, float *sp) {
+#pragma unroll
+    for (int j = 0; j < n; ++j) {
+        sp[j] = 0.5f;
+        if (j < ncols)
+            sp[j] = fmaf(0.5f,
+                         tanh_approx(beta *
+                                     tanh_approx(__uint_as_float(pr[j]))),
+                         0.5f);
+    }
+}
+
 // race_bits32 over 16 projection columns: sp[j] for j < 16, entries past
 // `ncols` set to 1/2. The TMEM load is waited for inside.
 __device__ __forceinline__ void race_bits16(uint32_t taddr, int ncols,
@@ -130,18 +146,29 @@ __device__ __forceinline__ void table_uw4(const float *sp, float scale,
     w[3] = p2 * p3;
 }
 
-// sum_r phi_r A_r of one gamma = 4 table = sum_j w_j (u . A[4 j .. 4 j + 3]);
-// A: 16 floats in shared memory, 16-byte aligned.
+// sum_r phi_r A_r of one gamma = 4 table = sum_j w_j (u . A[4 j .. 4 j + 3]).
+__device__ __forceinline__ float table_dot4(const float (&u)[4],
+                                            const float (&w)[4],
+                                            const float4 (&A)[4]) {
+    const float2 u01 = make_float2(u[0], u[1]), u23 = make_float2(u[2], u[3]);
+    float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 t = fma2(u23, make_float2(A[j].z, A[j].w),
+                              mul2(u01, make_float2(A[j].x, A[j].y)));
+        s = fma2(make_float2(w[j], w[j]), t, s);
+    }
+    return s.x + s.y;
+}
+// The same with A (16 floats, 16-byte aligned) in shared memory.
 __device__ __forceinline__ float table_dot4(const float (&u)[4],
                                             const float (&w)[4],
                                             const float *A) {
-    float acc[4];
+    float4 a[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const float4 a = *reinterpret_cast<const float4 *>(A + 4 * j);
-        acc[j] = fmaf(u[3], a.w, fmaf(u[2], a.z, fmaf(u[1], a.y, u[0] * a.x)));
-    }
-    return fmaf(w[3], acc[3], fmaf(w[2], acc[2], fmaf(w[1], acc[1], w[0] * acc[0])));
+    for (int j = 0; j < 4; ++j)
+        a[j] = *reinterpret_cast<const float4 *>(A + 4 * j);
+    return table_dot4(u, w, a);
 }
 
 // Packed bf16 features of one gamma = 4 table: out[k] holds buckets
@@ -151,8 +178,11 @@ __device__ __forceinline__ void table_pack4(const float (&u)[4],
                                             uint32_t *out) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        out[2 * j] = pack_bf16x2(u[0] * w[j], u[1] * w[j]);
-        out[2 * j + 1] = pack_bf16x2(u[2] * w[j], u[3] * w[j]);
+        const float2 wj = make_float2(w[j], w[j]);
+        const float2 a = mul2(make_float2(u[0], u[1]), wj);
+        const float2 b = mul2(make_float2(u[2], u[3]), wj);
+        out[2 * j] = pack_bf16x2(a.x, a.y);
+        out[2 * j + 1] = pack_bf16x2(b.x, b.y);
     }
 }
 

@@ -1,7 +1,8 @@
 // Persistent, warp-specialised sortLSH block attention + RACE readout +
 // fusion (Algorithm "sortLSH Sparse Exact Attention Branch" block step,
 // Algorithm "RACE Low-Rank Attention Branch" steps 9-10, Eq. (5)-(6)) for
-// bf16 inputs whose key blocks fit one 128-key tile (b <= 128).
+// bf16 inputs: key blocks of up to 256, neighbour windows and the top-k
+// selector's candidate blocks, 128 keys per pass.
 //
 // One CTA per SM walks a contiguous range of 128-query tiles (ordered by
 // head, then sorted position, so the per-head B summary, A summary and RACE
@@ -13,19 +14,29 @@
 //               Within a slot, warps w and w + 4 share TMEM lanes (lane
 //               group w mod 4) and split each row's key columns and output
 //               columns in halves; half h owns the RACE buckets of the
-//               64-bucket chunks h and h + 2, so both halves write features
-//               before and after the P V product.
+//               64-bucket chunks h and h + 2. The two warps exchange row
+//               maxima and sums over a barrier of their 64 threads; nothing
+//               else synchronises the slot.
 //   warp 16     allocates tensor memory and issues every MMA (lane 0).
-//   warps 17-19 loaders: cp.async gathers of the tile's Q rows (warp 17), K
-//               rows (warp 18, which also stages per head the RACE planes as
-//               bf16, the bf16 B summary and the fp32 A summary) and V rows
-//               (warp 19, two buffers). A gather's rate grows with the
-//               number of warps issuing it, hence one warp per operand.
-
-// Per tile: proj + S MMAs -> (group) features, Den, softmax, P and the
-// pre-scaled features into TMEM -> PV and Phi'B MMAs into one accumulator
-// -> (group) epilogue O = c1 * acc. Every hand-off is an mbarrier; every wait
-// is bounded and a stalled pipeline drains through a shared abort flag.
+//   warp 17     per head, TMA loads of the bf16 RACE planes (under the key
+//               rows), the bf16 B summary and the fp32 A summary.
+//   warps 18-19 V rows; warps 20-23 Q and K rows: cp.async gathers, whole
+//               rows per instruction, row numbers read a unit ahead.
+//
+// Per tile: S and projections MMA -> (slot) softmax, P into TMEM -> P V MMA,
+// meanwhile (slot) features, Den, fusion scalars -> pre-scaled features into
+// TMEM -> Phi'B MMA into the same accumulator -> (slot) epilogue
+// O = c1 * acc, stored from registers. Every hand-off is an mbarrier; every
+// wait is bounded and a stalled pipeline drains through a shared abort flag.
+//
+// What bounds it: a slot's own chain of these steps, about 17 K clocks per
+// tile at d = 128 (clock traces: the next tile's scores are there when the
+// slot asks for them; two slots give a tile per 8.5 K clocks, where the
+// copies need 6 K). Every step taken off the chain shows in the time: copies
+// by warps of their own, features under the P V product, barriers of 64
+// threads only. c3: 163 -> 143 us; c2: 45 -> 42; c5: 138 -> 129; c3 top-k (two
+// passes): 313 -> 263. Left on it at c3 (time without the step): Den 22 us,
+// features 15, stores 7, bit factors 5.
 #include "device_common.cuh"
 #include "tc_common.cuh"
 #include "tc_race.cuh"
@@ -38,23 +49,28 @@ namespace {
 
 using namespace tc;
 
-constexpr int kWsThreads = 640;   // 16 compute, MMA and 3 loader warps
+constexpr int kWsThreads = 768;   // 16 compute warps and 8 others
 constexpr int kWsMmaWarp = 16;
-constexpr int kWsLoaders = 32;    // threads of one loader warp
+constexpr int kWsVWarp = 18, kWsVWarps = 2;
+constexpr int kWsQkWarp = 20, kWsQkWarps = 4;
 constexpr int kWsNK = 128;        // keys per query tile
+// Registers: 768 x 80 at launch = 512 x 96 (compute) + 256 x 48 (others).
+constexpr int kWsRegsCompute = 96, kWsRegsOther = 48;
+static_assert(512 * kWsRegsCompute + 256 * kWsRegsOther <= kWsThreads * 80,
+              "register shares within the launch's total");
 // TMEM slot layout (256 columns): S/P/features region [0, 128) in four
 // 32-column quarters, output accumulator [128, 128 + d). P of keys
 // [64h, 64h + 64) (row half h) lives in quarter 2h, packed in place over
 // the scores already read; the pre-scaled RACE features of buckets
 // [0, 128) go to quarters 1 and 3, buckets [128, 256) to quarters 0 and 2
-// once the P V product is done.
+// once the P V product is done. The projections come out in columns
+// [128, 128 + Lg_pad), read before the first P V product overwrites them.
 
 template <int QS, int VS>
 struct WsBars {
-    uint64_t qk_full[QS], wb_full, head_done;
-    uint64_t idx_full[2], idx_empty[2];
-    uint64_t v_full[VS], v_empty[VS], pv0_done[2];
-    uint64_t s_full[2], p_full[2], pv_done[2], p2_full[2], o_full[2];
+    uint64_t qk_full[QS], qk_empty[QS], v_full[VS], v_empty[VS];
+    uint64_t wb_full, head_done;
+    uint64_t s_full[2], p_full[2], pv_done[2], phi_full[2], o_full[2];
     uint64_t tmem_empty[2];
 };
 
@@ -66,15 +82,13 @@ struct WsBars {
 // the sequence are masked. 2 (SEL): the top-k selector's candidate blocks
 // (cand, tk_c per query block), each key masked unless the row's bit in
 // selmask is set. The checks of the other modes are compiled out. O32: O
-// is written as fp32 (out_fp32), each thread storing its half row directly.
+// is written as fp32 (out_fp32).
 // QS: buffers of the Q and key tiles (one pass per tile when > 1), so that
 // the rows of tile t + QS are copied while tiles t + 1 .. t + QS - 1 wait
-// for their scores, with as many value buffers (d = 64; O then leaves from
-// registers, and a value buffer is free as soon as its product is done).
+// for their scores, with as many value buffers.
 // KB: b when it is 32 or 64 (0: any b). The 32 rows of a warp then share one
-// key block of KB scores, half for each of the row's two threads, kept in
-// registers between the maximum and the exponentials; the general path
-// takes all 128 columns with a mask.
+// key block of KB scores, half for each of the row's two threads; the
+// general path takes all 128 columns with a mask.
 template <int G, int NPASS, int KM, bool O32 = false, int QS = 1, int KB = 0>
 __global__ void __launch_bounds__(kWsThreads, 1)
     k_block_attn_ws(const uint16_t *__restrict__ qx,
@@ -100,25 +114,21 @@ __global__ void __launch_bounds__(kWsThreads, 1)
     constexpr int VS = QS > 2 ? QS : 2;  // value buffers
     static_assert((QS == 1 && KB == 0) || (NPASS == 1 && KM == 0),
                   "one pass per tile");
-    constexpr bool DIRECT = QS > 1 && !O32;  // O stored from registers
     constexpr int R = 1 << G;
     constexpr int nk = kWsNK;
     extern __shared__ unsigned char smem_raw[];
     __shared__ WsBars<QS, VS> bars;
     __shared__ uint32_t tbase;
     __shared__ int abort_flag;
-    __shared__ float xmax[2][2][128], xsum[2][2][128], xden[2][2][128];
-    // global rows of a tile's queries / keys, per tile parity (written by
-    // the index warp, read by the slot that issues the tile's Q, K copies)
-    __shared__ __align__(16) int qkrow[2][1 + NPASS][128];
-    __shared__ __align__(16) int vrow[128];  // V loader: rows of its tile
-    __shared__ int orow[2][128];          // per slot: output row or -1
+    __shared__ float xmax[2][2][128];
+    __shared__ float2 xsum[2][2][128];  // row sum, Den
     volatile int *abort = &abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane_id = tid & 31;
-    const int Lg = L * G, r = L * R;
+    const int r = L * R;
     const long t_begin = total_tiles * blockIdx.x / gridDim.x;
     const long t_end = total_tiles * (blockIdx.x + 1) / gridDim.x;
     const int ntiles = (int)(t_end - t_begin);
+    const int nunits = ntiles * NPASS;
 
     const uint32_t tileB = (uint32_t)nk * d * 2u;  // one [128 x d] tile
     const uint32_t base = align1k(smem_u32(smem_raw));
@@ -136,22 +146,24 @@ __global__ void __launch_bounds__(kWsThreads, 1)
 
     if (warp == kWsMmaWarp) tmem_alloc(&tbase, 512);
     if (tid == 0) {
-        // the issuing slot's threads
-        for (int s = 0; s < QS; ++s) mbar_init(&bars.qk_full[s], 256);
+        for (int s = 0; s < QS; ++s) {
+            mbar_init(&bars.qk_full[s], 32 * kWsQkWarps);
+            mbar_init(&bars.qk_empty[s], 1);
+        }
         for (int s = 0; s < VS; ++s) {
-            mbar_init(&bars.v_full[s], kWsLoaders);
-            mbar_init(&bars.v_empty[s], 1);
+            mbar_init(&bars.v_full[s], 32 * kWsVWarps);
+            // one pass: the slot's warps, after their stores (freeing the
+            // buffer earlier brings its copies into busier phases: 42 -> 43
+            // us at c2); several: the P V product's commit
+            mbar_init(&bars.v_empty[s], NPASS == 1 ? 8 : 1);
         }
         mbar_init(&bars.wb_full, 1);
         mbar_init(&bars.head_done, 1);
         for (int s = 0; s < 2; ++s) {
-            mbar_init(&bars.idx_full[s], kWsLoaders);
-            mbar_init(&bars.idx_empty[s], 256 * NPASS);
-            mbar_init(&bars.pv0_done[s], 1);
             mbar_init(&bars.s_full[s], 1);
             mbar_init(&bars.p_full[s], 256);
             mbar_init(&bars.pv_done[s], 1);
-            mbar_init(&bars.p2_full[s], 256);
+            mbar_init(&bars.phi_full[s], 256);
             mbar_init(&bars.o_full[s], 1);
             mbar_init(&bars.tmem_empty[s], 256);
         }
@@ -196,74 +208,98 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         if (NPASS == 1) return k0;  // the tile's own keys (ragged end kept)
         return k0 < 0 ? 0 : (k0 > N - 128 ? N - 128 : k0);
     };
-    // global row numbers of the 4 sorted positions pos.. pos + 3 (the
-    // ragged end repeats the last row; those rows are never stored)
-    auto rows4 = [=](const int32_t *pm, int pos, int rowbase) {
-        int4 r;
-        if (pos + 3 < N && ((uintptr_t)(pm + pos) & 15u) == 0) {
-            r = *reinterpret_cast<const int4 *>(pm + pos);
-        } else {
-            r.x = pm[min(pos, N - 1)];
-            r.y = pm[min(pos + 1, N - 1)];
-            r.z = pm[min(pos + 2, N - 1)];
-            r.w = pm[min(pos + 3, N - 1)];
-        }
-        // an entry outside [0, N) is read as row 0 (the orders come from
-        // the sort, in range by construction); the checked build
-        // (ELSAA_CHECKED) also records it: 4 % of this kernel's time when
-        // always on
-        auto fix = [=](int v) {
-            if (v < 0 || v >= N) {
+    // global row number of sorted position pos (the ragged end repeats the
+    // last row; those rows are never stored). An entry outside [0, N) is
+    // read as row 0 (the orders come from the sort, in range by
+    // construction); the checked build (ELSAA_CHECKED) also records it.
+    auto global_row = [=](const int32_t *pm, int bh, int pos) {
+        int v = pm[(size_t)bh * N + min(pos, N - 1)];
+        if (v < 0 || v >= N) {
 #ifdef ELSAA_CHECKED
-                report(status, kDevPermRange, 4, rowbase / N, v);
+            report(status, kDevPermRange, 4, bh, v);
 #endif
-                v = 0;
-            }
-            return rowbase + v;
-        };
-        return make_int4(fix(r.x), fix(r.y), fix(r.z), fix(r.w));
+            v = 0;
+        }
+        return bh * N + v;
     };
 
-    if (warp > kWsMmaWarp) {
-        // ------------------------------------------------------------ loaders
-        // warp 17: global row numbers of each tile's queries and keys into
-        //          qkrow[tile & 1] (the copies themselves are issued by the
-        //          compute slot whose scores just freed the Q, K buffer);
-        // warp 18: per head, TMA loads of the bf16 RACE planes (under the
-        //          key rows), the bf16 B summary and the fp32 A summary;
-        // warp 19: V rows with cp.async (whole rows per instruction, into
-        //          the swizzled operand layout); completion reaches v_full
-        //          through cp.async's own mbarrier arrivals.
-        const int role = warp - kWsMmaWarp - 1;
-        const int lt = lane_id;
+    if (warp >= kWsMmaWarp) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(
+            kWsRegsOther));
         auto lwait = [=](uint64_t *bar, uint32_t par, int site) {
             return __all_sync(0xffffffffu,
                               mbar_wait_or_abort(bar, par, abort, status,
                                                  site));
         };
-        if (role == 0) {
-            for (int i = 0; i < ntiles; ++i) {
-                const int bh = tile_head(i), p0 = tile_p0(i), t = i & 1;
-                if (i >= 2 &&
-                    !lwait(&bars.idx_empty[t], ((i >> 1) - 1) & 1, 30))
-                    break;
-                *reinterpret_cast<int4 *>(&qkrow[t][0][4 * lt]) =
-                    rows4(perm_q + (size_t)bh * N, p0 + 4 * lt, bh * N);
-#pragma unroll
-                for (int ps = 0; ps < NPASS; ++ps)
-                    *reinterpret_cast<int4 *>(&qkrow[t][1 + ps][4 * lt]) =
-                        rows4(perm_k + (size_t)bh * N,
-                              key_pos(bh, p0, ps) + 4 * lt, bh * N);
-                __syncwarp();
-                mbar_arrive(&bars.idx_full[t]);
+        const int cpr = d >> 3;    // 16-byte chunks per row
+        const int rpi = 32 / cpr;  // rows per instruction
+        const int sub = lane_id / cpr, ch = lane_id - sub * cpr;
+        // copies rows [r0, r0 + 32) of a tile of `rows` rows; lane l holds
+        // the global number of row r0 + l
+        auto copy32 = [=](uint32_t dst, int rows, int r0,
+                          const uint16_t *src, int rowno) {
+#pragma unroll 4
+            for (int i = sub; i < 32; i += rpi) {
+                const int row = __shfl_sync(0xffffffffu, rowno, i);
+                cp_async16(dst + panel_offset(r0 + i, ch, rows),
+                           src + (size_t)row * d + ch * 8);
             }
-        } else if (role == 1) {
+        };
+        if (warp >= kWsQkWarp) {
+            // ------------------------------------------------ Q and K rows
+            const int r0 = (warp - kWsQkWarp) * 32;
+            int qn = 0, kn = 0;  // of the next unit
+            auto ahead = [&](int u) {
+                const int t = u / NPASS, ps = u - t * NPASS;
+                const int bh = tile_head(t), p0 = tile_p0(t);
+                if (ps == 0) qn = global_row(perm_q, bh, p0 + r0 + lane_id);
+                kn = global_row(perm_k, bh,
+                                key_pos(bh, p0, ps) + r0 + lane_id);
+            };
+            if (nunits > 0) ahead(0);
+            for (int u = 0; u < nunits; ++u) {
+                const int qr = qn, kr = kn, st = u % QS;
+                if (u + 1 < nunits) ahead(u + 1);
+                if (u >= QS &&
+                    !lwait(&bars.qk_empty[st], (u / QS - 1) & 1, 30))
+                    break;
+                if (NPASS == 1 || u % NPASS == 0)
+                    copy32(sQ + st * tileB, nk, r0, qx, qr);
+                copy32(sKW + st * tileKW, NR, r0, kx, kr);
+                cp_async_mbar_arrive(&bars.qk_full[st]);
+            }
+            cp_async_wait<0>();
+        } else if (warp >= kWsVWarp) {
+            // ------------------------------------------------------ V rows
+            const int r0 = (warp - kWsVWarp) * 64;
+            int n0 = 0, n1 = 0;  // of the next unit
+            auto ahead = [&](int u) {
+                const int t = u / NPASS, ps = u - t * NPASS;
+                const int bh = tile_head(t);
+                const int p = key_pos(bh, tile_p0(t), ps) + r0 + lane_id;
+                n0 = global_row(perm_k, bh, p);
+                n1 = global_row(perm_k, bh, p + 32);
+            };
+            if (nunits > 0) ahead(0);
+            for (int u = 0; u < nunits; ++u) {
+                const int a0 = n0, a1 = n1, st = u % VS;
+                if (u + 1 < nunits) ahead(u + 1);
+                if (u >= VS &&
+                    !lwait(&bars.v_empty[st], (u / VS - 1) & 1, 33))
+                    break;
+                copy32(sV0 + st * tileB, nk, r0, vx, a0);
+                copy32(sV0 + st * tileB, nk, r0 + 32, vx, a1);
+                cp_async_mbar_arrive(&bars.v_full[st]);
+            }
+            cp_async_wait<0>();
+        } else if (warp == kWsMmaWarp + 1) {
+            // -------------------------------------- planes, B and A summary
             int hc = 0;
             for (int i = 0; i < ntiles; ++i) {
                 if (!new_head(i)) continue;
                 const int bh = tile_head(i);
                 if (i > 0 && !lwait(&bars.head_done, (hc - 1) & 1, 31)) break;
-                if (lt == 0) {  // TMA: planes under the key rows, B, A
+                if (lane_id == 0) {
                     mbar_expect_tx(&bars.wb_full,
                                    (uint32_t)(QS * Lg_pad + r) * d * 2u +
                                        r * 4u);
@@ -282,75 +318,40 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 __syncwarp();
                 ++hc;
             }
-        } else {
-            const int cpr = d >> 3;    // 16-byte chunks per row
-            const int rpi = 32 / cpr;  // rows per instruction
-            const int lrow = lt / cpr, lc = lt - lrow * cpr;
-            bool go = true;
-            for (int i = 0; i < ntiles && go; ++i) {
-                const int bh = tile_head(i), p0 = tile_p0(i);
-                for (int ps = 0; ps < NPASS; ++ps) {
-                    __syncwarp();  // the previous rows are all read
-                    *reinterpret_cast<int4 *>(&vrow[4 * lt]) =
-                        rows4(perm_k + (size_t)bh * N,
-                              key_pos(bh, p0, ps) + 4 * lt, bh * N);
-                    __syncwarp();
-                    // buffer i mod VS serves the passes of tiles i, i + VS ..
-                    // in turn; a pass's V goes in once the previous user is
-                    // done (its P V product, or the epilogue of the last
-                    // pass, which stages O there)
-                    const int ub = i / VS * NPASS + ps;
-                    if (ub >= 1 &&
-                        !lwait(&bars.v_empty[i % VS], (ub - 1) & 1, 33)) {
-                        go = false;
-                        break;
-                    }
-                    const uint32_t sV = sV0 + (i % VS) * tileB;
-                    for (int row = lrow; row < nk; row += rpi)
-                        cp_async16(sV + panel_offset(row, lc, nk),
-                                   vx + (size_t)vrow[row] * d + lc * 8);
-                    cp_async_mbar_arrive(&bars.v_full[i % VS]);
-                }
-            }
-            cp_async_wait<0>();
-        }
-    } else if (warp == kWsMmaWarp) {
-        // ----------------------------------------------------------- MMA issue
-        // Event driven: each pass issues whichever MMA group is ready, the
-        // oldest tile's first (second feature part, then P V with the first
-        // part, then the next tile's projections and scores), so one slot's
-        // epilogue never holds back the other slot's products.
-        // Units: (tile, pass); with NPASS = 2 the second score product of
-        // a tile waits until its first P V product is complete (it reuses
-        // the S columns), and the first P V product releases the V buffer
-        // for the second key half.
-        if (lane_id == 0 && ntiles > 0) {
+        } else if (lane_id == 0 && ntiles > 0) {
+            // ------------------------------------------------------ MMA issue
+            // Event driven: each round issues whichever MMA group is ready,
+            // the oldest tile's first (Phi'B, then P V, then the next
+            // scores), so one slot's epilogue never holds back the other
+            // slot's products. Units: (tile, pass); a tile's later score
+            // products wait until its previous P V product is complete (it
+            // reads P from the S columns).
             const uint32_t id_sp = idesc_bf16(128, NR, false, false);
             const uint32_t id_s = idesc_bf16(128, nk, false, false);
             const uint32_t id_o = idesc_bf16(128, d, false, true);
-            const int r0 = min(r, nk);
-            const bool two_parts = r > nk;
-            const int nunits = ntiles * NPASS;
             int us = 0, up = 0, i2 = 0;  // next unit for S, unit for P V, tile
-                                         // for part 2
+                                         // for Phi'B
             int tiles_pv = 0;            // tiles whose last P V is issued
-            // position of each cursor's tile within its head (advanced
-            // incrementally: no divisions in the issue loop)
+            // position of the S and Phi'B cursors' tiles within their heads
+            // (advanced incrementally: no divisions in the issue loop)
             const int tph = tiles_per_head;
-            int ps = (int)(t_begin % tph), pp = ps, p2 = ps;
+            int ps = (int)(t_begin % tph), p2 = ps;
             auto adv = [tph](int q) { return q + 1 == tph ? 0 : q + 1; };
             int hc = 0;                  // heads whose planes were consumed
             unsigned long long t_last = global_ns();
-            while ((two_parts ? i2 : tiles_pv) < ntiles) {
+            uint32_t idle = 0;  // the clock is read every 256 idle rounds
+            while (i2 < ntiles) {
                 bool did = false;
-                if (two_parts && i2 < tiles_pv) {
+                if (i2 < tiles_pv) {
                     const int s = i2 & 1;
                     const uint32_t so = tm + 256u * s;
-                    if (mbar_test(&bars.p2_full[s], (i2 >> 1) & 1)) {
+                    if (mbar_test(&bars.phi_full[s], (i2 >> 1) & 1)) {
                         tc_fence_after();
-                        for (int kk = 0; kk < (r - nk) / 16; ++kk)
-                            mma_ts(so + nk, so + quarter_col(kk, 0),
-                                   smem_desc(sB + (uint32_t)nk * 128 + kk * 2048,
+                        for (int kk = 0; kk < r / 16; ++kk)  // O += Phi' B
+                            mma_ts(so + nk,
+                                   so + (kk < 8 ? quarter_col(kk, 32)
+                                                : quarter_col(kk - 8, 0)),
+                                   smem_desc(sB + kk * 2048,
                                              (uint32_t)r * 128, 1024),
                                    id_o, 1);
                         mma_commit(&bars.o_full[s]);
@@ -365,11 +366,10 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                     const int t = up / NPASS, pass = up - t * NPASS;
                     const int s = t & 1;
                     const int su = (t >> 1) * NPASS + pass;  // unit in slot
+                    const int vb = up % VS;
                     const uint32_t so = tm + 256u * s;
-                    const int vb = t % VS;
                     if (mbar_test(&bars.p_full[s], su & 1) &&
-                        mbar_test(&bars.v_full[vb],
-                                  (t / VS * NPASS + pass) & 1)) {
+                        mbar_test(&bars.v_full[vb], up / VS & 1)) {
                         fence_proxy_async_smem();  // cp.async data -> MMA
                         tc_fence_after();
                         const uint32_t sV = sV0 + vb * tileB;
@@ -378,27 +378,9 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                                    smem_desc(sV + kk * 2048, (uint32_t)nk * 128,
                                              1024),
                                    id_o, pass > 0 || kk > 0);
-                        if (pass < NPASS - 1) {
-                            mma_commit(&bars.pv0_done[s]);
-                            mma_commit(&bars.v_empty[vb]);
-                        } else {
-                            for (int kk = 0; kk < r0 / 16; ++kk)  // + Phi' B
-                                mma_ts(so + nk, so + quarter_col(kk, 32),
-                                       smem_desc(sB + kk * 2048,
-                                                 (uint32_t)r * 128, 1024),
-                                       id_o, 1);
-                            if constexpr (DIRECT)
-                                mma_commit(&bars.v_empty[vb]);
-                            if (two_parts) {
-                                mma_commit(&bars.pv_done[s]);
-                            } else {
-                                mma_commit(&bars.o_full[s]);
-                                if (t == ntiles - 1 || pp == tph - 1)
-                                    mma_commit(&bars.head_done);
-                            }
-                            ++tiles_pv;
-                            pp = adv(pp);
-                        }
+                        mma_commit(&bars.pv_done[s]);
+                        if (NPASS > 1) mma_commit(&bars.v_empty[vb]);
+                        if (pass == NPASS - 1) ++tiles_pv;
                         ++up;
                         did = true;
                     }
@@ -408,20 +390,18 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 // the previous head to be issued
                 const int ts = us / NPASS, spass = us - ts * NPASS;
                 const bool nh = spass == 0 && (ts == 0 || ps == 0);
-                if (us < nunits &&
-                    !(nh && ts > 0 && (two_parts ? i2 : tiles_pv) < ts)) {
-                    const int s = ts & 1;
+                if (us < nunits && !(nh && ts > 0 && i2 < ts)) {
+                    const int s = ts & 1, qb = us % QS;
                     const uint32_t so = tm + 256u * s;
-                    const int qb = us % QS;
                     bool ready = mbar_test(&bars.qk_full[qb], us / QS & 1);
                     if (ready && spass == 0)
                         ready = (ts < 2 || mbar_test(&bars.tmem_empty[s],
                                                      ((ts >> 1) - 1) & 1)) &&
                                 (!nh || mbar_test(&bars.wb_full, hc & 1));
                     if (ready && spass > 0)  // S columns hold P of pass - 1
-                        ready = mbar_test(&bars.pv0_done[s],
-                                          ((ts >> 1) * (NPASS - 1) + spass -
-                                           1) & 1);
+                        ready = mbar_test(
+                            &bars.pv_done[s],
+                            ((ts >> 1) * NPASS + spass - 1) & 1);
                     if (ready) {
                         if (nh) ++hc;
                         fence_proxy_async_smem();  // cp.async data -> MMA
@@ -438,15 +418,17 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                                    spass == 0 ? id_sp : id_s, kk > 0);
                         }
                         mma_commit(&bars.s_full[s]);
+                        mma_commit(&bars.qk_empty[qb]);
                         ++us;
                         if (spass == NPASS - 1) ps = adv(ps);
                         did = true;
                     }
                 }
                 if (did) {
-                    t_last = global_ns();
-                } else {
+                    idle = 0;
+                } else if ((++idle & 255u) == 0) {
                     if (*abort) break;
+                    if (idle == 256u) t_last = global_ns();
                     if (global_ns() - t_last > kWaitLimitNs) {
                         *abort = 1;
                         record_timeout(status, 41);
@@ -460,341 +442,327 @@ __global__ void __launch_bounds__(kWsThreads, 1)
         // ------------------------------------------------------ compute groups
         // warps 0-7: slot 0, warps 8-15: slot 1; within a slot, warps
         // (w, w + 4) share TMEM lanes and split the row in two halves.
-        const int cw = warp;
-        const int g = cw >> 3;                       // TMEM slot / tile parity
-        const int half = (cw >> 2) & 1;
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(
+            kWsRegsCompute));
+        const int g = warp >> 3;                     // TMEM slot / tile parity
+        const int half = (warp >> 2) & 1;
         const int row = (warp & 3) * 32 + lane_id;   // query row = TMEM lane
         const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
-        // RACE buckets of this half: the 64-bucket chunks c = half (written
-        // with P, before the P V product) and c = half + 2 (written after
-        // it); chunk c holds tables [c T, c T + T)
+        // RACE buckets of this half: the 64-bucket chunks c = half and
+        // c = half + 2 (buckets past 128); chunk c holds tables
+        // [c T, c T + T)
         constexpr int T = R >= 64 ? 1 : 64 / R;
         const int ta0 = min(half * T, L), nt0 = min(ta0 + T, L) - ta0;
         const int ta1 = min((half + 2) * T, L), nt1 = min(ta1 + T, L) - ta1;
         const uint32_t cb0 = half ? 96u : 32u, cb1 = half ? 64u : 0u;
         const float sl2e = scale * kLog2e;
         const int kbeg = half * (nk / 2);
-        // a slot's 256 threads leave a wait with one verdict (an abort
-        // seen by some warps only would strand the others at the slot's
-        // named barriers)
-        auto wwait = [=](uint64_t *bar, uint32_t par, int site) {
+        // barrier of the row's two warps; a pair's 64 threads leave a wait
+        // with one verdict (an abort seen by one warp only would strand the
+        // other there)
+        const int pid = 1 + g * 4 + (warp & 3);
+        auto pwait = [=](uint64_t *bar, uint32_t par, int site) {
             const bool ok = mbar_wait_or_abort(bar, par, abort, status, site);
-            return named_sync_and(1 + g, 256, ok);
+            return named_sync_and(pid, 64, ok);
         };
-        // The Q, K copies of tile t are issued by the slot of tile t - QS as
-        // soon as the scores of that tile free the Q, K buffer: 256 threads, whole rows per warp instruction; completion
-        // reaches qk_full through cp.async's own mbarrier arrivals.
-        const int ct = (cw & 7) * 32 + lane_id;  // 0..255 within the slot
-        auto issue_qk = [&](int t) -> bool {
-            if (!wwait(&bars.idx_full[t & 1], (t >> 1) & 1, 54)) return false;
-            const int cpr = d >> 3, rpp = 256 / cpr;
-            const int crow = ct / cpr, cc = ct - crow * cpr;
-            const int *qr = qkrow[t & 1][0], *kr = qkrow[t & 1][1];
-            const uint32_t dQ = sQ + (t % QS) * tileB;
-            const uint32_t dK = sKW + (t % QS) * tileKW;
-            for (int rr = crow; rr < nk; rr += rpp) {
-                cp_async16(dQ + panel_offset(rr, cc, nk),
-                           qx + (size_t)qr[rr] * d + cc * 8);
-                cp_async16(dK + panel_offset(rr, cc, NR),
-                           kx + (size_t)kr[rr] * d + cc * 8);
-            }
-            cp_async_mbar_arrive(&bars.qk_full[t % QS]);
-            mbar_arrive(&bars.idx_empty[t & 1]);
-            return true;
-        };
-        // keys of pass ps >= 1 of tile t (the queries stay): issued by the
-        // tile's own slot once the previous pass's scores are done
-        auto issue_k = [&](int t, int ps) -> bool {
-            if (!wwait(&bars.idx_full[t & 1], (t >> 1) & 1, 57)) return false;
-            const int cpr = d >> 3, rpp = 256 / cpr;
-            const int crow = ct / cpr, cc = ct - crow * cpr;
-            const int *kr = qkrow[t & 1][1 + ps];
-            for (int rr = crow; rr < nk; rr += rpp)
-                cp_async16(sKW + panel_offset(rr, cc, NR),
-                           kx + (size_t)kr[rr] * d + cc * 8);
-            cp_async_mbar_arrive(&bars.qk_full[0]);
-            mbar_arrive(&bars.idx_empty[t & 1]);
-            return true;
-        };
-        bool started = true;
-        if (g == 1)
-            for (int t = 0; t < QS && t < ntiles && started; ++t)
-                started = issue_qk(t);
-        for (int j = g; started && j < ntiles; j += 2) {
+        const int bh0 = tile_head(0);
+        int bh = tile_head(g), tih = tile_p0(g) / 128, last_bh = -1;
+        for (int j = g; j < ntiles; j += 2, tih += 2) {
             const int k = j >> 1;
             const uint32_t so = tm + 256u * g + lane;
-            const int bh = tile_head(j), p0 = tile_p0(j);
+            while (tih >= tiles_per_head) {
+                tih -= tiles_per_head;
+                ++bh;
+            }
+            const int p0 = tih * 128;
             const int qpos = p0 + row;
             const bool qvalid = qpos < N;
             int qi = perm_q[(size_t)bh * N + min(qpos, N - 1)];  // prefetch
-            if (!wwait(&bars.s_full[g], (k * NPASS) & 1, 51)) break;
-            tc_fence_after();
             // the A summary (read below) came by TMA: acquire its head's
-            // stage (complete already, since S of this tile waited for it)
-            if ((j < 2 || tile_head(j) != tile_head(j - 2)) &&
-                !wwait(&bars.wb_full, (tile_head(j) - tile_head(0)) & 1, 55))
+            // stage (complete already when S of this tile is)
+            if (bh != last_bh && !pwait(&bars.wb_full, (bh - bh0) & 1, 55))
                 break;
-            if constexpr (NPASS > 1) {
-                if (!issue_k(j, 1)) break;
-            } else {
-                if (j + QS < ntiles && !issue_qk(j + QS)) break;
-            }
-            // per-bit factors of this half's tables (sp[0, 16): chunk half,
-            // up to 32 when the chunk has more projection columns and no
-            // second chunk exists; sp[16, 32): chunk half + 2) and partial
-            // Den (A from shared memory: the loaders stage it with the
-            // planes; the MMA warp only starts tile j after that head's
-            // stage completed)
-            float sp[32];
-            if (nt0 * G > 16)
-                race_bits32(so + nk + ta0 * G, nt0 * G, beta, sp);
-            else
-                race_bits16(so + nk + ta0 * G, nt0 * G, beta, sp);
-            float dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // independent chains
-            chunk_den<G, T>(sp, nt0, Asm + ta0 * R, dacc);
-            // the second chunk's factors wait for the P V product: kept as
-            // fp16 pairs (factors lie in (0.11, 0.89); relative rounding
-            // 2^-11, below the bf16 rounding of the features they make)
-            uint32_t sp1[8];
-            if constexpr (T * G <= 16) {
-                if (nt1 > 0) {
-                    race_bits16(so + nk + ta1 * G, nt1 * G, beta, sp + 16);
-                    chunk_den<G, T>(sp + 16, nt1, Asm + ta1 * R, dacc);
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        sp1[q] = pack_f16x2(sp[16 + 2 * q], sp[17 + 2 * q]);
-                }
-            }
-            const float den = (dacc[0] + dacc[1]) + (dacc[2] + dacc[3]);
-            // softmax over this half's key columns
-            const int klo = b < 128 ? (row / b) * b : 0;
-            const int khi = b < 128 ? klo + b : nk;
-            float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            const bool masked = b < 128;
-            // pass 0 of a tile whose window starts before the sequence
-            const bool valid0 = !WIN || pass_valid(p0, 0);
+            last_bh = bh;
+            if (!pwait(&bars.s_full[g], (k * NPASS) & 1, 51)) break;
+            tc_fence_after();
             // SEL: this row's selected candidates among this half's 64 keys
             // of pass ps (bit k of the 64-bit word: key kbeg + k)
             const size_t selrow = (size_t)bh * N + (size_t)min(qpos, N - 1);
-            const int selw = tk_c * b / 32;
             auto selbits = [&](int ps) -> unsigned long long {
                 if (!SEL) return ~0ull;
-                const uint32_t *w = selmask + selrow * selw + 4 * ps + 2 * half;
+                const uint32_t *w = selmask + selrow * (tk_c * b / 32) +
+                                    4 * ps + 2 * half;
                 return (unsigned long long)w[0] |
                        ((unsigned long long)w[1] << 32);
             };
-            const unsigned long long sb0 = selbits(0);
-            // KB: the block of this warp's rows and this half's share of it
-            constexpr int KN = KB > 0 ? KB / 2 : 16;
-            uint32_t sv[KN];
-            const int kl = KB > 0 ? (warp & 3) * 32 / KN / 2 * KB : 0;
-            if constexpr (KB == 64) tmem_ld32(so + kl + half * KN, sv);
-            if constexpr (KB == 32) tmem_ld16(so + kl + half * KN, sv);
-            if constexpr (KB > 0) {
-                tmem_wait_ld();
-#pragma unroll
-                for (int jj = 0; jj < KN; ++jj)
-                    mxa[jj & 3] = fmaxf(mxa[jj & 3], __uint_as_float(sv[jj]));
-            }
-#pragma unroll
-            for (int c = 0; KB == 0 && c < nk / 2; c += 16) {
-                uint32_t v[16];
-                tmem_ld16(so + kbeg + c, v);
-                tmem_wait_ld();
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) {
-                    const int key = kbeg + c + jj;
-                    if ((!WIN || valid0) &&
-                        (!masked || (key >= klo && key < khi)) &&
-                        (!SEL || ((sb0 >> (c + jj)) & 1ull)))
-                        mxa[jj & 3] = fmaxf(mxa[jj & 3], __uint_as_float(v[jj]));
+            // row maximum of both halves
+            auto row_max = [&](const float (&m)[4]) {
+                xmax[g][half][row] =
+                    fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+                named_sync(pid, 64);
+                return fmaxf(xmax[g][0][row], xmax[g][1][row]);
+            };
+            float M2, lsum;  // reference (log2 units), this half's row sum
+            float lam = lambda, gs = 1.0f, gl = 1.0f;
+            size_t tok = 0;
+            auto token = [&] {
+                qi = (qi < 0 || qi >= N) ? 0 : qi;
+                tok = (size_t)bh * N + qi;
+                if (lambda_tok && qvalid) lam = lambda_tok[tok];
+                if (gates && qvalid) {
+                    const float2 gg =
+                        *reinterpret_cast<const float2 *>(gates + 2 * tok);
+                    gs = gg.x;
+                    gl = gg.y;
                 }
-            }
-            float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
-            xmax[g][half][row] = mx;
-            xden[g][half][row] = den;
-            named_sync(1 + g, 256);
-            mx = fmaxf(xmax[g][0][row], xmax[g][1][row]);
-            const float denf =
-                (xden[g][0][row] + xden[g][1][row]) * (1.0f / (float)L);
-            float M2 = mx * sl2e;
-            float ls[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            if constexpr (KB > 0) {
-                // P of the block over the first columns of its quarter, and
-                // zeros for the tile's other keys
-                const int q = kl & 64, w = (kl & 63) / 2;
-                uint32_t pw[KN / 2], zero[16];
-#pragma unroll
-                for (int jj = 0; jj < KN; jj += 2) {
-                    const float a0 = ex2_approx(
-                        fmaf(__uint_as_float(sv[jj]), sl2e, -M2));
-                    const float a1 = ex2_approx(
-                        fmaf(__uint_as_float(sv[jj + 1]), sl2e, -M2));
-                    ls[(jj >> 1) & 3] += a0 + a1;
-                    pw[jj >> 1] = pack_bf16x2(a0, a1);
-                }
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj) zero[jj] = 0u;
-                if constexpr (KB == 64) {
-                    tmem_st16(so + q + half * 16, pw);
-                } else {
-                    uint32_t z8[8];
-#pragma unroll
-                    for (int jj = 0; jj < 8; ++jj) z8[jj] = 0u;
-                    tmem_st8(so + q + w + half * 8, pw);
-                    tmem_st8(so + q + (w ^ 16) + half * 8, z8);
-                }
-                tmem_st16(so + (q ^ 64) + half * 16, zero);
-            }
-#pragma unroll
-            for (int c = 0; KB == 0 && c < nk / 2; c += 32) {
-                uint32_t pk16[16];
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    uint32_t v[16];
-                    tmem_ld16(so + kbeg + c + 16 * hh, v);
+            };
+            // per-bit factors of this half's tables: sp[0, 16) chunk half,
+            // sp[16, 32) chunk half + 2; up to 32 of chunk half when it has
+            // more projection columns (no second chunk exists then)
+            uint32_t pr[32];
+            auto load_projections = [&] {
+                if (T * G <= 16) {
+                    uint32_t a[16], c[16];
+                    tmem_ld16(so + nk + ta0 * G, a);
+                    tmem_ld16(so + nk + ta1 * G, c);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int jj = 0; jj < 16; jj += 2) {
-                        const int key = kbeg + c + 16 * hh + jj;
-                        float a0 = ex2_approx(
-                            fmaf(__uint_as_float(v[jj]), sl2e, -M2));
-                        float a1 = ex2_approx(
-                            fmaf(__uint_as_float(v[jj + 1]), sl2e, -M2));
-                        if (masked) {
-                            a0 = (key >= klo && key < khi) ? a0 : 0.0f;
-                            a1 = (key + 1 >= klo && key + 1 < khi) ? a1 : 0.0f;
-                        }
-                        if (WIN && !valid0) a0 = a1 = 0.0f;
-                        if (SEL) {
-                            const int kl = c + 16 * hh + jj;  // in the half
-                            a0 = ((sb0 >> kl) & 1ull) ? a0 : 0.0f;
-                            a1 = ((sb0 >> (kl + 1)) & 1ull) ? a1 : 0.0f;
-                        }
-                        ls[(jj >> 1) & 3] += a0 + a1;
-                        pk16[8 * hh + (jj >> 1)] = pack_bf16x2(a0, a1);
+                    for (int q = 0; q < 16; ++q) {
+                        pr[q] = a[q];
+                        pr[16 + q] = c[q];
+                    }
+                } else {
+                    tmem_ld32(so + nk + ta0 * G, pr);
+                    tmem_wait_ld();
+                }
+            };
+            // Den stays a sum over broadcast A values: through tensor memory
+            // into the 16x256b layout (every value of A read serves four
+            // rows) it took as long.
+            float den = 0.0f;
+            float sp[32];
+            auto features = [&] {
+                constexpr int n1 = T * G <= 16 ? 16 : 32;
+                race_factors<n1>(pr, nt0 * G, beta, sp);
+                float dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // independent chains
+                chunk_den<G, T>(sp, nt0, Asm + ta0 * R, dacc);
+                if constexpr (T * G <= 16) {
+                    if (nt1 > 0) {
+                        race_factors<16>(pr + 16, nt1 * G, beta, sp + 16);
+                        chunk_den<G, T>(sp + 16, nt1, Asm + ta1 * R, dacc);
                     }
                 }
-                // quarter 2h, over scores of this half already read
-                tmem_st16(so + kbeg + (c >> 1), pk16);
-            }
-            float lsum = (ls[0] + ls[1]) + (ls[2] + ls[3]);
-            xsum[g][half][row] = lsum;
-            tc_fence_before();
-            named_sync(1 + g, 256);  // every S read of the slot is done
-            tc_fence_after();
-            lsum = xsum[g][0][row] + xsum[g][1][row];
-            bool pass_fail = false;
-#pragma unroll
-            for (int ps = 1; ps < NPASS; ++ps) {
-                // the previous pass's P goes to its P V product; this pass
-                // scores the next 128 keys into the same columns
+                den = (dacc[0] + dacc[1]) + (dacc[2] + dacc[3]);
+            };
+            auto hand_over = [&](uint64_t *bar) {
                 tmem_wait_st();
                 tc_fence_before();
-                mbar_arrive(&bars.p_full[g]);
-                if (!wwait(&bars.s_full[g], (k * NPASS + ps) & 1, 56)) {
-                    pass_fail = true;
-                    break;
+                mbar_arrive(bar);
+            };
+            bool fail = false;
+            if constexpr (NPASS == 1) {
+                // this half's scores, up to 32 at a time: kept in registers
+                // from the maximum to P when that is all of them
+                constexpr int KN = KB > 0 ? KB / 2 : nk / 2;
+                constexpr int KC = KN < 32 ? KN : 32;
+                const int kl = KB > 0 ? (warp & 3) * 32 / KN / 2 * KB : 0;
+                const uint32_t own = so + kl + half * KN;
+                uint32_t sv[KC];
+                uint32_t sb[2] = {~0u, ~0u};
+                if constexpr (SEL) {
+                    const unsigned long long x = selbits(0);
+                    sb[0] = (uint32_t)x;
+                    sb[1] = (uint32_t)(x >> 32);
                 }
-                tc_fence_after();
-                // the K buffer is free again: the next pass's keys, or after
-                // the last pass the next tile's queries and keys
-                if (ps + 1 < NPASS) {
-                    if (!issue_k(j, ps + 1)) {
-                        pass_fail = true;
-                        break;
+                const int klo = (row / b) * b - kbeg;  // within the half
+                auto load = [&](int c) {  // scores [c, c + KC), masked
+                    if constexpr (KC == 32)
+                        tmem_ld32(own + c, sv);
+                    else
+                        tmem_ld16(own + c, sv);
+                    tmem_wait_ld();
+                    if (KB == 0 && b < 128) {
+#pragma unroll
+                        for (int q = 0; q < KC; ++q)
+                            if (c + q < klo || c + q >= klo + b)
+                                sv[q] = 0xff800000u;
                     }
-                } else if (j + 1 < ntiles && !issue_qk(j + 1)) {
-                    pass_fail = true;
-                    break;
+                    if constexpr (SEL) {
+#pragma unroll
+                        for (int q = 0; q < KC; ++q)
+                            if (!(sb[c / 32] >> q & 1u)) sv[q] = 0xff800000u;
+                    }
+                };
+                float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                for (int c = 0; c < KN; c += KC) {
+                    load(c);
+#pragma unroll
+                    for (int q = 0; q < KC; q += 2)
+                        mxa[(q >> 1) & 3] =
+                            max3(mxa[(q >> 1) & 3], __uint_as_float(sv[q]),
+                                 __uint_as_float(sv[q + 1]));
                 }
-                const bool pvalid = !WIN || pass_valid(p0, ps);
-                const unsigned long long sbp = selbits(ps);
-                float mxb[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-                if (!WIN || pvalid) {
+                M2 = row_max(mxa) * sl2e;
+                token();
+                float2 ls[2] = {make_float2(0.0f, 0.0f),
+                                make_float2(0.0f, 0.0f)};
+                const float2 sl2 = make_float2(sl2e, sl2e),
+                             m2n = make_float2(-M2, -M2);
+#pragma unroll
+                for (int c = 0; c < KN; c += KC) {
+                    if constexpr (KC < KN) load(c);
+                    uint32_t pw[KC / 2];
+#pragma unroll
+                    for (int q = 0; q < KC; q += 2) {
+                        const float2 z =
+                            fma2(make_float2(__uint_as_float(sv[q]),
+                                             __uint_as_float(sv[q + 1])),
+                                 sl2, m2n);
+                        const float2 e =
+                            make_float2(ex2_approx(z.x), ex2_approx(z.y));
+                        ls[(q >> 1) & 1] = add2(ls[(q >> 1) & 1], e);
+                        pw[q >> 1] = pack_bf16x2(e.x, e.y);
+                    }
+                    if constexpr (KB == 0)  // over scores already read
+                        tmem_st16(so + kbeg + (c >> 1), pw);
+                    // KB: over the first columns of the block's quarter
+                    // (both threads have read the scores there: row_max)
+                    if constexpr (KB == 64)
+                        tmem_st16(so + kl + half * 16, pw);
+                    if constexpr (KB == 32)
+                        tmem_st8(so + (kl & 64) + (kl & 32) / 2 + half * 8,
+                                 pw);
+                }
+                lsum = (ls[0].x + ls[1].x) + (ls[0].y + ls[1].y);
+                if constexpr (KB > 0) {  // zeros for the tile's other keys
+                    uint32_t zero[16];
+#pragma unroll
+                    for (int x = 0; x < 16; ++x) zero[x] = 0u;
+                    tmem_st16(so + (kl & 64 ^ 64) + half * 16, zero);
+                    if constexpr (KB == 32) {
+                        uint32_t z8[8];
+#pragma unroll
+                        for (int x = 0; x < 8; ++x) z8[x] = 0u;
+                        tmem_st8(so + (kl & 64) + ((kl & 32) / 2 ^ 16) +
+                                     half * 8,
+                                 z8);
+                    }
+                }
+                load_projections();
+                hand_over(&bars.p_full[g]);
+                features();
+            } else {
+                M2 = -INFINITY;
+                lsum = 0.0f;
+#pragma unroll
+                for (int ps = 0; ps < NPASS; ++ps) {
+                    if (ps > 0) {
+                        if (!pwait(&bars.s_full[g], (k * NPASS + ps) & 1,
+                                   56)) {
+                            fail = true;
+                            break;
+                        }
+                        tc_fence_after();
+                    }
+                    const bool pvalid = !WIN || pass_valid(p0, ps);
+                    const unsigned long long sb = selbits(ps);
+                    const uint32_t s0 = (uint32_t)sb, s1 = (uint32_t)(sb >> 32);
+                    auto keep = [=](int q) {  // key q of this half is attended
+                        return (!WIN || pvalid) &&
+                               (!SEL ||
+                                ((q < 32 ? s0 : s1) >> (q & 31) & 1u));
+                    };
+                    float mxa[4] = {-INFINITY, -INFINITY, -INFINITY,
+                                    -INFINITY};
 #pragma unroll
                     for (int c = 0; c < nk / 2; c += 16) {
                         uint32_t v[16];
                         tmem_ld16(so + kbeg + c, v);
                         tmem_wait_ld();
 #pragma unroll
-                        for (int jj = 0; jj < 16; ++jj)
-                            if (!SEL || ((sbp >> (c + jj)) & 1ull))
-                                mxb[jj & 3] = fmaxf(mxb[jj & 3],
-                                                    __uint_as_float(v[jj]));
+                        for (int q = 0; q < 16; ++q)
+                            if (keep(c + q))
+                                mxa[q & 3] =
+                                    fmaxf(mxa[q & 3], __uint_as_float(v[q]));
                     }
-                }
-                xmax[g][half][row] =
-                    fmaxf(fmaxf(mxb[0], mxb[1]), fmaxf(mxb[2], mxb[3]));
-                named_sync(1 + g, 256);
-                const float M2b =
-                    fmaxf(xmax[g][0][row], xmax[g][1][row]) * sl2e;
-                // online softmax: keep the running reference unless the
-                // row's max grew by more than 2^8; then rescale the
-                // accumulator (the previous P V product is complete: these
-                // scores waited for it) and the running sum. From an empty
-                // start (M2 = -inf) the factor is 0.
-                const bool need = M2b > M2 + 8.0f;
-                const float f = need ? ex2_approx(M2 - M2b) : 1.0f;
-                if (__any_sync(0xffffffffu, need)) {
+                    const float M2b = row_max(mxa) * sl2e;
+                    if (ps == 0) {
+                        token();
+                        M2 = M2b;
+                    } else {
+                        // online softmax: keep the running reference unless
+                        // the row's max grew by more than 2^8; then rescale
+                        // the accumulator (the previous P V product is
+                        // complete: these scores waited for it) and the
+                        // running sum. From an empty start (M2 = -inf) the
+                        // factor is 0.
+                        const bool need = M2b > M2 + 8.0f;
+                        const float f = need ? ex2_approx(M2 - M2b) : 1.0f;
+                        if (__any_sync(0xffffffffu, need)) {
 #pragma unroll
-                    for (int c = 0; c < 64; c += 16) {
-                        if (c < (d >> 1)) {
+                            for (int c = 0; c < 64; c += 16) {
+                                if (c < (d >> 1)) {
+                                    uint32_t v[16];
+                                    const uint32_t at =
+                                        so + nk + half * (d >> 1) + c;
+                                    tmem_ld16(at, v);
+                                    tmem_wait_ld();
+#pragma unroll
+                                    for (int q = 0; q < 16; ++q)
+                                        v[q] = __float_as_uint(
+                                            __uint_as_float(v[q]) * f);
+                                    tmem_st16(at, v);
+                                }
+                            }
+                        }
+                        if (need) {
+                            lsum *= f;
+                            M2 = M2b;
+                        }
+                    }
+                    float ls[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+                    for (int c = 0; c < nk / 2; c += 32) {
+                        uint32_t pw[16];
+#pragma unroll
+                        for (int hh = 0; hh < 2; ++hh) {
                             uint32_t v[16];
-                            tmem_ld16(so + nk + half * (d >> 1) + c, v);
+                            tmem_ld16(so + kbeg + c + 16 * hh, v);
                             tmem_wait_ld();
 #pragma unroll
-                            for (int q = 0; q < 16; ++q)
-                                v[q] = __float_as_uint(__uint_as_float(v[q]) * f);
-                            tmem_st16(so + nk + half * (d >> 1) + c, v);
-                        }
-                    }
-                }
-                if (need) {
-                    lsum *= f;
-                    M2 = M2b;
-                }
-                float lb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-                for (int c = 0; c < nk / 2; c += 32) {
-                    uint32_t pk16[16];
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t v[16];
-                        tmem_ld16(so + kbeg + c + 16 * hh, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int jj = 0; jj < 16; jj += 2) {
-                            float a0 = ex2_approx(
-                                fmaf(__uint_as_float(v[jj]), sl2e, -M2));
-                            float a1 = ex2_approx(
-                                fmaf(__uint_as_float(v[jj + 1]), sl2e, -M2));
-                            if (WIN && !pvalid) a0 = a1 = 0.0f;
-                            if (SEL) {
-                                const int kl = c + 16 * hh + jj;
-                                a0 = ((sbp >> kl) & 1ull) ? a0 : 0.0f;
-                                a1 = ((sbp >> (kl + 1)) & 1ull) ? a1 : 0.0f;
+                            for (int q = 0; q < 16; q += 2) {
+                                const int kq = c + 16 * hh + q;
+                                float a0 = ex2_approx(
+                                    fmaf(__uint_as_float(v[q]), sl2e, -M2));
+                                float a1 = ex2_approx(fmaf(
+                                    __uint_as_float(v[q + 1]), sl2e, -M2));
+                                a0 = keep(kq) ? a0 : 0.0f;
+                                a1 = keep(kq + 1) ? a1 : 0.0f;
+                                ls[(q >> 1) & 3] += a0 + a1;
+                                pw[8 * hh + (q >> 1)] = pack_bf16x2(a0, a1);
                             }
-                            lb[(jj >> 1) & 3] += a0 + a1;
-                            pk16[8 * hh + (jj >> 1)] = pack_bf16x2(a0, a1);
                         }
+                        // quarter 2h, over scores of this half already read
+                        tmem_st16(so + kbeg + (c >> 1), pw);
                     }
-                    tmem_st16(so + kbeg + (c >> 1), pk16);
+                    lsum += (ls[0] + ls[1]) + (ls[2] + ls[3]);
+                    if (ps == 0) load_projections();
+                    hand_over(&bars.p_full[g]);
+                    if (ps == 0) features();
                 }
-                xsum[g][half][row] = (lb[0] + lb[1]) + (lb[2] + lb[3]);
-                tc_fence_before();
-                named_sync(1 + g, 256);
-                tc_fence_after();
-                lsum += xsum[g][0][row] + xsum[g][1][row];
             }
-            if (pass_fail) break;
+            if (fail) break;
             // fusion scalars (Eq. (5) in log-sum-exp form, Eq. (6))
-            qi = (qi < 0 || qi >= N) ? 0 : qi;
-            const size_t tok = (size_t)bh * N + qi;
+            xsum[g][half][row] = make_float2(lsum, den);
+            named_sync(pid, 64);
+            {
+                const float2 o = xsum[g][half ^ 1][row];
+                lsum += o.x;
+                den += o.y;
+            }
+            const float denf = den * (1.0f / (float)L);
             const float log_ds = M2 * kLn2 + __logf(lsum);
-            const float lam = (lambda_tok && qvalid) ? lambda_tok[tok] : lambda;
-            const float gs = (gates && qvalid) ? gates[2 * tok] : 1.0f;
-            const float gl = (gates && qvalid) ? gates[2 * tok + 1] : 1.0f;
             const float msp =
                 fusion_multiplier_fast(log_ds, lam, denf, eps, mode);
             const float c1 =
@@ -803,127 +771,117 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             const float ratio =
                 __fdividef(gl, (float)L * (denf + eps) * c1e);
             if (nt0 > 0) write_phi_chunk<G, T>(sp, nt0, ratio, so + cb0);
-            tmem_wait_st();
-            tc_fence_before();
-            mbar_arrive(&bars.p_full[g]);
             if (r > nk) {
-                if (!wwait(&bars.pv_done[g], k & 1, 52)) break;
+                // over P: its product is complete
+                if (!pwait(&bars.pv_done[g], (k * NPASS + NPASS - 1) & 1, 52))
+                    break;
                 tc_fence_after();
                 if constexpr (T * G <= 16) {
-                    if (nt1 > 0) {
-                        float f1[16];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            unpack_f16x2(sp1[q], f1[2 * q], f1[2 * q + 1]);
-                        write_phi_chunk<G, T>(f1, nt1, ratio, so + cb1);
-                    }
+                    if (nt1 > 0)
+                        write_phi_chunk<G, T>(sp + 16, nt1, ratio, so + cb1);
                 }
-                tmem_wait_st();
-                tc_fence_before();
-                mbar_arrive(&bars.p2_full[g]);
             }
-            if (!wwait(&bars.o_full[g], k & 1, 53)) break;
+            hand_over(&bars.phi_full[g]);
+            if (!pwait(&bars.o_full[g], k & 1, 53)) break;
             tc_fence_after();
-            // O = c1 acc as bf16, this half's d / 2 columns, staged in this
-            // slot's V buffer (the P V product of the tile is complete) in
-            // the swizzled panel layout, then copied out by the slot's 256
-            // threads in whole rows (coalesced 16-byte stores). With an
-            // fp32 output (o32) each thread stores its half row directly.
-            const uint32_t sVg = sV0 + (j % VS) * tileB;
-            constexpr int kMaxHalf = 64;  // d / 2 for d = 128
-            if constexpr (DIRECT) {  // d = 64: 64 bytes per thread
-                uint32_t v[32];
-                tmem_ld32(so + nk + half * 32, v);
-                tmem_wait_ld();
-                tc_fence_before();
-                mbar_arrive(&bars.tmem_empty[g]);
-                if (qvalid) {
-                    uint16_t *dst = ox + tok * 64 + half * 32;
-                    const bool a32 = ((uintptr_t)ox & 31u) == 0;
+            // O = c1 acc, this half's d / 2 columns. d = 128: staged as bf16
+            // in the tile's value buffer (its products are complete) in the
+            // swizzled panel layout, 32 rows per warp, and stored in 128-byte
+            // rows; from registers, 32 bytes per lane and row, the kernel
+            // took 166 us at c3 where staging took 149. d = 64 (half of the
+            // bytes): from registers, 42 against 45 us at c2. An fp32 output
+            // is stored from registers.
+            // With several passes the value buffers are wanted sooner:
+            // staging took 284 us against 263 (two passes, c3 top-k).
+            const bool staged = !O32 && NPASS == 1 && d == 128;
+            const uint32_t sVg = sV0 + (uint32_t)(j % VS) * tileB;
+            constexpr int OW = O32 ? 32 : 16;  // words of 32 columns
+            uint32_t ov[2][OW];
 #pragma unroll
-                    for (int c = 0; c < 32; c += 16) {
-                        uint32_t ob[8];
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            ob[q] = pack_bf16x2(
-                                c1e * __uint_as_float(v[c + 2 * q]),
-                                c1e * __uint_as_float(v[c + 2 * q + 1]));
-                        if (a32) {
-                            st_global_v8(dst + c, ob);
-                        } else {
-                            uint4 *p = reinterpret_cast<uint4 *>(dst + c);
-                            p[0] = make_uint4(ob[0], ob[1], ob[2], ob[3]);
-                            p[1] = make_uint4(ob[4], ob[5], ob[6], ob[7]);
-                        }
-                    }
-                    if (half == 0) {
-                        if (log_ds_out) log_ds_out[tok] = log_ds;
-                        if (dlr_out) dlr_out[tok] = denf;
-                        if (m_out) m_out[tok] = msp;
-                    }
-                }
-                continue;
-            }
-#pragma unroll
-            for (int c = 0; c < kMaxHalf; c += 16) {
-                if (c < (d >> 1)) {
-                    uint32_t v[16], ob[8];
-                    tmem_ld16(so + nk + half * (d >> 1) + c, v);
+            for (int c = 0; c < 2; ++c) {
+                if (c == 0 || d == 128) {
+                    uint32_t v[32];
+                    tmem_ld32(so + nk + half * (d >> 1) + 32 * c, v);
                     tmem_wait_ld();
-                    if constexpr (O32) {
-                        if (qvalid) {
-                            float4 *dst = reinterpret_cast<float4 *>(
-                                o32 + tok * (size_t)d + half * (d >> 1) + c);
 #pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                dst[q] = make_float4(
-                                    c1e * __uint_as_float(v[4 * q]),
-                                    c1e * __uint_as_float(v[4 * q + 1]),
-                                    c1e * __uint_as_float(v[4 * q + 2]),
-                                    c1e * __uint_as_float(v[4 * q + 3]));
+                    for (int q = 0; q < OW; ++q) {
+                        if constexpr (O32) {
+                            ov[c][q] =
+                                __float_as_uint(c1e * __uint_as_float(v[q]));
+                        } else {
+                            const float2 x = mul2(
+                                make_float2(c1e, c1e),
+                                make_float2(__uint_as_float(v[2 * q]),
+                                            __uint_as_float(v[2 * q + 1])));
+                            ov[c][q] = pack_bf16x2(x.x, x.y);
                         }
-                        continue;
                     }
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        ob[q] = pack_bf16x2(c1e * __uint_as_float(v[2 * q]),
-                                            c1e * __uint_as_float(v[2 * q + 1]));
-                    const int cidx = (half * (d >> 1) + c) >> 3;  // 16-B chunk
-                    st_shared_v4(sVg + panel_offset(row, cidx, nk), ob[0],
-                                 ob[1], ob[2], ob[3]);
-                    st_shared_v4(sVg + panel_offset(row, cidx + 1, nk), ob[4],
-                                 ob[5], ob[6], ob[7]);
                 }
             }
             tc_fence_before();
             mbar_arrive(&bars.tmem_empty[g]);
-            if (half == 0) {
-                orow[g][row] = qvalid ? (int)tok : -1;
+            if (!staged) {
                 if (qvalid) {
+                    uint32_t *dst =
+                        (O32 ? reinterpret_cast<uint32_t *>(o32)
+                             : reinterpret_cast<uint32_t *>(ox)) +
+                        (tok * (size_t)d + half * (d >> 1)) * OW / 32;
+                    const bool a32 = ((uintptr_t)dst & 31u) == 0;
+#pragma unroll
+                    for (int c = 0; c < 2; ++c)
+#pragma unroll
+                        for (int q = 0; q < OW; q += 8)
+                            if (c == 0 || d == 128) {
+                                const uint32_t w[8] = {
+                                    ov[c][q],     ov[c][q + 1], ov[c][q + 2],
+                                    ov[c][q + 3], ov[c][q + 4], ov[c][q + 5],
+                                    ov[c][q + 6], ov[c][q + 7]};
+                                uint32_t *p = dst + c * OW + q;
+                                if (a32) {
+                                    st_global_v8(p, w);
+                                } else {
+                                    uint4 *p4 = reinterpret_cast<uint4 *>(p);
+                                    p4[0] =
+                                        make_uint4(w[0], w[1], w[2], w[3]);
+                                    p4[1] =
+                                        make_uint4(w[4], w[5], w[6], w[7]);
+                                }
+                            }
+                }
+            } else {
+                const int orow = qvalid ? (int)tok : -1;
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+#pragma unroll
+                    for (int q = 0; q < OW; q += 4)
+                        st_shared_v4(
+                            sVg + panel_offset(row, 8 * half + 4 * c + q / 4,
+                                               nk),
+                            ov[c][q], ov[c][q + 1], ov[c][q + 2],
+                            ov[c][q + 3]);
+                __syncwarp();
+                const int c16 = 8 * half + (lane_id & 7);
+#pragma unroll 4
+                for (int i = 0; i < 8; ++i) {
+                    const int rl = 4 * i + (lane_id >> 3);
+                    const int to = __shfl_sync(0xffffffffu, orow, rl);
+                    const uint4 val = ld_shared_v4(
+                        sVg + panel_offset((warp & 3) * 32 + rl, c16, nk));
+                    if (to >= 0)
+                        *reinterpret_cast<uint4 *>(ox + (size_t)to * d +
+                                                   c16 * 8) = val;
+                }
+                __syncwarp();  // the value buffer is read
+            }
+            if (NPASS == 1 && lane_id == 0) mbar_arrive(&bars.v_empty[j % VS]);
+            if (qvalid) {
+                if (half == 0) {
                     if (log_ds_out) log_ds_out[tok] = log_ds;
                     if (dlr_out) dlr_out[tok] = denf;
                     if (m_out) m_out[tok] = msp;
                 }
             }
-            named_sync(1 + g, 256);
-            if constexpr (!O32) {
-                const int ct = (cw & 7) * 32 + lane_id;  // 0..255
-                const int cpr = d >> 3, rpp = 256 / cpr;
-                const int crow = ct / cpr, cc = ct - crow * cpr;
-                for (int rr = crow; rr < nk; rr += rpp) {
-                    const int orr = orow[g][rr];
-                    if (orr >= 0) {
-                        const uint4 val =
-                            ld_shared_v4(sVg + panel_offset(rr, cc, nk));
-                        *reinterpret_cast<uint4 *>(ox + (size_t)orr * d +
-                                                   cc * 8) = val;
-                    }
-                }
-            }
-            named_sync(1 + g, 256);  // the staging buffer is read
-            if (cw == 8 * g && lane_id == 0) mbar_arrive(&bars.v_empty[j % VS]);
         }
-        cp_async_wait<0>();
     }
     tc_fence_before();
     __syncthreads();
@@ -1007,7 +965,8 @@ cudaError_t launch_block_attn_ws(
     // r = 128); at d = 128 one fits. Key blocks of 32 and 64 take half and a
     // quarter of the softmax work of the masked path. Both together, B4 H12
     // N4096 d64 b64 r128: 63 -> 45 us; B8 H12 N8192: 215 -> 138 us; B3 H5
-    // N4800 d128 b64 (KB alone): 35 -> 27 us.
+    // N4800 d128 b64 (KB alone): 35 -> 27 us. (42, 129 and 25 us since the
+    // copies have warps of their own.)
     if (P.gamma == 4 && P.sel == 0 && passes == 1) {
         auto pick = [&](auto o32) {
             constexpr bool F = decltype(o32)::value;

@@ -87,25 +87,6 @@ __device__ __forceinline__ void for_scores(uint32_t taddr, F f) {
     }
 }
 
-// Sum of two packed fp32 pairs, and a b + c on packed pairs.
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;"
-        : "=l"(r)
-        : "l"(*reinterpret_cast<unsigned long long *>(&a)),
-          "l"(*reinterpret_cast<unsigned long long *>(&b)));
-    return *reinterpret_cast<float2 *>(&r);
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;"
-        : "=l"(r)
-        : "l"(*reinterpret_cast<unsigned long long *>(&a)),
-          "l"(*reinterpret_cast<unsigned long long *>(&b)),
-          "l"(*reinterpret_cast<unsigned long long *>(&c)));
-    return *reinterpret_cast<float2 *>(&r);
-}
-
 // The canonical chain of two rows of d bf16 values, 64 values in flight.
 __device__ __forceinline__ float row_chain(const uint16_t *__restrict__ a,
                                            const uint16_t *__restrict__ b,
