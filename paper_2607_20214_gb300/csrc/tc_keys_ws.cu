@@ -6,9 +6,9 @@
 // N = d + 16 and its last 16 columns accumulate Phi^T 1.
 //
 // Roles (320 threads):
-//   warp 0      loader (lane 0): TMA loads of key tiles (two buffers) and
-//               value tiles (one buffer, one tile behind the keys);
-//               completion is counted in bytes on the buffers' mbarriers.
+//   warp 0      loader (lane 0): TMA loads of key tiles and value tiles
+//               (two buffers, one tile behind the keys); completion is
+//               counted in bytes on the buffers' mbarriers.
 //   warp 1      allocates tensor memory and issues the MMAs (lane 0): the
 //               projections W^(l) K of tile i+1 (double-buffered in TMEM)
 //               are issued before the summary MMAs of tile i.
@@ -37,7 +37,7 @@ struct KwBars {
 };
 
 template <int G>
-__global__ void __launch_bounds__(kKwThreads, 1)
+__global__ void __launch_bounds__(kKwThreads, 2)
     k_race_keys_ws(const __grid_constant__ CUtensorMap tmK,
                    const __grid_constant__ CUtensorMap tmV,
                    const __grid_constant__ CUtensorMap tmW, int N, int d,
@@ -59,10 +59,23 @@ __global__ void __launch_bounds__(kKwThreads, 1)
 
     const uint32_t base = align1k(smem_u32(smem_raw));
     const uint32_t tileB = 128u * d * 2u;
+    // One feature tile, two value tiles and one panel of ones that serves
+    // both: the panels of a B operand are a fixed stride apart, so value tile
+    // 0 lies 16 KB panel by panel before the ones and value tile 1 at a
+    // wider stride, around a key tile. d = 128: key tiles 0 and 1, d = 64:
+    // one (two CTAs then still fit an SM).
+    //   d = 128  W | K1 | V1.0 | K0 | V1.1 | V0.0 | V0.1 | ones | features
+    //   d = 64   W | K0 | V1 | V0 | ones | features
+    const int nkb = d == 128 ? 2 : 1;
     const uint32_t sW = base;
-    const uint32_t sK0 = sW + align1k(Lg_pad * d * 2);  // two key tiles
-    const uint32_t sV = sK0 + 2 * tileB;  // value tile, then a ones panel
-    const uint32_t sPhi = sV + tileB + 16384u;  // one feature tile
+    const uint32_t s1 = sW + align1k(Lg_pad * d * 2);
+    const uint32_t sK0 = d == 128 ? s1 + tileB + 16384u : s1;
+    const uint32_t sK1 = s1;
+    const uint32_t sV1 = s1 + tileB;
+    const uint32_t vs1 = d == 128 ? 49152u : 32768u;  // panel stride of V1
+    const uint32_t sOnes = sV1 + vs1 * (d / 64);
+    const uint32_t sV0 = sOnes - tileB;
+    const uint32_t sPhi = sOnes + 16384u;
 
     // TMEM columns: per M-tile an accumulator of d + 16 columns (B, then A
     // repeated 16 times), then two projection buffers of 64 columns.
@@ -87,7 +100,7 @@ __global__ void __launch_bounds__(kKwThreads, 1)
     }
     for (int i = tid; i < 16384 / 16; i += kKwThreads)  // bf16 ones
         asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
-                         sV + tileB + i * 16),
+                         sOnes + i * 16),
                      "r"(0x3F803F80u)
                      : "memory");
     fence_proxy_async_smem();
@@ -126,43 +139,37 @@ __global__ void __launch_bounds__(kKwThreads, 1)
     if (warp == 0) {
         // ------------------------------------------------------------- loader
         if (lane_id == 0) {
-            // K(i) needs the projection of tile i-2 done, V(i) the summary
-            // MMAs of tile i-1; K runs ahead of V
-            int iv = 0;
-            for (int i = 0; i < ntiles; ++i) {
-                const int b = i & 1;
-                if (i >= 2 && !mbar_wait_or_abort(&bars.k_empty[b],
+            // K(i) needs the projection of tile i - nkb done, V(i) the
+            // summary MMAs of tile i - 2; V runs one tile behind K
+            auto load_v = [&](int i) {
+                if (i >= 2 && !mbar_wait_or_abort(&bars.v_empty[i & 1],
                                                   ((i >> 1) - 1) & 1, abort,
-                                                  status, 61))
-                    break;
-                // rows past the chunk are loaded too (next head, or zeros
-                // past the tensor) and get zero features
-                const int y = bh * N + c0 + i * 128;
-                mbar_expect_tx(&bars.k_full[b], tileB);
+                                                  status, 62))
+                    return false;
+                mbar_expect_tx(&bars.v_full[i & 1], tileB);
                 for (int pnl = 0; pnl < d / 64; ++pnl)
-                    tma_load_2d(sK0 + b * tileB + pnl * 16384, &tmK, 64 * pnl,
-                                y, &bars.k_full[b]);
-                // values up to tile i - 1 (one tile behind the keys)
-                for (; iv < i; ++iv) {
-                    if (iv >= 1 && !mbar_wait_or_abort(&bars.v_empty[0],
-                                                       (iv - 1) & 1, abort,
-                                                       status, 62))
+                    tma_load_2d((i & 1) ? sV1 + pnl * vs1
+                                        : sV0 + pnl * 16384,
+                                &tmV, 64 * pnl, bh * N + c0 + i * 128,
+                                &bars.v_full[i & 1]);
+                return true;
+            };
+            for (int i = 0; i <= ntiles; ++i) {
+                if (i < ntiles) {
+                    const int b = i % nkb;
+                    if (i >= nkb && !mbar_wait_or_abort(&bars.k_empty[b],
+                                                        (i / nkb - 1) & 1,
+                                                        abort, status, 61))
                         break;
-                    mbar_expect_tx(&bars.v_full[0], tileB);
+                    // rows past the chunk are loaded too (next head, or
+                    // zeros past the tensor) and get zero features
+                    mbar_expect_tx(&bars.k_full[b], tileB);
                     for (int pnl = 0; pnl < d / 64; ++pnl)
-                        tma_load_2d(sV + pnl * 16384, &tmV, 64 * pnl,
-                                    bh * N + c0 + iv * 128, &bars.v_full[0]);
+                        tma_load_2d((b ? sK1 : sK0) + pnl * 16384, &tmK,
+                                    64 * pnl, bh * N + c0 + i * 128,
+                                    &bars.k_full[b]);
                 }
-            }
-            for (; iv < ntiles; ++iv) {
-                if (iv >= 1 && !mbar_wait_or_abort(&bars.v_empty[0],
-                                                   (iv - 1) & 1, abort,
-                                                   status, 62))
-                    break;
-                mbar_expect_tx(&bars.v_full[0], tileB);
-                for (int pnl = 0; pnl < d / 64; ++pnl)
-                    tma_load_2d(sV + pnl * 16384, &tmV, 64 * pnl,
-                                bh * N + c0 + iv * 128, &bars.v_full[0]);
+                if (i > 0 && !load_v(i - 1)) break;
             }
         }
         __syncwarp();
@@ -173,7 +180,8 @@ __global__ void __launch_bounds__(kKwThreads, 1)
             const uint32_t id_b = idesc_bf16(128, d + 16, true, true);
             const int last0 = last_mtile(0), last1 = last_mtile(1);
             auto proj = [=](int it) {
-                const uint32_t sK = sK0 + (it & 1) * tileB;
+                const int kb = it % nkb;
+                const uint32_t sK = kb ? sK1 : sK0;
                 const uint32_t dst = t + colP + 64u * (it & 1);
                 for (int k = 0; k < d / 16; ++k) {
                     uint32_t oa = (k >> 2) * 128 * 128 + (k & 3) * 32;
@@ -182,14 +190,15 @@ __global__ void __launch_bounds__(kKwThreads, 1)
                            smem_desc(sW + ow, 16, 1024), id_proj, k > 0);
                 }
                 mma_commit(&bars.proj_full[it & 1]);
-                mma_commit(&bars.k_empty[it & 1]);
+                mma_commit(&bars.k_empty[kb]);
             };
             // projections run two tiles ahead (both TMEM buffers); each
             // iteration issues the summary MMAs of tile i, then the
             // projection of tile i + 2
             bool ok = mbar_wait_or_abort(&bars.w_full, 0, abort, status, 60);
             for (int it = 0; it < 2 && it < ntiles && ok; ++it) {
-                ok = mbar_wait_or_abort(&bars.k_full[it], 0, abort, status, 63);
+                ok = mbar_wait_or_abort(&bars.k_full[it % nkb], (it / nkb) & 1,
+                                        abort, status, 63);
                 if (ok) {
                     tc_fence_after();
                     proj(it);
@@ -197,8 +206,10 @@ __global__ void __launch_bounds__(kKwThreads, 1)
             }
             for (int i = 0; i < ntiles && ok; ++i) {
                 const int b = i & 1;
-                ok = mbar_wait_or_abort(&bars.v_full[0], i & 1, abort,
+                ok = mbar_wait_or_abort(&bars.v_full[b], (i >> 1) & 1, abort,
                                         status, 66);
+                const uint32_t sV = b ? sV1 : sV0;
+                const uint32_t vst = b ? vs1 : 16384u;
                 bool got0 = false, got1 = false;
                 for (int m = 0; m < nM && ok; ++m) {
                     if (tile_needs(m, 0) && !got0)
@@ -214,19 +225,19 @@ __global__ void __launch_bounds__(kKwThreads, 1)
                                                16384, 1024);
                         uint32_t acc = (i > 0 || k > 0) ? 1u : 0u;
                         mma_ss(t + m * accN, a,
-                               smem_desc(sV + k * 2048, 128 * 128, 1024), id_b,
+                               smem_desc(sV + k * 2048, vst, 1024), id_b,
                                acc);
                     }
                     if (m == last0) mma_commit(&bars.phi_empty[0]);
                     if (m == last1) mma_commit(&bars.phi_empty[1]);
                 }
                 if (!ok) break;
-                mma_commit(&bars.v_empty[0]);
+                mma_commit(&bars.v_empty[b]);
                 if (i + 2 < ntiles) {
                     // the features of tile i have read projection buffer b
-                    ok = mbar_wait_or_abort(&bars.k_full[b],
-                                            ((i + 2) >> 1) & 1, abort, status,
-                                            64);
+                    ok = mbar_wait_or_abort(&bars.k_full[(i + 2) % nkb],
+                                            ((i + 2) / nkb) & 1, abort,
+                                            status, 64);
                     if (!ok) break;
                     tc_fence_after();
                     proj(i + 2);
@@ -255,13 +266,16 @@ __global__ void __launch_bounds__(kKwThreads, 1)
         for (int i = 0; i < ntiles; ++i) {
             const int b = i & 1;
             ok = wwait(&bars.proj_full[b], (i >> 1) & 1, 67);
-            if (ok && i >= 1 && writes)
-                ok = wwait(&bars.phi_empty[hb], (i - 1) & 1, 68);
             if (!ok) break;
             tc_fence_after();
+            // the bit factors need only the projections: they are computed
+            // while the summary MMAs still read the last features
             float sp[32];
             race_bits32(t + lane + colP + 64u * b + l0 * G, (l1 - l0) * G,
                         beta, sp);
+            if (i >= 1 && writes)
+                ok = wwait(&bars.phi_empty[hb], (i - 1) & 1, 68);
+            if (!ok) break;
             const bool valid = c0 + i * 128 + row < c1;
             float buf[8];
 #pragma unroll
@@ -361,7 +375,8 @@ size_t race_keys_ws_smem(const Plan &P) {
     const size_t r_pad = (P.r + 127) / 128 * 128;
     const size_t lg_pad = (P.L * P.gamma + 15) / 16 * 16;
     return 1024 + (lg_pad * P.d * 2 + 1023) / 1024 * 1024 +
-           3 * (size_t)128 * P.d * 2 + 16384 + 128 * r_pad * 2;
+           (P.d == 128 ? 4 : 3) * (size_t)128 * P.d * 2 + 16384 +
+           128 * r_pad * 2;
 }
 
 uint32_t race_keys_ws_cols(const Plan &P) {
