@@ -363,6 +363,287 @@ __global__ void __launch_bounds__(kKwThreads, 2)
     if (warp == 1) tmem_dealloc(t, tmem_cols);
 }
 
+// The same summaries for d = 128 and gamma = 4, with the product turned
+// round: D = V^T Phi, lanes = value dimensions, N = r buckets, so that a tile
+// takes 8 MMAs of N = r where Phi^T [V | 1] takes 16 of N = 144 (which ran at
+// 80 ns each beside the copies and feature stores: shared-memory bandwidth),
+// and the feature tile is handed over per 64 keys. A = Phi^T 1 is summed by
+// four more warps, one per 64 buckets, from the bf16 features that the MMAs
+// read. Live beside the sort hash: c3 103 -> 82 us, c4 412 -> 340 us (with A as
+// MMAs of N = 16 against ones, 0.8 us per tile, 97 us at c3; summed by the
+// feature threads 141). Roles and copies as above.
+struct KtBars {
+    uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2], w_full, done;
+    uint64_t proj_full[2];
+    uint64_t phi_full[2], phi_empty[2];  // per 64 keys
+};
+
+constexpr int kKtThreads = kKwThreads + 128;
+
+template <int NT>  // tables per row half, 4 or 8 (L <= 2 NT)
+__global__ void __launch_bounds__(kKtThreads, 1)
+    k_race_keys_t(const __grid_constant__ CUtensorMap tmK,
+                  const __grid_constant__ CUtensorMap tmV,
+                  const __grid_constant__ CUtensorMap tmW, int N, int H, int L,
+                  int Lg_pad, int chunk, float beta, float *__restrict__ part,
+                  DeviceStatus *status) {
+    constexpr int d = 128;
+    constexpr uint32_t tileB = 128u * d * 2u, colP = 256;
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ KtBars bars;
+    __shared__ uint32_t tbase;
+    __shared__ int abort_flag;
+    volatile int *abort = &abort_flag;
+    const int s = blockIdx.x, bh = blockIdx.y, S = gridDim.x;
+    const int h = bh % H;
+    const int tid = threadIdx.x, warp = tid >> 5, lane_id = tid & 31;
+    const int r = 16 * L;
+    const uint32_t sW = align1k(smem_u32(smem_raw));
+    const uint32_t sK0 = sW + align1k(Lg_pad * d * 2);
+    const uint32_t sV0 = sK0 + 2 * tileB;
+    const uint32_t sPhi = sV0 + 2 * tileB;
+    const int panels = (r + 63) >> 6;
+
+    if (warp == 1) tmem_alloc(&tbase, 512);
+    if (tid == 0) {
+        mbar_init(&bars.done, 1);
+        mbar_init(&bars.w_full, 1);
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&bars.k_full[b], 1);
+            mbar_init(&bars.k_empty[b], 1);
+            mbar_init(&bars.v_full[b], 1);
+            mbar_init(&bars.v_empty[b], 1);
+            mbar_init(&bars.proj_full[b], 1);
+            mbar_init(&bars.phi_full[b], 128);
+            mbar_init(&bars.phi_empty[b], 1 + panels);
+        }
+        abort_flag = 0;
+        fence_mbar_init();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t t = tbase;
+    const int c0 = s * chunk;
+    const int c1 = min(N, c0 + chunk);
+    const int ntiles = c1 > c0 ? (c1 - c0 + 127) / 128 : 0;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------- loader
+        if (lane_id == 0 && ntiles > 0) {
+            mbar_expect_tx(&bars.w_full, (uint32_t)Lg_pad * d * 2u);
+            for (int pnl = 0; pnl < 2; ++pnl)
+                tma_load_2d(sW + pnl * Lg_pad * 128, &tmW, 64 * pnl,
+                            h * Lg_pad, &bars.w_full);
+            // K(i) needs the projection of tile i - 2 done, V(i) the summary
+            // MMAs of tile i - 2; V runs one tile behind K. Rows past the
+            // chunk are loaded too (next head, or zeros past the tensor)
+            // and get zero features.
+            auto load = [&](int i, uint64_t *full, uint64_t *empty,
+                            uint32_t dst, const CUtensorMap *map, int site) {
+                const int b = i & 1;
+                if (i >= 2 && !mbar_wait_or_abort(&empty[b],
+                                                  ((i >> 1) - 1) & 1, abort,
+                                                  status, site))
+                    return false;
+                mbar_expect_tx(&full[b], tileB);
+                for (int pnl = 0; pnl < 2; ++pnl)
+                    tma_load_2d(dst + b * tileB + pnl * 16384, map, 64 * pnl,
+                                bh * N + c0 + i * 128, &full[b]);
+                return true;
+            };
+            for (int i = 0; i <= ntiles; ++i) {
+                if (i < ntiles &&
+                    !load(i, bars.k_full, bars.k_empty, sK0, &tmK, 61))
+                    break;
+                if (i > 0 &&
+                    !load(i - 1, bars.v_full, bars.v_empty, sV0, &tmV, 62))
+                    break;
+            }
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ----------------------------------------------------------- MMA issue
+        if (lane_id == 0 && ntiles > 0) {
+            const uint32_t id_proj = idesc_bf16(128, Lg_pad, false, false);
+            const uint32_t id_b = idesc_bf16(128, r, true, true);
+            auto proj = [=](int it) {
+                const uint32_t sK = sK0 + (it & 1) * tileB;
+                const uint32_t dst = t + colP + 64u * (it & 1);
+                for (int k = 0; k < d / 16; ++k) {
+                    uint32_t oa = (k >> 2) * 128 * 128 + (k & 3) * 32;
+                    uint32_t ow = (k >> 2) * Lg_pad * 128 + (k & 3) * 32;
+                    mma_ss(dst, smem_desc(sK + oa, 16, 1024),
+                           smem_desc(sW + ow, 16, 1024), id_proj, k > 0);
+                }
+                mma_commit(&bars.proj_full[it & 1]);
+                mma_commit(&bars.k_empty[it & 1]);
+            };
+            // projections run two tiles ahead (both TMEM buffers)
+            bool ok = mbar_wait_or_abort(&bars.w_full, 0, abort, status, 60);
+            for (int it = 0; it < 2 && it < ntiles && ok; ++it) {
+                ok = mbar_wait_or_abort(&bars.k_full[it], 0, abort, status, 63);
+                if (ok) {
+                    tc_fence_after();
+                    proj(it);
+                }
+            }
+            for (int i = 0; i < ntiles && ok; ++i) {
+                const int b = i & 1;
+                ok = mbar_wait_or_abort(&bars.v_full[b], (i >> 1) & 1, abort,
+                                        status, 66);
+                for (int kh = 0; kh < 2 && ok; ++kh) {
+                    ok = mbar_wait_or_abort(&bars.phi_full[kh], i & 1, abort,
+                                            status, 65);
+                    if (!ok) break;
+                    tc_fence_after();
+                    for (int k = 4 * kh; k < 4 * kh + 4; ++k)  // 16 keys each
+                        mma_ss(t,
+                               smem_desc(sV0 + b * tileB + k * 2048, 16384,
+                                         1024),
+                               smem_desc(sPhi + k * 2048, 16384, 1024), id_b,
+                               (i > 0 || k > 0) ? 1u : 0u);
+                    mma_commit(&bars.phi_empty[kh]);
+                }
+                if (!ok) break;
+                mma_commit(&bars.v_empty[b]);
+                if (i + 2 < ntiles) {
+                    // the features of tile i have read projection buffer b
+                    ok = mbar_wait_or_abort(&bars.k_full[b],
+                                            ((i + 2) >> 1) & 1, abort, status,
+                                            64);
+                    if (!ok) break;
+                    tc_fence_after();
+                    proj(i + 2);
+                }
+            }
+            if (ok) mma_commit(&bars.done);
+        }
+        __syncwarp();
+    } else if (warp >= 10) {
+        // ------------------------------------------- A of buckets 64 p + ..
+        const int p = warp - 10;
+        if (p < panels) {
+            // lane: 8 buckets (16-byte chunk lane mod 8) of every fourth key
+            const int ch = lane_id & 7, sub = lane_id >> 3;
+            float2 a[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) a[q] = make_float2(0.0f, 0.0f);
+            bool ok = true;
+            for (int i = 0; i < ntiles && ok; ++i)
+                for (int kh = 0; kh < 2 && ok; ++kh) {
+                    ok = __all_sync(0xffffffffu,
+                                    mbar_wait_or_abort(&bars.phi_full[kh],
+                                                       i & 1, abort, status,
+                                                       70));
+                    if (!ok) break;
+                    const uint32_t at = sPhi + p * 16384;
+#pragma unroll 8
+                    for (int x = 0; x < 16; ++x) {
+                        const uint4 v = ld_shared_v4(
+                            at + panel_offset(64 * kh + 4 * x + sub, ch, 128));
+                        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q)
+                            a[q] = add2(
+                                a[q],
+                                make_float2(
+                                    __uint_as_float(w[q] << 16),
+                                    __uint_as_float(w[q] & 0xffff0000u)));
+                    }
+                    __syncwarp();
+                    if (lane_id == 0) mbar_arrive(&bars.phi_empty[kh]);
+                }
+            float *outA =
+                part + ((size_t)bh * S + s) * ((size_t)r * d + r) +
+                (size_t)r * d;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+#pragma unroll
+                for (int o = 8; o < 32; o <<= 1) {
+                    a[q].x += __shfl_xor_sync(0xffffffffu, a[q].x, o);
+                    a[q].y += __shfl_xor_sync(0xffffffffu, a[q].y, o);
+                }
+                const int bucket = 64 * p + 8 * ch + 2 * q;
+                if (sub == 0 && ok && ntiles > 0 && bucket < r)
+                    *reinterpret_cast<float2 *>(outA + bucket) = a[q];
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ features
+        const int half = (warp - 2) >> 2;
+        const int row = (warp & 3) * 32 + lane_id;  // key row = TMEM lane
+        const int kh = row >> 6;
+        const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
+        const int l0 = min(half * NT, L), nt = min(l0 + NT, L) - l0;
+        auto wwait = [=](uint64_t *bar, uint32_t par, int site) {
+            return __all_sync(0xffffffffu,
+                              mbar_wait_or_abort(bar, par, abort, status,
+                                                 site));
+        };
+        bool ok = true;
+        for (int i = 0; i < ntiles; ++i) {
+            const int b = i & 1;
+            ok = wwait(&bars.proj_full[b], (i >> 1) & 1, 67);
+            if (!ok) break;
+            tc_fence_after();
+            float sp[NT * 4];
+            if constexpr (NT == 8) {
+                uint32_t pr[32];
+                tmem_ld32(t + lane + colP + 64u * b + l0 * 4, pr);
+                tmem_wait_ld();
+                race_factors<32>(pr, beta, sp);
+            } else {
+                uint32_t pr[16];
+                tmem_ld16(t + lane + colP + 64u * b + l0 * 4, pr);
+                tmem_wait_ld();
+                race_factors<16>(pr, beta, sp);
+            }
+            if (i >= 1) ok = wwait(&bars.phi_empty[kh], (i - 1) & 1, 68);
+            if (!ok) break;
+            const float one = c0 + i * 128 + row < c1 ? 1.0f : 0.0f;
+#pragma unroll
+            for (int lt = 0; lt < NT; ++lt) {
+                if (lt < nt) {
+                    float u[4], w[4];
+                    table_uw4(&sp[lt * 4], one, u, w);
+                    uint32_t pk[8];
+                    table_pack4(u, w, pk);
+                    const uint32_t cc = (uint32_t)(l0 + lt) * 2;
+                    st_shared_v4(sPhi + panel_offset(row, cc, 128), pk[0],
+                                 pk[1], pk[2], pk[3]);
+                    st_shared_v4(sPhi + panel_offset(row, cc + 1, 128), pk[4],
+                                 pk[5], pk[6], pk[7]);
+                }
+            }
+            fence_proxy_async_smem();
+            tc_fence_before();
+            mbar_arrive(&bars.phi_full[kh]);
+        }
+        // partial summaries of this chunk: lane = value dimension; the
+        // halves take every other 16 buckets
+        float *out = part + ((size_t)bh * S + s) * ((size_t)r * d + r);
+        if (ok && ntiles > 0) ok = wwait(&bars.done, 0, 69);
+        if (ok && ntiles > 0) {
+            tc_fence_after();
+            for (int c = half; c < L; c += 2) {
+                uint32_t v[16];
+                tmem_ld16(t + lane + 16 * c, v);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    out[(size_t)(16 * c + j) * d + row] =
+                        __uint_as_float(v[j]);
+            }
+        } else if (ntiles == 0) {
+            for (int i = tid - 64; i < r * d + r; i += 256) out[i] = 0.0f;
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) tmem_dealloc(t, 512);
+}
+
 uint32_t pow2_cols_kw(uint32_t n) {
     uint32_t c = 32;
     while (c < n) c <<= 1;
@@ -437,6 +718,21 @@ cudaError_t launch_race_keys_ws(const Plan &P, const void *k, const void *v,
             P.beta, cols, part, status);
         return cudaGetLastError();
     };
+    if (P.d == 128 && P.gamma == 4) {
+        const size_t sm = 1024 + (size_t)lg_pad * P.d * 2 +
+                          4 * (size_t)128 * P.d * 2 +
+                          (size_t)((P.r + 63) / 64) * 16384;
+        auto launch_t = [&](auto kern) {
+            cudaFuncSetAttribute(
+                kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+            kern<<<grid, kKtThreads, sm, st>>>(tmK, tmV, tmW, P.N, P.H, P.L,
+                                               lg_pad, P.chunk, P.beta, part,
+                                               status);
+            return cudaGetLastError();
+        };
+        return P.L > 8 ? launch_t(k_race_keys_t<8>)
+                       : launch_t(k_race_keys_t<4>);
+    }
     switch (P.gamma) {
         case 1: return launch(k_race_keys_ws<1>);
         case 2: return launch(k_race_keys_ws<2>);

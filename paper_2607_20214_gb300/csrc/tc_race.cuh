@@ -84,19 +84,15 @@ __device__ __forceinline__ void race_factors16(const uint32_t *pr, int ncols,
 }
 
 // The per-bit factors of n projections already loaded from TMEM (fp32 bits
-// in pr), entries past `ncols` set to 1/2.
+// in pr). Columns past the last table give values that nothing reads.
 template <int n>
-__device__ __forceinline__ void race_factors(const uint32_t *pr, int ncols,
-                                             float beta, float *sp) {
+__device__ __forceinline__ void race_factors(const uint32_t *pr, float beta,
+                                             float *sp) {
 #pragma unroll
-    for (int j = 0; j < n; ++j) {
-        sp[j] = 0.5f;
-        if (j < ncols)
-            sp[j] = fmaf(0.5f,
-                         tanh_approx(beta *
-                                     tanh_approx(__uint_as_float(pr[j]))),
-                         0.5f);
-    }
+    for (int j = 0; j < n; ++j)
+        sp[j] = fmaf(0.5f,
+                     tanh_approx(beta * tanh_approx(__uint_as_float(pr[j]))),
+                     0.5f);
 }
 
 // race_bits32 over 16 projection columns: sp[j] for j < 16, entries past

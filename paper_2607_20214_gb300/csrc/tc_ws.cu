@@ -543,12 +543,12 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             float sp[32];
             auto features = [&] {
                 constexpr int n1 = T * G <= 16 ? 16 : 32;
-                race_factors<n1>(pr, nt0 * G, beta, sp);
+                race_factors<n1>(pr, beta, sp);
                 float dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // independent chains
                 chunk_den<G, T>(sp, nt0, Asm + ta0 * R, dacc);
                 if constexpr (T * G <= 16) {
                     if (nt1 > 0) {
-                        race_factors<16>(pr + 16, nt1 * G, beta, sp + 16);
+                        race_factors<16>(pr + 16, beta, sp + 16);
                         chunk_den<G, T>(sp + 16, nt1, Asm + ta1 * R, dacc);
                     }
                 }
