@@ -41,6 +41,7 @@ __global__ void __launch_bounds__(kRaceThreads)
     float *vt = kt + kRaceTok * ds;    // [kRaceTok][d]
     float *ph = vt + kRaceTok * d;     // [kRaceTok][64]
     float *wr = ph + kRaceTok * 64;    // [tables in slice][gamma][d]
+    float *fac = wr + (t1 - t0) * gamma * d;  // [kRaceTok][planes][2] factors
     __shared__ float wt[kRaceTok];     // A weights of the staged tokens
 
     for (int i = tid; i < (t1 - t0) * gamma * d; i += kRaceThreads)
@@ -73,28 +74,30 @@ __global__ void __launch_bounds__(kRaceThreads)
             wt[tid] = n < c1 ? (wA ? wA[(size_t)bh * N + n] : 1.f) : 0.f;
         }
         __syncthreads();
-        // features: one task per (token, table)
-        for (int task = tid; task < kRaceTok * (t1 - t0); task += kRaceThreads) {
-            int tok = task % kRaceTok, tl = task / kRaceTok;
-            float *out = ph + tok * 64 + tl * R;
-            if (base + tok >= c1) {
-                for (int rr = 0; rr < R; ++rr) out[rr] = 0.f;
-                continue;
-            }
-            float sp[8], sn[8];
+        // bit factors, one task per (token, plane), then features, one per
+        // (token, bucket)
+        const int np = (t1 - t0) * gamma;
+        for (int task = tid; task < kRaceTok * np; task += kRaceThreads) {
+            const int tok = task % kRaceTok, pl = task / kRaceTok;
             const float *xr = kt + tok * ds;
-            for (int bb = 0; bb < gamma; ++bb) {
-                const float *w = wr + (tl * gamma + bb) * d;
-                float a = 0.f;
-                for (int i = 0; i < d; ++i) a = fmaf(w[i], xr[i], a);
-                race_bit_factors(a, beta, sp[bb], sn[bb]);
-            }
-            for (int rr = 0; rr < R; ++rr) {
-                float pr = 1.f;
-                for (int bb = 0; bb < gamma; ++bb)
-                    pr *= ((rr >> bb) & 1) ? sp[bb] : sn[bb];
-                out[rr] = pr;
-            }
+            const float *w = wr + pl * d;
+            float a = 0.f;
+#pragma unroll 16
+            for (int i = 0; i < d; ++i) a = fmaf(w[i], xr[i], a);
+            float sp, sn;
+            race_bit_factors(a, beta, sp, sn);
+            fac[(tok * np + pl) * 2] = sn;
+            fac[(tok * np + pl) * 2 + 1] = sp;
+        }
+        __syncthreads();
+        for (int task = tid; task < kRaceTok * nb; task += kRaceThreads) {
+            const int tok = task / nb, rb = task - tok * nb;
+            const int tl = rb / R, rr = rb - tl * R;
+            const float *f = fac + (tok * np + tl * gamma) * 2;
+            float pr = base + tok < c1 ? 1.f : 0.f;
+            for (int bb = 0; bb < gamma; ++bb)
+                pr *= f[2 * bb + ((rr >> bb) & 1)];
+            ph[tok * 64 + rb] = pr;
         }
         __syncthreads();
         for (int tok = 0; tok < kRaceTok; ++tok) {
@@ -148,10 +151,9 @@ __global__ void k_race_reduce(const float *__restrict__ part, int S, int r,
 // phi(Q_i) and Num/Den from the summaries (Algorithm RACE, steps 9-10);
 // Eq. (5)-(6) fusion; row written at the query's original index (un-permute).
 constexpr int kBlkThreads = 256;
-constexpr int kQPerWarp = kSimtQT / (kBlkThreads / 32);  // 4
 constexpr int kKC = 32;  // keys per staged chunk
 
-template <typename T>
+template <typename T, int QT>
 __global__ void __launch_bounds__(kBlkThreads)
     k_block_attn(const T *__restrict__ qx, const T *__restrict__ kx,
                  const T *__restrict__ vx, const float *__restrict__ w_race,
@@ -167,18 +169,19 @@ __global__ void __launch_bounds__(kBlkThreads)
                  float scale, float lambda, int mode, DeviceStatus *status,
                  const int32_t *__restrict__ cand,
                  const uint32_t *__restrict__ selmask, int tk_c) {
+    constexpr int kQPerWarp = QT / (kBlkThreads / 32);
     extern __shared__ float smem[];
     const int bh = blockIdx.y, h = bh % H;
-    const int pos0 = blockIdx.x * kSimtQT;
+    const int pos0 = blockIdx.x * QT;
     const int blk = pos0 / b;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int R = 1 << gamma, r = L * R;
     const int ds = d + 1;
-    float *qs = smem;                 // [32][d]
-    float *ks = qs + kSimtQT * d;     // [32][d + 1]
+    float *qs = smem;                 // [QT][d + 1]
+    float *ks = qs + QT * ds;         // [32][d + 1]
     float *vs = ks + kKC * ds;        // [32][d]
-    __shared__ int qidx[kSimtQT];
-    __shared__ float s_logds[kSimtQT], s_den[kSimtQT], s_m[kSimtQT];
+    __shared__ int qidx[QT];
+    __shared__ float s_logds[QT], s_den[QT], s_m[QT];
 
     const T *qh = qx + (size_t)bh * N * d;
     const T *kh = kx + (size_t)bh * N * d;
@@ -186,7 +189,7 @@ __global__ void __launch_bounds__(kBlkThreads)
     const int32_t *pq = perm_q + (size_t)bh * N;
     const int32_t *pk = perm_k + (size_t)bh * N;
 
-    if (tid < kSimtQT) {
+    if (tid < QT) {
         int i = pq[pos0 + tid];
         if (i < 0 || i >= N) {
             report(status, kDevPermRange, 1, bh, i);
@@ -195,9 +198,9 @@ __global__ void __launch_bounds__(kBlkThreads)
         qidx[tid] = i;
     }
     __syncthreads();
-    for (int i = tid; i < kSimtQT * d; i += kBlkThreads) {
+    for (int i = tid; i < QT * d; i += kBlkThreads) {
         int row = i / d, col = i - row * d;
-        qs[i] = to_f32<T>(qh[(size_t)qidx[row] * d + col]);
+        qs[row * ds + col] = to_f32<T>(qh[(size_t)qidx[row] * d + col]);
     }
 
     // ---- sparse branch: online softmax over the key block
@@ -248,9 +251,10 @@ __global__ void __launch_bounds__(kBlkThreads)
         __syncthreads();
 #pragma unroll
         for (int qq = 0; qq < kQPerWarp; ++qq) {
-            const float *qr = qs + (wid * kQPerWarp + qq) * d;
+            const float *qr = qs + (wid * kQPerWarp + qq) * ds;
             const float *kr = ks + lane * ds;
             float z = 0.f;
+#pragma unroll 16
             for (int e = 0; e < d; ++e) z = fmaf(qr[e], kr[e], z);
             z *= scale;
             bool keep = true;
@@ -265,6 +269,7 @@ __global__ void __launch_bounds__(kBlkThreads)
             l_run[qq] = l_run[qq] * alpha + warp_sum(p);
 #pragma unroll
             for (int c = 0; c < 4; ++c) o_acc[qq][c] *= alpha;
+#pragma unroll 8
             for (int j = 0; j < kKC; ++j) {
                 float pj = __shfl_sync(0xffffffffu, p, j);
 #pragma unroll
@@ -290,58 +295,81 @@ __global__ void __launch_bounds__(kBlkThreads)
     }
 
     // ---- RACE readout for the 32 queries, slice by slice of tables
-    float *phq = vs;                   // [32][64] features of the slice
-    float *wr = phq + kSimtQT * 64;    // [tps][gamma][d]
+    // Rows of queries and features are padded by one word: their threads
+    // read them a row per lane.
+    constexpr int kPh = 65;
+    float *phq = vs;                 // [QT][65] features of the slice
+    float *fac = phq + QT * kPh;     // [QT][tps gamma][2] bit factors
+    float *wr = fac + QT * 2 * tps * gamma;  // [tps][gamma][d]
     const int ngrp = kBlkThreads / d;
     const int e = tid % d, grp = tid / d;
-    const int nq = kSimtQT / ngrp;     // queries per thread (<= 32)
-    float num[32];
+    const int nq = QT / ngrp;        // queries per thread (<= QT)
+    float num[QT];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) num[j] = 0.f;
-    float den = 0.f;
+    for (int j = 0; j < QT; ++j) num[j] = 0.f;
+    float den[kQPerWarp];
+#pragma unroll
+    for (int qq = 0; qq < kQPerWarp; ++qq) den[qq] = 0.f;
     const float *Ah = Ag + (size_t)bh * r;
     const float *Bh = Bg + (size_t)bh * r * d;
     for (int t0 = 0; t0 < L; t0 += tps) {
         const int t1 = min(L, t0 + tps);
-        const int nb = (t1 - t0) * R;
+        const int nb = (t1 - t0) * R, np = (t1 - t0) * gamma;
         __syncthreads();
-        for (int i = tid; i < (t1 - t0) * gamma * d; i += kBlkThreads)
+        for (int i = tid; i < np * d; i += kBlkThreads)
             wr[i] = w_race[((size_t)h * L + t0) * gamma * d + i];
         __syncthreads();
-        for (int task = tid; task < kSimtQT * (t1 - t0); task += kBlkThreads) {
-            int qrow = task % kSimtQT, tl = task / kSimtQT;
-            const float *xr = qs + qrow * d;
-            float sp[8], sn[8];
-            for (int bb = 0; bb < gamma; ++bb) {
-                const float *w = wr + (tl * gamma + bb) * d;
-                float a = 0.f;
-                for (int i = 0; i < d; ++i) a = fmaf(w[i], xr[i], a);
-                race_bit_factors(a, beta, sp[bb], sn[bb]);
-            }
-            for (int rr = 0; rr < R; ++rr) {
-                float pr = 1.f;
-                for (int bb = 0; bb < gamma; ++bb)
-                    pr *= ((rr >> bb) & 1) ? sp[bb] : sn[bb];
-                phq[qrow * 64 + tl * R + rr] = pr;
-            }
+        for (int task = tid; task < QT * np; task += kBlkThreads) {
+            const int qrow = task % QT, pl = task / QT;
+            const float *xr = qs + qrow * ds;
+            const float *w = wr + pl * d;
+            float a = 0.f;
+#pragma unroll 16
+            for (int i = 0; i < d; ++i) a = fmaf(w[i], xr[i], a);
+            float sp, sn;
+            race_bit_factors(a, beta, sp, sn);
+            float *f = fac + (qrow * np + pl) * 2;
+            f[0] = sn;
+            f[1] = sp;
         }
         __syncthreads();
+        for (int task = tid; task < QT * nb; task += kBlkThreads) {
+            const int qrow = task / nb, rb = task - qrow * nb;
+            const int tl = rb / R, rr = rb - tl * R;
+            const float *f = fac + (qrow * np + tl * gamma) * 2;
+            float pr = 1.f;
+            for (int bb = 0; bb < gamma; ++bb)
+                pr *= f[2 * bb + ((rr >> bb) & 1)];
+            phq[qrow * kPh + rb] = pr;
+        }
+        __syncthreads();
+#pragma unroll 8
         for (int rb = 0; rb < nb; ++rb) {
             float bv = Bh[(size_t)(t0 * R + rb) * d + e];
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-                if (j < nq) num[j] = fmaf(phq[(grp + j * ngrp) * 64 + rb], bv,
+            for (int j = 0; j < QT; ++j)
+                if (j < nq) num[j] = fmaf(phq[(grp + j * ngrp) * kPh + rb], bv,
                                          num[j]);
         }
-        if (tid < kSimtQT)
-            for (int rb = 0; rb < nb; ++rb)
-                den = fmaf(phq[tid * 64 + rb], Ah[t0 * R + rb], den);
+        for (int rb = lane; rb < nb; rb += 32) {
+            const float av = Ah[t0 * R + rb];
+#pragma unroll
+            for (int qq = 0; qq < kQPerWarp; ++qq)
+                den[qq] = fmaf(phq[(wid * kQPerWarp + qq) * kPh + rb], av,
+                               den[qq]);
+        }
     }
+#pragma unroll
+    for (int qq = 0; qq < kQPerWarp; ++qq) {
+        const float v = warp_sum(den[qq]);
+        if (lane == 0) s_den[wid * kQPerWarp + qq] = v;
+    }
+    __syncthreads();
     const float invL = 1.0f / (float)L;
-    if (tid < kSimtQT) {
+    if (tid < QT) {
         const int i = qidx[tid];
         const size_t tok = (size_t)bh * N + i;
-        float dl = den * invL;
+        float dl = s_den[tid] * invL;
         float lam = lambda_tok ? lambda_tok[tok] : lambda;
         float mm = fusion_multiplier(s_logds[tid], lam, dl, eps, mode);
         s_den[tid] = dl;
@@ -352,7 +380,7 @@ __global__ void __launch_bounds__(kBlkThreads)
     }
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
+    for (int j = 0; j < QT; ++j) {
         if (j >= nq) break;
         const int row = grp + j * ngrp;
         const int i = qidx[row];
@@ -377,7 +405,8 @@ cudaError_t launch_race_partial_simt(const Plan &P, const void *k,
     size_t smem = sizeof(float) *
                   ((size_t)kRaceTok * (P.d + 1) + (size_t)kRaceTok * P.d +
                    (size_t)kRaceTok * 64 +
-                   (size_t)P.tables_per_slice * P.gamma * P.d);
+                   (size_t)P.tables_per_slice * P.gamma *
+                       (P.d + 2 * kRaceTok));
     if (P.dtype == ELSAA_FP32) {
         auto kern = k_race_partial<float, float>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -405,7 +434,8 @@ cudaError_t launch_race_partial_weighted(const Plan &P, const void *x,
     size_t smem = sizeof(float) *
                   ((size_t)kRaceTok * (P.d + 1) + (size_t)kRaceTok * P.d +
                    (size_t)kRaceTok * 64 +
-                   (size_t)P.tables_per_slice * P.gamma * P.d);
+                   (size_t)P.tables_per_slice * P.gamma *
+                       (P.d + 2 * kRaceTok));
     if (P.dtype == ELSAA_FP32) {
         auto kern = k_race_partial<float, float>;
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -436,6 +466,7 @@ __global__ void k_race_reduce4(const float *__restrict__ part, int S, int r,
          i < per; i += 4 * (size_t)gridDim.x * blockDim.x) {
         const float *p = part + (size_t)bh * S * per + i;
         float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 8
         for (int c = 0; c < S; ++c) {
             const float4 x =
                 *reinterpret_cast<const float4 *>(p + (size_t)c * per);
@@ -484,18 +515,23 @@ cudaError_t launch_block_attn_simt(
     const float *gates, void *o, float *log_d_sparse, float *d_lr,
     float *m_sparse, DeviceStatus *status, cudaStream_t st,
     const int32_t *cand, const uint32_t *selmask) {
-    dim3 grid(P.N / kSimtQT, P.BH);
-    // phase 1: qs + ks(padded) + vs; phase 2 reuses ks, vs for outputs,
-    // features and planes.
-    size_t ph1 = (size_t)kSimtQT * P.d + (size_t)kKC * (P.d + 1) +
-                 (size_t)kKC * P.d;
-    size_t ph2 = (size_t)kSimtQT * P.d + (size_t)kKC * (P.d + 1) +
-                 (size_t)kSimtQT * 64 +
-                 (size_t)P.tables_per_slice * P.gamma * P.d;
+    // 32 queries per CTA, or 8 when that leaves most of the chip idle: c1
+    // (one head of 1024 rows) runs 128 CTAs instead of 32. With the padded
+    // rows (the features had read the queries through one bank) it takes
+    // 18 us instead of 78.
+    const int qt = (long)(P.N / kSimtQT) * P.BH < 152 ? 8 : kSimtQT;
+    dim3 grid(P.N / qt, P.BH);
+    // phase 1: qs + ks (both padded) + vs; phase 2 reuses ks, vs for outputs,
+    // features, bit factors and planes.
+    const size_t qk = (size_t)qt * (P.d + 1) + (size_t)kKC * (P.d + 1);
+    const size_t ph1 = qk + (size_t)kKC * P.d;
+    const size_t ph2 = qk + (size_t)qt * 65 +
+                       (size_t)qt * 2 * P.tables_per_slice * P.gamma +
+                       (size_t)P.tables_per_slice * P.gamma * P.d;
     size_t smem = sizeof(float) * (ph1 > ph2 ? ph1 : ph2);
 #define ELSAA_LAUNCH_BLK(T)                                                   \
     do {                                                                      \
-        auto kern = k_block_attn<T>;                                          \
+        auto kern = qt == 8 ? k_block_attn<T, 8> : k_block_attn<T, kSimtQT>;  \
         cudaFuncSetAttribute(kern,                                            \
                              cudaFuncAttributeMaxDynamicSharedMemorySize,     \
                              (int)smem);                                      \
