@@ -470,11 +470,12 @@ int causal_forward(const elsaa_params *params, const void *q, const void *k,
     uint16_t *Wbf = (uint16_t *)(ws + C.off_W);
     int *ctr = (int *)(ws + C.off_ctr);
 
-    ELSAA_CHECK_LAUNCH(cudaMemsetAsync(status, 0, sizeof(DeviceStatus), st),
-                       "status reset");
-    ELSAA_CHECK_LAUNCH(
-        cudaMemsetAsync(ctr, 0, (size_t)(C.Lv + 1) * sizeof(int), st),
-        "counter reset");
+    // status and work counters cleared, bf16 planes
+    ELSAA_CHECK_LAUNCH(timed("prep_planes", st, [&] {
+                           return launch_begin(P, w_race, Wbf, status, ctr,
+                                               C.Lv + 1, st);
+                       }),
+                       "prep_planes");
     // sparse branch: codes, sorted halves, base segments, then the levels
     ELSAA_CHECK_LAUNCH(timed("sort_hash", st, [&] {
                            return launch_sort_hash(P, q, k, w_sort, keyrank,
@@ -501,10 +502,6 @@ int causal_forward(const elsaa_params *params, const void *q, const void *k,
     cudaStream_t ks = side->s;
     ELSAA_CHECK_LAUNCH(cudaEventRecord(side->fork, st), "fork");
     ELSAA_CHECK_LAUNCH(cudaStreamWaitEvent(ks, side->fork, 0), "fork wait");
-    ELSAA_CHECK_LAUNCH(timed("prep_planes", ks, [&] {
-                           return launch_prep_planes(P, w_race, Wbf, ks);
-                       }),
-                       "prep_planes");
     ELSAA_CHECK_LAUNCH(timed("race_keys_ws", ks, [&] {
                            return launch_race_keys_ws(C.Pc, k, v, Wbf, part,
                                                       status, ks);
@@ -615,20 +612,40 @@ int forward_impl(const elsaa_params *params, const void *q, const void *k,
     uint16_t *Bh = (uint16_t *)(ws + P.off_Bh);
     uint16_t *Wbf = (uint16_t *)(ws + P.off_W);
 
-    ELSAA_CHECK_LAUNCH(cudaMemsetAsync(status, 0, sizeof(DeviceStatus), st),
-                       "status reset");
-    // RACE key side (no sort needed) on the side stream, launched first so
-    // that its CTAs are placed before the hash kernel's
+    // The RACE key side needs no sort: it runs on the side stream. Short
+    // calls are bound by their launches: the status reset and the bf16
+    // planes share one before the fork, and the scatter scans (44 -> 40 us
+    // for 12 heads of 1024 rows). In long ones the planes go with the side
+    // stream, enqueued first: made before the fork, with the hash enqueued
+    // first, they cost 6 us at c3 and at c2.
+    const bool brief = short_call(P);
+    const bool tcp = P.impl == 2;
+    auto planes = [&](cudaStream_t s) {
+        return timed("prep_planes", s, [&] {
+            return launch_begin(P, w_race, Wbf, brief ? status : nullptr,
+                                nullptr, 0, s);
+        });
+    };
+    auto hash = [&] {
+        return timed("sort_hash", st, [&] {
+            return launch_sort_hash(P, q, k, w_sort, keyrank, hist, status,
+                                    st);
+        });
+    };
+    if (brief && tcp)
+        ELSAA_CHECK_LAUNCH(planes(st), "prep_planes");
+    else
+        ELSAA_CHECK_LAUNCH(
+            cudaMemsetAsync(status, 0, sizeof(DeviceStatus), st),
+            "status reset");
     SideStream *side = nullptr;
     ELSAA_CHECK_LAUNCH(side_stream(&side), "side stream");
     cudaStream_t ks = side->s;
     ELSAA_CHECK_LAUNCH(cudaEventRecord(side->fork, st), "fork");
+    if (brief) ELSAA_CHECK_LAUNCH(hash(), "sort_hash");
     ELSAA_CHECK_LAUNCH(cudaStreamWaitEvent(ks, side->fork, 0), "fork wait");
-    if (P.impl == 2) {
-        ELSAA_CHECK_LAUNCH(timed("prep_planes", ks, [&] {
-                               return launch_prep_planes(P, w_race, Wbf, ks);
-                           }),
-                           "prep_planes");
+    if (tcp) {
+        if (!brief) ELSAA_CHECK_LAUNCH(planes(ks), "prep_planes");
         ELSAA_CHECK_LAUNCH(timed("race_keys_ws", ks, [&] {
                                return launch_race_keys_ws(P, k, v, Wbf, part,
                                                           status, ks);
@@ -646,14 +663,12 @@ int forward_impl(const elsaa_params *params, const void *q, const void *k,
                        }),
                        "race_reduce");
     ELSAA_CHECK_LAUNCH(cudaEventRecord(side->join, ks), "join");
-    ELSAA_CHECK_LAUNCH(timed("sort_hash", st, [&] {
-                           return launch_sort_hash(P, q, k, w_sort, keyrank,
-                                                   hist, status, st);
-                       }),
-                       "sort_hash");
-    ELSAA_CHECK_LAUNCH(timed("sort_scan", st,
-                             [&] { return launch_sort_scan(P, hist, st); }),
-                       "sort_scan");
+    if (!brief) ELSAA_CHECK_LAUNCH(hash(), "sort_hash");
+    if (!sort_fused(P))
+        ELSAA_CHECK_LAUNCH(timed("sort_scan", st, [&] {
+                               return launch_sort_scan(P, hist, st);
+                           }),
+                           "sort_scan");
     ELSAA_CHECK_LAUNCH(timed("sort_scatter", st, [&] {
                            return launch_sort_scatter(P, keyrank, hist, pq,
                                                       pk, status, st);
@@ -851,15 +866,11 @@ extern "C" int elsaa_forward_race_summaries(const elsaa_params *params,
     cudaStream_t st = (cudaStream_t)stream;
     const char *ws = (const char *)workspace;
     ELSAA_CHECK_LAUNCH(
-        cudaMemcpyAsync(race_A, ws + P.off_A,
-                        (size_t)P.BH * P.r * sizeof(float),
-                        cudaMemcpyDeviceToDevice, st),
-        "copy of A");
-    ELSAA_CHECK_LAUNCH(
-        cudaMemcpyAsync(race_B, ws + P.off_B,
-                        (size_t)P.BH * P.r * P.d * sizeof(float),
-                        cudaMemcpyDeviceToDevice, st),
-        "copy of B");
+        launch_copy_summaries((const float *)(ws + P.off_A),
+                              (const float *)(ws + P.off_B),
+                              (size_t)P.BH * P.r, (size_t)P.BH * P.r * P.d,
+                              race_A, race_B, st),
+        "copy of A and B");
     return ELSAA_OK;
 }
 

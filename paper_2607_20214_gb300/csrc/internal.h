@@ -72,6 +72,10 @@ cudaError_t launch_sort_hash(const Plan &P, const void *q, const void *k,
                              const float *w_sort, uint32_t *keyrank,
                              int *hist, DeviceStatus *status,
                              cudaStream_t st);
+bool short_call(const Plan &P);
+// sort_fused: the scatter launch scans as well and launch_sort_scan does
+// nothing.
+bool sort_fused(const Plan &P);
 cudaError_t launch_sort_scan(const Plan &P, int *hist, cudaStream_t st);
 cudaError_t launch_sort_scatter(const Plan &P, const uint32_t *keyrank,
                                 const int *hist, int32_t *perm_q,
@@ -88,6 +92,10 @@ cudaError_t launch_race_partial_weighted(const Plan &P, const void *x,
                                          cudaStream_t st);
 cudaError_t launch_race_reduce(const Plan &P, const float *part, float *A,
                                float *Bm, uint16_t *Bh, cudaStream_t st);
+// Copies A (na values) and B (nb values) out of the workspace.
+cudaError_t launch_copy_summaries(const float *a, const float *b, size_t na,
+                                  size_t nb, float *oa, float *ob,
+                                  cudaStream_t st);
 cudaError_t launch_block_attn_simt(
     const Plan &P, const void *q, const void *k, const void *v,
     const float *w_race, const int32_t *perm_q, const int32_t *perm_k,
@@ -239,6 +247,11 @@ cudaError_t make_tma_map_bf16_narrow(CUtensorMap *map, const void *base,
 // operand image the tensor-core kernels load with TMA.
 cudaError_t launch_prep_planes(const Plan &P, const float *w_race,
                                uint16_t *w_bf16, cudaStream_t st);
+// The same, and the status word and `n_zero` ints at `zero` cleared: the
+// first launch of a call.
+cudaError_t launch_begin(const Plan &P, const float *w_race, uint16_t *w_bf16,
+                         DeviceStatus *status, int *zero, int n_zero,
+                         cudaStream_t st);
 
 // Warp-specialised RACE key summaries (tensor-core path).
 size_t race_keys_ws_smem(const Plan &P);

@@ -473,6 +473,56 @@ __global__ void __launch_bounds__(kHashTile)
     perm[pos] = n;
 }
 
+// Scan and scatter in one launch, for heads of few tiles: every CTA scans the
+// whole [bins][tiles] histogram of its head (at most kFusedScan entries, in
+// shared memory) and places its own tile.
+constexpr int kFusedScan = 2048;
+__global__ void __launch_bounds__(kHashTile)
+    k_sort_scan_scatter(const uint32_t *__restrict__ keyrank,
+                        const int *__restrict__ hist, int N, int tiles,
+                        int bins, int32_t *__restrict__ perm_q,
+                        int32_t *__restrict__ perm_k, DeviceStatus *status) {
+    __shared__ int off[kFusedScan];
+    __shared__ int warp_tot[kHashTile / 32];
+    const int tile = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
+    const int BH = gridDim.y, tid = threadIdx.x, lane = tid & 31;
+    const int E = tiles * bins;
+    const int n = tile * kHashTile + tid;
+    const size_t row = (size_t)which * BH + bh;
+    const uint32_t kr = n < N ? keyrank[row * N + n] : 0u;
+    const int *h = hist + row * E;
+    for (int e = tid; e < E; e += kHashTile) off[e] = h[e];
+    __syncthreads();
+    const int per = (E + kHashTile - 1) / kHashTile;
+    const int e0 = min(E, tid * per), e1 = min(E, e0 + per);
+    int sum = 0;
+    for (int e = e0; e < e1; ++e) sum += off[e];
+    int incl = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) warp_tot[tid >> 5] = incl;
+    __syncthreads();
+    int run = incl - sum;
+    for (int w = 0; w < tid >> 5; ++w) run += warp_tot[w];
+    for (int e = e0; e < e1; ++e) {
+        const int v = off[e];
+        off[e] = run;
+        run += v;
+    }
+    __syncthreads();
+    if (n >= N) return;
+    const int pos = off[(kr & 0xffffu) * tiles + tile] + (int)(kr >> 16);
+    if (pos < 0 || pos >= N) {
+        report(status, kDevSortRange, 0, bh, pos);
+        return;
+    }
+    int32_t *perm = (which ? perm_k : perm_q) + (size_t)bh * N;
+    perm[pos] = n;
+}
+
 template <typename T, int NS>
 cudaError_t launch_hash_t(const Plan &P, const void *q, const void *k,
                           const float *w_sort, uint32_t *keyrank, int *hist,
@@ -567,7 +617,17 @@ cudaError_t launch_sort_hash(const Plan &P, const void *q, const void *k,
                                             st);
 }
 
+// Calls of so few rows that their launches decide.
+bool short_call(const Plan &P) { return (long)P.BH * P.N <= 32768; }
+
+// With many tiles the repeated scans cost more than the launch they save (c2:
+// 1536 tiles, 4 us).
+bool sort_fused(const Plan &P) {
+    return short_call(P) && P.tiles * P.bins <= kFusedScan;
+}
+
 cudaError_t launch_sort_scan(const Plan &P, int *hist, cudaStream_t st) {
+    if (sort_fused(P)) return cudaSuccess;
     k_sort_scan<<<2 * P.BH, kScanThreads, 0, st>>>(hist, P.tiles, P.bins);
     return cudaGetLastError();
 }
@@ -577,6 +637,11 @@ cudaError_t launch_sort_scatter(const Plan &P, const uint32_t *keyrank,
                                 int32_t *perm_k, DeviceStatus *status,
                                 cudaStream_t st) {
     dim3 grid(P.tiles, P.BH, 2);
+    if (sort_fused(P)) {
+        k_sort_scan_scatter<<<grid, kHashTile, 0, st>>>(
+            keyrank, hist, P.N, P.tiles, P.bins, perm_q, perm_k, status);
+        return cudaGetLastError();
+    }
     k_sort_scatter<<<grid, kHashTile, 0, st>>>(keyrank, hist, P.N, P.tiles,
                                                P.bins, perm_q, perm_k, status);
     return cudaGetLastError();

@@ -228,6 +228,20 @@ def _ptr(t, name, dtype=None, numel=None, device=None):
     return t.data_ptr()
 
 
+# torch.cuda.current_stream builds a Stream object (2 us, as much as a kernel
+# launch); the raw handle is all that is needed
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream_of(stream, dev):
+    """cudaStream_t of `stream`, by default torch's current one on dev."""
+    if stream is None:
+        if _raw_stream is not None and dev.index is not None:
+            return _raw_stream(dev.index)
+        stream = torch.cuda.current_stream(dev)
+    return getattr(stream, "cuda_stream", stream)
+
+
 def new_workspace(params: elsaa_params, device) -> torch.Tensor:
     """Caller-owned scratch of elsaa_workspace_size bytes (256-aligned)."""
     n = elsaa_workspace_size(params)
@@ -255,9 +269,7 @@ def elsaa_forward(params: elsaa_params, q, k, v, w_sort, w_race,
         o = torch.empty(q.shape, dtype=odt, device=dev)
     if workspace is None:
         workspace = new_workspace(params, dev)
-    if stream is None:
-        stream = torch.cuda.current_stream(dev)
-    sp = stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
+    sp = _stream_of(stream, dev)
     args = [
         _ptr(q, "q", tdt, nqkv, dev), _ptr(k, "k", tdt, nqkv, dev),
         _ptr(v, "v", tdt, nqkv, dev),
@@ -305,9 +317,7 @@ def elsaa_forward_race_summaries(params: elsaa_params, workspace,
     if race_B is None:
         race_B = torch.empty((params.B, params.H, r, params.d_h),
                              dtype=torch.float32, device=dev)
-    if stream is None:
-        stream = torch.cuda.current_stream(dev)
-    sp = stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
+    sp = _stream_of(stream, dev)
     rc = lib.elsaa_forward_race_summaries(
         ctypes.byref(params), _ptr(workspace, "workspace", None, None, dev),
         workspace.numel() * workspace.element_size(),
@@ -340,9 +350,7 @@ def elsaa_backward(params: elsaa_params, q, k, v, w_sort, w_race, d_o,
     if workspace is None:
         n = elsaa_backward_workspace_size(params)
         workspace = torch.empty(max(n, 256), dtype=torch.uint8, device=dev)
-    if stream is None:
-        stream = torch.cuda.current_stream(dev)
-    sp = stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
+    sp = _stream_of(stream, dev)
     args = [
         _ptr(q, "q", tdt, nqkv, dev), _ptr(k, "k", tdt, nqkv, dev),
         _ptr(v, "v", tdt, nqkv, dev),
@@ -419,9 +427,7 @@ def elsaa_gates(params: elsaa_params, mlp: dict, q, gates=None,
     if workspace is None:
         n = elsaa_gates_workspace_size(params, mlp, dev)
         workspace = torch.empty(max(n, 256), dtype=torch.uint8, device=dev)
-    if stream is None:
-        stream = torch.cuda.current_stream(dev)
-    sp = stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
+    sp = _stream_of(stream, dev)
     rc = lib.elsaa_gates(
         ctypes.byref(params), ctypes.byref(m),
         _ptr(q, "q", tdt, BHN * params.d_h, dev),
@@ -491,9 +497,7 @@ def elsaa_forward_noalloc(params: elsaa_params, q, k, v, w_sort, w_race,
     odt = torch.float32 if params.out_fp32 else tdt
     BHN = params.B * params.H * params.N
     nqkv = BHN * params.d_h
-    if stream is None:
-        stream = torch.cuda.current_stream(dev)
-    sp = stream.cuda_stream if hasattr(stream, "cuda_stream") else stream
+    sp = _stream_of(stream, dev)
     args = [
         _ptr(q, "q", tdt, nqkv, dev), _ptr(k, "k", tdt, nqkv, dev),
         _ptr(v, "v", tdt, nqkv, dev),
