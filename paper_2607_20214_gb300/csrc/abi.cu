@@ -488,9 +488,8 @@ int causal_forward(const elsaa_params *params, const void *q, const void *k,
                        }),
                        "seg_sort");
     ELSAA_CHECK_LAUNCH(timed("causal_attn_base", st, [&] {
-                           return launch_causal_attn(P, 0, C.n_leaf, 0, q, k,
-                                                     v, perms, ctr, RO, RL,
-                                                     status, st);
+                           return launch_causal_base(P, C.n_leaf, q, k, v, ctr,
+                                                     RO, RL, status, st);
                        }),
                        "causal_attn_base");
     // the low-rank branch (chunk summaries, prefix states) on the side
@@ -515,8 +514,7 @@ int causal_forward(const elsaa_params *params, const void *q, const void *k,
     ELSAA_CHECK_LAUNCH(cudaEventRecord(side->join, ks), "join");
     for (int level = C.Lv; level >= 1; --level)
         ELSAA_CHECK_LAUNCH(timed("causal_attn_merge", st, [&] {
-                               return launch_causal_attn(P, 1, C.n_leaf,
-                                                         level, q, k, v,
+                               return launch_causal_attn(P, level, q, k, v,
                                                          perms, ctr + level,
                                                          RO, RL, status, st);
                            }),

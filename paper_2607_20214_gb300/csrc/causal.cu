@@ -11,7 +11,10 @@
 // a future half. So:
 //   k_seg_sort       stable counting sort of each node's future-half query
 //                    codes and past-half key codes (codes from the sort hash)
-//   k_causal_attn_tc base segments (exact causal attention, 128-row tiles
+//   k_causal_base    (causal_base.cu) exact causal attention of the base
+//                    segments
+//   k_causal_attn_tc the SortLSH blocks of each level, deepest first, merged
+//                    into the running result (MergeLSE)
 //                    over 128-key tiles with an online softmax), then one
 //                    launch per level, deepest first, for the SortLSH blocks,
 //                    merged into the running (O, log d) with MergeLSE
@@ -130,15 +133,11 @@ __device__ __forceinline__ void f2unpack(unsigned long long d, float &lo,
 
 // ------------------------------------------------------- attention tiles
 
-// One CTA = one tile of 128 query rows and its key tiles, online softmax:
-//   mode 0 (base segments): rows leaf n_leaf + 128 qt + [0, 128), key tiles
-//          kt = 0..qt of the same segment, the last one masked j <= i;
-//          writes (O, log d) of exact causal attention.
-//   mode 1 (SortLSH of one level): rows = sorted future-half queries
-//          128 qt.. of node j, keys = the node's sorted past-half keys of
-//          the same block (b >= 128: b / 128 key tiles; b < 128: one tile,
-//          rows and keys paired by block, r / b == c / b); MergeLSE into
-//          the running (O, log d).
+// SortLSH of one level: one CTA = one tile of 128 sorted future-half queries
+// 128 qt.. of node j, keys = the node's sorted past-half keys of the same
+// block (b >= 128: b / 128 key tiles, online softmax; b < 128: one tile, rows
+// and keys paired by block, r / b == c / b); MergeLSE into the running
+// (O, log d) that the base segments (causal_base.cu) and deeper levels left.
 // Per key tile: MMA S = Q K^T (TMEM [0, 128)); the next K tile's copies
 // start at once (K is consumed); CUDA scale, mask, running max and
 // P = exp(S - max), packed as bf16 pairs into TMEM over the scores already
@@ -149,14 +148,13 @@ __device__ __forceinline__ void f2unpack(unsigned long long d, float &lo,
 // cp.async groups are committed in a fixed order (Q and K0, V0, then per
 // tile: next K, next V; empty groups past the last tile), so "all but the
 // newest group done" always means the operand about to be used has landed.
-template <int D, int MODE>
+template <int D>
 __global__ void __launch_bounds__(kCaThreads, 2)
     k_causal_attn_tc(const uint16_t *__restrict__ qx,
                      const uint16_t *__restrict__ kx,
                      const uint16_t *__restrict__ vx,
                      const int32_t *__restrict__ permq,
-                     const int32_t *__restrict__ permk, int N, int n_leaf,
-                     int m, int b, int items, int *__restrict__ next_item,
+                     const int32_t *__restrict__ permk, int N, int m, int b, int items, int *__restrict__ next_item,
                      float scale, float eps, float *__restrict__ RO,
                      float *__restrict__ RL, DeviceStatus *status) {
     extern __shared__ unsigned char smem_raw[];
@@ -165,7 +163,7 @@ __global__ void __launch_bounds__(kCaThreads, 2)
     __shared__ int abort_flag;
     __shared__ float xm[2][128], xl[2][128];
     __shared__ int qrow_s[128];
-    __shared__ int krow_s[2][128];  // MODE 1: key rows of the next tiles
+    __shared__ int krow_s[2][128];  // key rows of the next tiles
     __shared__ int item_s;
     volatile int *abort = &abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane_id = tid & 31;
@@ -210,42 +208,24 @@ __global__ void __launch_bounds__(kCaThreads, 2)
         const int item = item_s;
         if (item >= items) break;
         // ---- work item
-        int bh, qt, nkt, kt0;
-        int seg0 = 0;  // MODE 0: first row of the segment (within the head)
-        const int32_t *ql = nullptr, *kl = nullptr;
-        if (MODE == 0) {
-            // item -> (row tile, segment, head), row tiles with the most key
-            // tiles first across all segments and heads
-            const int nq = n_leaf / 128, nleaves = N / n_leaf;
-            const int per = items / nq;  // segments x heads
-            qt = nq - 1 - item / per;
-            const int rest = item % per;
-            const int leaf = rest % nleaves;
-            bh = rest / nleaves;
-            seg0 = leaf * n_leaf;
-            kt0 = 0;
-            nkt = qt + 1;
+        int nkt, kt0;
+        const int tpn = m / 128, nodes = N / (2 * m);
+        const int qt = item % tpn, rest = item / tpn;
+        const int j = rest % nodes, bh = rest / nodes;
+        const int32_t *ql = permq + (size_t)bh * (N >> 1) + (size_t)j * m;
+        const int32_t *kl = permk + (size_t)bh * (N >> 1) + (size_t)j * m;
+        if (b >= 128) {
+            kt0 = (qt * 128 / b) * (b / 128);
+            nkt = b / 128;
         } else {
-            const int tpn = m / 128, nodes = N / (2 * m);
-            qt = item % tpn;
-            const int rest = item / tpn;
-            const int j = rest % nodes;
-            bh = rest / nodes;
-            ql = permq + (size_t)bh * (N >> 1) + (size_t)j * m;
-            kl = permk + (size_t)bh * (N >> 1) + (size_t)j * m;
-            if (b >= 128) {
-                kt0 = (qt * 128 / b) * (b / 128);
-                nkt = b / 128;
-            } else {
-                kt0 = qt;
-                nkt = 1;
-            }
+            kt0 = qt;
+            nkt = 1;
         }
         const size_t hN = (size_t)bh * N;
-        // key rows of tile kt (tokens within the head); MODE 1 reads them
-        // from the level's index list into krow_s[kt & 1] (then a barrier)
+        // key rows of tile kt (tokens within the head), from the level's
+        // index list into krow_s[kt & 1] (then a barrier)
         auto stage_rows = [&](int kt) {
-            if (MODE == 1 && tid < 128) {
+            if (tid < 128) {
                 int t = kl[kt * 128 + tid];
                 if (t < 0 || t >= N) {  // read as row 0 (checked: recorded)
 #ifdef ELSAA_CHECKED
@@ -259,8 +239,7 @@ __global__ void __launch_bounds__(kCaThreads, 2)
         auto load_tile = [&](uint32_t dst, const uint16_t *src, int kt) {
             for (int i = tid; i < 128 * (D / 8); i += kCaThreads) {
                 const int rr = i / (D / 8), c = i % (D / 8);
-                const int t =
-                    MODE == 0 ? seg0 + kt * 128 + rr : krow_s[kt & 1][rr];
+                const int t = krow_s[kt & 1][rr];
                 cp_async16(dst + panel_offset(rr, c, 128),
                            src + (hN + t) * D + c * 8);
             }
@@ -271,17 +250,12 @@ __global__ void __launch_bounds__(kCaThreads, 2)
             __syncthreads();
         };
         if (tid < 128) {
-            int t;
-            if (MODE == 0) {
-                t = seg0 + qt * 128 + tid;
-            } else {
-                t = ql[qt * 128 + tid];
-                if (t < 0 || t >= N) {  // read as row 0 (checked: recorded)
+            int t = ql[qt * 128 + tid];
+            if (t < 0 || t >= N) {  // read as row 0 (checked: recorded)
 #ifdef ELSAA_CHECKED
-                    report(status, kDevPermRange, 15, bh, t);
+                report(status, kDevPermRange, 15, bh, t);
 #endif
-                    t = 0;
-                }
+                t = 0;
             }
             qrow_s[tid] = t;
         }
@@ -318,24 +292,20 @@ __global__ void __launch_bounds__(kCaThreads, 2)
             }
             if (!(ok = mma_done(120))) break;
             if (it + 1 < nkt) {
-                if (MODE == 1) {
-                    stage_rows(kt + 1);
-                    __syncthreads();
-                }
+                stage_rows(kt + 1);
+                __syncthreads();
                 load_tile(sK, kx, kt + 1);
             }
             cp_async_commit();
 
             // ---- running max (two 32-column passes over the raw scores;
             // the scale is positive), then P = 2^(scale log2e S - max)
-            // packed over the scores already read. Masks only on the
-            // diagonal tile (MODE 0) or with several blocks per tile
-            // (MODE 1, b < 128).
-            const bool any_mask = MODE == 0 ? kt == qt : b < 128;
-            // kept key columns [klo, khi) of this row: the causal prefix of
-            // the diagonal tile, or the row's own block
-            const int klo = MODE == 0 ? 0 : (row / b) * b;
-            const int khi = MODE == 0 ? row + 1 : klo + b;
+            // packed over the scores already read. With several blocks per
+            // tile (b < 128) a row keeps its own block's key columns
+            // [klo, khi).
+            const bool any_mask = b < 128;
+            const int klo = (row / b) * b;
+            const int khi = klo + b;
             auto keep = [&](int c) -> bool { return c >= klo && c < khi; };
             float mx = -INFINITY;
 #pragma unroll
@@ -439,35 +409,26 @@ __global__ void __launch_bounds__(kCaThreads, 2)
         float of[DH];
 #pragma unroll
         for (int j = 0; j < DH / 2; ++j) f2unpack(o_acc[j], of[2 * j], of[2 * j + 1]);
-        if (MODE == 0) {
+        // MergeLSE(running = diag, this = off)
+        const float ld1 = RL[tok];
+        const float mu = fmaxf(ld1, logd);
+        const float w1 = __expf(ld1 - mu), w2 = __expf(logd - mu);
+        const float ssum = w1 + w2;
+        const float r = 1.0f / (ssum + eps);
+        const float c1 = w1 * r, c2 = w2 * inv * r;
 #pragma unroll
-            for (int j = 0; j < DH; j += 4)
-                *reinterpret_cast<float4 *>(o + j) =
-                    make_float4(of[j] * inv, of[j + 1] * inv,
-                                of[j + 2] * inv, of[j + 3] * inv);
-            if (half == 0) RL[tok] = logd;
-        } else {
-            // MergeLSE(running = diag, this = off)
-            const float ld1 = RL[tok];
-            const float mu = fmaxf(ld1, logd);
-            const float w1 = __expf(ld1 - mu), w2 = __expf(logd - mu);
-            const float ssum = w1 + w2;
-            const float r = 1.0f / (ssum + eps);
-            const float c1 = w1 * r, c2 = w2 * inv * r;
-#pragma unroll
-            for (int j = 0; j < DH; j += 4) {
-                float4 a = *reinterpret_cast<float4 *>(o + j);
-                a.x = c1 * a.x + c2 * of[j];
-                a.y = c1 * a.y + c2 * of[j + 1];
-                a.z = c1 * a.z + c2 * of[j + 2];
-                a.w = c1 * a.w + c2 * of[j + 3];
-                *reinterpret_cast<float4 *>(o + j) = a;
-            }
-            ld_new = mu + __logf(ssum + eps);
+        for (int j = 0; j < DH; j += 4) {
+            float4 a = *reinterpret_cast<float4 *>(o + j);
+            a.x = c1 * a.x + c2 * of[j];
+            a.y = c1 * a.y + c2 * of[j + 1];
+            a.z = c1 * a.z + c2 * of[j + 2];
+            a.w = c1 * a.w + c2 * of[j + 3];
+            *reinterpret_cast<float4 *>(o + j) = a;
         }
+        ld_new = mu + __logf(ssum + eps);
         __syncthreads();  // qrow_s is rewritten by the next item; both
                           // halves read RL before it changes
-        if (MODE == 1 && half == 0) RL[tok] = ld_new;
+        if (half == 0) RL[tok] = ld_new;
     }
     cp_async_wait<0>();
     tc_fence_before();
@@ -1079,24 +1040,18 @@ cudaError_t launch_seg_sort(const Plan &P, int Lv, const uint32_t *keyrank,
     return cudaGetLastError();
 }
 
-// mode 0: base segments of n_leaf rows; mode 1: SortLSH blocks of level
-// `level` (1 = top) whose halves hold m = N / 2^level rows.
-cudaError_t launch_causal_attn(const Plan &P, int mode, int n_leaf, int level,
-                               const void *q, const void *k, const void *v,
+// SortLSH blocks of level `level` (1 = top), whose halves hold
+// m = N / 2^level rows.
+cudaError_t launch_causal_attn(const Plan &P, int level, const void *q,
+                               const void *k, const void *v,
                                const int32_t *perms, int *next_item, float *RO,
                                float *RL, DeviceStatus *status,
                                cudaStream_t st) {
-    int items, m = 0;
-    const int32_t *pq = nullptr, *pk = nullptr;
-    if (mode == 0) {
-        items = P.BH * (P.N / n_leaf) * (n_leaf / 128);
-    } else {
-        m = P.N >> level;
-        items = P.BH * (P.N / (2 * m)) * (m / 128);
-        const size_t lvl = (size_t)(level - 1) * 2 * P.BH * (P.N / 2);
-        pq = perms + lvl;
-        pk = perms + lvl + (size_t)P.BH * (P.N / 2);
-    }
+    const int m = P.N >> level;
+    const int items = P.BH * (P.N / (2 * m)) * (m / 128);
+    const size_t lvl = (size_t)(level - 1) * 2 * P.BH * (P.N / 2);
+    const int32_t *pq = perms + lvl;
+    const int32_t *pk = pq + (size_t)P.BH * (P.N / 2);
     // at most two CTAs per SM (each holds 256 TMEM columns); persistent
     // CTAs, two per SM of a 152-SM GB300
     size_t smem = causal_attn_smem(P.d);
@@ -1107,15 +1062,12 @@ cudaError_t launch_causal_attn(const Plan &P, int mode, int n_leaf, int level,
                              (int)smem);
         kern<<<grid, kCaThreads, smem, st>>>(
             (const uint16_t *)q, (const uint16_t *)k, (const uint16_t *)v, pq,
-            pk, P.N, n_leaf, m, P.b, items, next_item, P.scale, P.eps, RO, RL,
+            pk, P.N, m, P.b, items, next_item, P.scale, P.eps, RO, RL,
             status);
         return cudaGetLastError();
     };
-    if (P.d == 128)
-        return mode == 0 ? launch(k_causal_attn_tc<128, 0>)
-                         : launch(k_causal_attn_tc<128, 1>);
-    return mode == 0 ? launch(k_causal_attn_tc<64, 0>)
-                     : launch(k_causal_attn_tc<64, 1>);
+    return P.d == 128 ? launch(k_causal_attn_tc<128>)
+                      : launch(k_causal_attn_tc<64>);
 }
 
 int causal_segments(const Plan &P) {

@@ -192,10 +192,15 @@ cudaError_t launch_bwd_keys_tc(const Plan &P, const void *k, const void *v,
 bool causal_tc_supported(const Plan &P, int n_leaf);
 cudaError_t launch_seg_sort(const Plan &P, int Lv, const uint32_t *keyrank,
                             int32_t *perms, cudaStream_t st);
-cudaError_t launch_causal_attn(const Plan &P, int mode, int n_leaf, int level,
-                               const void *q, const void *k, const void *v,
+cudaError_t launch_causal_attn(const Plan &P, int level, const void *q,
+                               const void *k, const void *v,
                                const int32_t *perms, int *next_item, float *RO,
                                float *RL, DeviceStatus *status,
+                               cudaStream_t st);
+// Exact causal attention of the base segments (causal_base.cu).
+cudaError_t launch_causal_base(const Plan &P, int n_leaf, const void *q,
+                               const void *k, const void *v, int *next_item,
+                               float *RO, float *RL, DeviceStatus *status,
                                cudaStream_t st);
 int causal_segments(const Plan &P);
 cudaError_t launch_causal_scan(const Plan &P, const void *k, const void *v,
