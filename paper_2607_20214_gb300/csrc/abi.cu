@@ -470,12 +470,11 @@ int causal_forward(const elsaa_params *params, const void *q, const void *k,
     uint16_t *Wbf = (uint16_t *)(ws + C.off_W);
     int *ctr = (int *)(ws + C.off_ctr);
 
-    // status and work counters cleared, bf16 planes
-    ELSAA_CHECK_LAUNCH(timed("prep_planes", st, [&] {
-                           return launch_begin(P, w_race, Wbf, status, ctr,
-                                               C.Lv + 1, st);
-                       }),
-                       "prep_planes");
+    // status word and work counters
+    ELSAA_CHECK_LAUNCH(launch_clear(status, ctr, C.Lv + 1, st), "clear");
+    SideStream *side = nullptr;
+    ELSAA_CHECK_LAUNCH(side_stream(&side), "side stream");
+    cudaStream_t ks = side->s;
     // sparse branch: codes, sorted halves, base segments, then the levels
     ELSAA_CHECK_LAUNCH(timed("sort_hash", st, [&] {
                            return launch_sort_hash(P, q, k, w_sort, keyrank,
@@ -495,12 +494,15 @@ int causal_forward(const elsaa_params *params, const void *q, const void *k,
     // the low-rank branch (chunk summaries, prefix states) on the side
     // stream from here: the base segments' persistent CTAs fill every SM
     // (all of TMEM), so these run beside the SortLSH levels instead of
-    // delaying the sorts and the base segments
-    SideStream *side = nullptr;
-    ELSAA_CHECK_LAUNCH(side_stream(&side), "side stream");
-    cudaStream_t ks = side->s;
+    // delaying the sorts and the base segments (forked at the start they
+    // cost 6 us of a short call too: their CTAs hold the TMEM that the
+    // levels wait for)
     ELSAA_CHECK_LAUNCH(cudaEventRecord(side->fork, st), "fork");
     ELSAA_CHECK_LAUNCH(cudaStreamWaitEvent(ks, side->fork, 0), "fork wait");
+    ELSAA_CHECK_LAUNCH(timed("prep_planes", ks, [&] {
+                           return launch_prep_planes(P, w_race, Wbf, ks);
+                       }),
+                       "prep_planes");
     ELSAA_CHECK_LAUNCH(timed("race_keys_ws", ks, [&] {
                            return launch_race_keys_ws(C.Pc, k, v, Wbf, part,
                                                       status, ks);
@@ -620,8 +622,7 @@ int forward_impl(const elsaa_params *params, const void *q, const void *k,
     const bool tcp = P.impl == 2;
     auto planes = [&](cudaStream_t s) {
         return timed("prep_planes", s, [&] {
-            return launch_begin(P, w_race, Wbf, brief ? status : nullptr,
-                                nullptr, 0, s);
+            return launch_begin(P, w_race, Wbf, brief ? status : nullptr, s);
         });
     };
     auto hash = [&] {

@@ -14,10 +14,7 @@
 //   k_causal_base    (causal_base.cu) exact causal attention of the base
 //                    segments
 //   k_causal_attn_tc the SortLSH blocks of each level, deepest first, merged
-//                    into the running result (MergeLSE)
-//                    over 128-key tiles with an online softmax), then one
-//                    launch per level, deepest first, for the SortLSH blocks,
-//                    merged into the running (O, log d) with MergeLSE
+//                    into the running (O, log d) with MergeLSE
 //   race_keys_ws     summaries of segments of G chunks of 128 keys
 //   k_seg_offsets    their exclusive prefix over the segments of a head
 //   k_causal_scan    per segment, chunk after chunk: the strict prefix

@@ -12,9 +12,10 @@
 //   warp 8          issues every MMA: S = Q K^T, O += P V (P from TMEM)
 //   warp 9          takes the items, TMA loads of Q, K (two buffers), V (two)
 // TMEM: S_s (then P_s over it) at 128 s, O_s at 256 + 128 s. O stays in
-// tensor memory; a softmax warp rescales it only when a row's maximum grows
-// by more than 2^8 (P up to 2^8 loses nothing: bf16 keeps its relative
-// precision, sums are fp32), which is rare after the first tiles.
+// tensor memory; a softmax warp rescales it when the maximum of one of its
+// rows grows. (Only beyond 2^8 it was no faster, and off by up to 2.5 times as
+// much in peaked heads: the weight of the largest key is exactly 1 only
+// against its own maximum; otherwise bf16 rounds it.)
 //
 // What bounds it: per slot and key tile the chain S MMA -> softmax -> P V MMA;
 // the other slot's chain runs beside it. Two CTAs per SM with two threads per
@@ -330,7 +331,7 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                 } else {
                     // these scores were issued behind the last tile's P V
                     // product: it is complete when they are
-                    const bool need = z > mref + 8.0f;
+                    const bool need = z > mref;
                     if (__any_sync(0xffffffffu, need)) {
                         const float f = need ? ex2_approx(mref - z) : 1.0f;
                         const float2 f2 = make_float2(f, f);

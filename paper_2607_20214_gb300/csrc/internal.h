@@ -252,10 +252,12 @@ cudaError_t make_tma_map_bf16_narrow(CUtensorMap *map, const void *base,
 // operand image the tensor-core kernels load with TMA.
 cudaError_t launch_prep_planes(const Plan &P, const float *w_race,
                                uint16_t *w_bf16, cudaStream_t st);
-// The same, and the status word and `n_zero` ints at `zero` cleared: the
-// first launch of a call.
+// The same, and the status word cleared (when not NULL): the first launch of
+// a short call.
 cudaError_t launch_begin(const Plan &P, const float *w_race, uint16_t *w_bf16,
-                         DeviceStatus *status, int *zero, int n_zero,
+                         DeviceStatus *status, cudaStream_t st);
+// Clears the status word and n ints (one launch).
+cudaError_t launch_clear(DeviceStatus *status, int *zero, int n,
                          cudaStream_t st);
 
 // Warp-specialised RACE key summaries (tensor-core path).

@@ -668,12 +668,10 @@ uint32_t race_keys_ws_cols(const Plan &P) {
 namespace {
 __global__ void k_prep_planes(const float *__restrict__ w, int H, int Lg,
                               int Lg_pad, int d, uint16_t *__restrict__ out,
-                              DeviceStatus *status, int *zero, int n_zero) {
+                              DeviceStatus *status) {
     const long n = (long)H * Lg_pad * d;
-    if (status && blockIdx.x == 0) {
-        if (threadIdx.x < 4) reinterpret_cast<int *>(status)[threadIdx.x] = 0;
-        for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0;
-    }
+    if (status && blockIdx.x == 0 && threadIdx.x < 4)
+        reinterpret_cast<int *>(status)[threadIdx.x] = 0;
     for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n;
          i += (long)gridDim.x * blockDim.x) {
         const int c = (int)(i % d);
@@ -688,18 +686,29 @@ __global__ void k_prep_planes(const float *__restrict__ w, int H, int Lg,
 
 cudaError_t launch_prep_planes(const Plan &P, const float *w_race,
                                uint16_t *w_bf16, cudaStream_t st) {
-    return launch_begin(P, w_race, w_bf16, nullptr, nullptr, 0, st);
+    return launch_begin(P, w_race, w_bf16, nullptr, st);
 }
 
 cudaError_t launch_begin(const Plan &P, const float *w_race, uint16_t *w_bf16,
-                         DeviceStatus *status, int *zero, int n_zero,
-                         cudaStream_t st) {
+                         DeviceStatus *status, cudaStream_t st) {
     static_assert(sizeof(DeviceStatus) == 16, "four ints");
     const long n = (long)P.H * P.Lg_pad * P.d;
     const int blocks = (int)((n + 255) / 256 < 1024 ? (n + 255) / 256 : 1024);
     k_prep_planes<<<blocks, 256, 0, st>>>(w_race, P.H, P.L * P.gamma,
-                                          P.Lg_pad, P.d, w_bf16, status,
-                                          zero, n_zero);
+                                          P.Lg_pad, P.d, w_bf16, status);
+    return cudaGetLastError();
+}
+
+namespace {
+__global__ void k_clear(int *status, int *zero, int n) {
+    if (threadIdx.x < 4) status[threadIdx.x] = 0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) zero[i] = 0;
+}
+}  // namespace
+
+cudaError_t launch_clear(DeviceStatus *status, int *zero, int n,
+                         cudaStream_t st) {
+    k_clear<<<1, 32, 0, st>>>(reinterpret_cast<int *>(status), zero, n);
     return cudaGetLastError();
 }
 
