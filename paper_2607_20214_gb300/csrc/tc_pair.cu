@@ -17,19 +17,29 @@
 // and the freed shared memory double-buffers the query tile and holds one
 // key and one value buffer per pass.
 //
-// Roles (640 threads per CTA): warps 0-15 compute (two TMEM slots of 256
-// columns, slot g takes the CTA's blocks of local index = g mod 2; within a
-// slot warps w and w + 4 split each row's keys, tables and output columns
-// in halves), warp 16 issues every MMA in the even CTA and relays the odd
-// CTA's readiness to it, warp 17 resolves row numbers, warp 18 loads the
-// per-head planes and summaries with TMA, warp 19 gathers values.
+// Roles (768 threads per CTA, as in the one-CTA kernel): warps 0-15 compute
+// (two TMEM slots of 256 columns, slot g takes the CTA's blocks of local
+// index = g mod 2; within a slot warps w and w + 4 split each row's keys,
+// tables and output columns in halves and meet at a barrier of their 64
+// threads), warp 16 issues every MMA in the even CTA and relays the odd
+// CTA's readiness to it, warp 17 loads the per-head planes and summaries
+// with TMA, warps 18-19 gather values, warps 20-23 queries and keys.
+//
+// What bounds it: the slots' own chain of hand-offs (the two slots' work is
+// about a third of the issue slots and the products about a quarter of the
+// tensor pipe's), so everything that another slot or pass can cover is off
+// that chain: gathers have warps of their own, the two slots' products are
+// issued independently of each other, the second pass's scores go out right
+// behind the first P V product, P is handed over before the features and
+// the fusion scalars are computed, and all features go to one product.
 //
 // TMEM columns of a slot (same layout in both CTAs): pass 0 scores keys
 // [0, 64) at [0, 64), the projections of row half 0's tables at [64, 96),
 // keys [64, 128) at [96, 160), row half 1's projections at [160, 192);
 // pass 1 scores keys [0, 64) at [0, 64), keys [64, 128) at [64, 128); P of
 // row half h in quarter 2h ([64h, 64h + 32)); the output accumulator at
-// [128, 256); the pre-scaled features as in the one-CTA kernel.
+// [128, 256); the pre-scaled features of buckets [0, 128) at [32, 64) and
+// [96, 128), those of buckets [128, 256) over P once P V is complete.
 //
 // Every hand-off is an mbarrier with a bounded wait; the odd CTA's
 // arrivals reach the even CTA's barriers through the relay (one remote
@@ -44,9 +54,15 @@ namespace {
 
 using namespace tc;
 
-constexpr int kPrThreads = 640;
+constexpr int kPrThreads = 768;
 constexpr int kPrMmaWarp = 16;
-constexpr int kPrLoaders = 32;
+constexpr int kPrVWarp = 18;   // 2 warps
+constexpr int kPrQkWarp = 20;  // 4 warps
+constexpr int kPrVThreads = 64, kPrQkThreads = 128;
+// registers: 16 compute warps and 8 others share the launch's 80 a thread
+constexpr int kPrRegsCompute = 96, kPrRegsOther = 48;
+static_assert(512 * kPrRegsCompute + 256 * kPrRegsOther <= kPrThreads * 80,
+              "register shares exceed what the block is launched with");
 constexpr int kPrNK = 128;   // keys per pass, query rows per CTA
 constexpr int kPrNP = 2;     // passes per block (b = 256)
 constexpr int kPrD = 128;    // head dimension
@@ -56,14 +72,11 @@ constexpr int kPrKRows1 = 64;  // pass-1 key buffer: 64 keys
 struct PrBars {
     // copies, relayed: the even CTA's copy also counts the odd CTA's phase
     uint64_t q_full[2], k_full[kPrNP], v_full[kPrNP], wb_full;
-    // compute hand-offs: the odd CTA's slot arrives once on the even CTA's
-    // barrier after its own named barrier
-    uint64_t tmem_empty[2], p_full[2], p2_full[2];
+    // compute hand-offs: one arrival per warp of the slot in both CTAs
+    uint64_t tmem_empty[2], p_full[2], phi_full[2];
     // MMA completions, committed to both CTAs
-    uint64_t s_full[2], pv0_done[2], pv_done[2], o_full[2], v_empty[kPrNP];
-    uint64_t head_done;
-    // local
-    uint64_t idx_full[2], idx_empty[2];
+    uint64_t q_empty[2], k_empty[kPrNP], v_empty[kPrNP];
+    uint64_t s_full[2], pv_done[2], o_full[2], head_done;
 };
 constexpr int kPrRelayed = 2 + kPrNP + kPrNP + 1;  // copy barriers
 
@@ -90,12 +103,8 @@ __global__ void __launch_bounds__(kPrThreads, 1)
     __shared__ PrBars bars;
     __shared__ uint32_t tbase;
     __shared__ int abort_flag;
-    __shared__ float xmax[2][2][128], xsum[2][2][128], xden[2][2][128];
-    // row numbers of a block's queries (this CTA's 128) and of this CTA's
-    // 64 keys of each pass, per block parity
-    __shared__ __align__(16) int qrow[2][128];
-    __shared__ __align__(16) int krow[2][NP][64];
-    __shared__ __align__(16) int vrow[128];  // value loader: the pass's keys
+    __shared__ float xmax[kPrNP][2][2][128];  // by pass
+    __shared__ float2 xsum[2][2][128];        // partial sums, Den
     volatile int *abort = &abort_flag;
     const int tid = threadIdx.x, warp = tid >> 5, lane_id = tid & 31;
     const uint32_t crank = cluster_rank();  // 0: issues the MMAs
@@ -121,7 +130,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
     // shared memory: two query tiles, the pass-0 key buffer (64 keys and
     // this CTA's 32 plane rows), the pass-1 key buffer, one value buffer per
     // pass (128 keys x this CTA's 64 columns), this CTA's 64 columns of the
-    // B summary, the A summary
+    // B summary, the A summary, 2 KB per compute warp for output rows
     const uint32_t tileQ = (uint32_t)nk * d * 2u;
     const uint32_t base = align1k(smem_u32(smem_raw));
     const uint32_t sQ = base;
@@ -130,6 +139,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
     const uint32_t sV = sK1 + kPrKRows1 * d * 2;
     const uint32_t sB = sV + NP * 16384u;
     const uint32_t sA = sB + align1k((uint32_t)r * 128u);
+    const uint32_t sO = sA + align1k((uint32_t)r * 4u);
     const float *Asm = reinterpret_cast<const float *>(
         smem_raw + (sA - smem_u32(smem_raw)));
     auto kbuf = [=](int p) { return p == 0 ? sK0 : sK1; };
@@ -139,20 +149,19 @@ __global__ void __launch_bounds__(kPrThreads, 1)
     if (tid == 0) {
         const uint32_t x = leader ? 1u : 0u;  // the relayed odd-CTA phase
         for (int s = 0; s < 2; ++s) {
-            mbar_init(&bars.q_full[s], 256 + x);
-            mbar_init(&bars.tmem_empty[s], 256 + x);
-            mbar_init(&bars.p_full[s], 256 + x);
-            mbar_init(&bars.p2_full[s], 256 + x);
+            mbar_init(&bars.q_full[s], kPrQkThreads + x);
+            mbar_init(&bars.q_empty[s], 1);
+            mbar_init(&bars.tmem_empty[s], 16);
+            mbar_init(&bars.p_full[s], 16);
+            mbar_init(&bars.phi_full[s], 16);
             mbar_init(&bars.s_full[s], 1);
-            mbar_init(&bars.pv0_done[s], 1);
             mbar_init(&bars.pv_done[s], 1);
             mbar_init(&bars.o_full[s], 1);
-            mbar_init(&bars.idx_full[s], kPrLoaders);
-            mbar_init(&bars.idx_empty[s], 256 * (1 + NP));
         }
         for (int p = 0; p < NP; ++p) {
-            mbar_init(&bars.k_full[p], 256 + x);
-            mbar_init(&bars.v_full[p], kPrLoaders + x);
+            mbar_init(&bars.k_full[p], kPrQkThreads + x);
+            mbar_init(&bars.k_empty[p], 1);
+            mbar_init(&bars.v_full[p], kPrVThreads + x);
             mbar_init(&bars.v_empty[p], 1);
         }
         mbar_init(&bars.wb_full, 1 + x);
@@ -166,60 +175,80 @@ __global__ void __launch_bounds__(kPrThreads, 1)
     tc_fence_after();
     const uint32_t tm = tbase;
 
-    // global row numbers of the 4 sorted positions pos.. pos + 3 of one
-    // head (rowbase = its first row); an entry outside [0, N) is read as
-    // row 0 (the orders come from the sort); the checked build records it
-    auto rows4 = [=](const int32_t *pm, int pos, int rowbase) {
-        int4 v;  // pos + 3 < N: N is a multiple of 256
-        if (((uintptr_t)(pm + pos) & 15u) == 0) {
-            v = *reinterpret_cast<const int4 *>(pm + pos);
-        } else {
-            v = make_int4(pm[pos], pm[pos + 1], pm[pos + 2], pm[pos + 3]);
-        }
-        auto fix = [=](int u) {
-            if (u < 0 || u >= N) {
+    // global row number of sorted position pos of one head (rowbase = its
+    // first row); an entry outside [0, N) is read as row 0 (the orders come
+    // from the sort); the checked build records it
+    auto global_row = [=](const int32_t *pm, int bh, int pos) {
+        int v = pm[(size_t)bh * N + pos];  // pos < N: N is a multiple of 256
+        if (v < 0 || v >= N) {
 #ifdef ELSAA_CHECKED
-                report(status, kDevPermRange, 14, rowbase / N, u);
+            report(status, kDevPermRange, 14, bh, v);
 #endif
-                u = 0;
-            }
-            return rowbase + u;
-        };
-        return make_int4(fix(v.x), fix(v.y), fix(v.z), fix(v.w));
+            v = 0;
+        }
+        return bh * N + v;
     };
 
+    if (warp >= kPrMmaWarp)
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(
+            kPrRegsOther));
     if (warp > kPrMmaWarp) {
         // ------------------------------------------------------------ loaders
-        const int role = warp - kPrMmaWarp - 1;
         const int lt = lane_id;
         auto lwait = [=](uint64_t *bar, uint32_t par, int site) {
             return __all_sync(0xffffffffu,
                               mbar_wait_or_abort(bar, par, abort, status,
                                                  site));
         };
-        if (role == 0) {
-            // row numbers of block j (this CTA's queries, its keys of each
-            // pass) into slot j & 1 once block j - 2's gathers went out
-            for (int j = 0; j < nblk; ++j) {
-                const int t = j & 1, bh = blk_head(j), pos = blk_pos(j);
-                if (j >= 2 &&
-                    !lwait(&bars.idx_empty[t], ((j >> 1) - 1) & 1, 70))
-                    break;
-                *reinterpret_cast<int4 *>(&qrow[t][4 * lt]) =
-                    rows4(perm_q + (size_t)bh * N, pos + 128 * crank + 4 * lt,
-                          bh * N);
-                if (lt < 16) {
+        if (warp >= kPrQkWarp) {
+            // queries and keys: per block this warp's 32 of the CTA's 128
+            // queries and, per pass, 16 of the CTA's 64 keys, two rows an
+            // instruction; lane l holds the number of query row l and of
+            // key l & 15 of pass l >> 4
+            const int w = warp - kPrQkWarp;
+            const int sub = lt >> 4, ch = lt & 15;
+            int qn = 0, kn = 0;  // of the next block
+            auto ahead = [&](int j) {
+                const int bh = blk_head(j), pos = blk_pos(j);
+                qn = global_row(perm_q, bh, pos + 128 * (int)crank + 32 * w +
+                                                lt);
+                kn = global_row(perm_k, bh,
+                                pos + 128 * (lt >> 4) + 64 * (int)crank +
+                                    16 * w + (lt & 15));
+            };
+            auto gather_k = [&](int p, int rows) {
 #pragma unroll
-                    for (int p = 0; p < NP; ++p)
-                        *reinterpret_cast<int4 *>(&krow[t][p][4 * lt]) =
-                            rows4(perm_k + (size_t)bh * N,
-                                  pos + 128 * p + 64 * crank + 4 * lt,
-                                  bh * N);
+                for (int i = 0; i < 16; i += 2) {
+                    const int rn =
+                        __shfl_sync(0xffffffffu, rows, 16 * p + i + sub);
+                    cp_async16(kbuf(p) + panel_offset(16 * w + i + sub, ch,
+                                                      krows(p)),
+                               kx + (size_t)rn * d + ch * 8);
                 }
-                __syncwarp();
-                mbar_arrive(&bars.idx_full[t]);
+                cp_async_mbar_arrive(&bars.k_full[p]);
+            };
+            if (nblk > 0) ahead(0);
+            for (int j = 0; j < nblk; ++j) {
+                const int qr = qn, kr = kn, s = j & 1;
+                if (j + 1 < nblk) ahead(j + 1);
+                if (j >= 1 && !lwait(&bars.k_empty[0], (j - 1) & 1, 70)) break;
+                gather_k(0, kr);
+                if (j >= 2 &&
+                    !lwait(&bars.q_empty[s], ((j >> 1) - 1) & 1, 75))
+                    break;
+#pragma unroll 4
+                for (int i = 0; i < 32; i += 2) {
+                    const int rn = __shfl_sync(0xffffffffu, qr, i + sub);
+                    cp_async16(sQ + s * tileQ +
+                                   panel_offset(32 * w + i + sub, ch, nk),
+                               qx + (size_t)rn * d + ch * 8);
+                }
+                cp_async_mbar_arrive(&bars.q_full[s]);
+                if (j >= 1 && !lwait(&bars.k_empty[1], (j - 1) & 1, 76)) break;
+                gather_k(1, kr);
             }
-        } else if (role == 1) {
+            cp_async_wait<0>();
+        } else if (warp == kPrMmaWarp + 1) {
             // per head, TMA: this CTA's 32 plane rows (its row half's tables:
             // rows [16 c, 16 c + 16) and [32 + 16 c, 48 + 16 c) of the head's
             // planes) under the pass-0 keys, its 64 columns of the B summary,
@@ -250,31 +279,35 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                 ++hc;
             }
         } else {
-            // values: for each pass, the pass's 128 keys, this CTA's 64
-            // columns (128 bytes of each row) into the pass's buffer once
-            // the previous block's P V product of that pass is done
-            const int lrow = lt >> 3, lc = lt & 7;  // 4 rows per instruction
-            bool go = true;
-            for (int j = 0; j < nblk && go; ++j) {
-                const int bh = blk_head(j), pos = blk_pos(j);
-                for (int p = 0; p < NP; ++p) {
-                    __syncwarp();  // the previous rows are all read
-                    *reinterpret_cast<int4 *>(&vrow[4 * lt]) =
-                        rows4(perm_k + (size_t)bh * N, pos + 128 * p + 4 * lt,
-                              bh * N);
-                    __syncwarp();
-                    if (j >= 1 &&
-                        !lwait(&bars.v_empty[p], (j - 1) & 1, 72)) {
-                        go = false;
-                        break;
-                    }
-                    const uint32_t dst = sV + p * 16384u;
-                    for (int row = lrow; row < nk; row += 4)
-                        cp_async16(dst + panel_offset(row, lc, nk),
-                                   vx + (size_t)vrow[row] * d +
-                                       64 * (int)crank + lc * 8);
-                    cp_async_mbar_arrive(&bars.v_full[p]);
+            // values: for each pass, this warp's 64 of the pass's 128 keys,
+            // this CTA's 64 columns (128 bytes of each row, four rows an
+            // instruction) into the pass's buffer once the previous block's
+            // P V product of that pass is done
+            const int r0 = 64 * (warp - kPrVWarp);
+            const int sub = lt >> 3, ch = lt & 7;
+            int n0 = 0, n1 = 0;  // of the next unit
+            auto ahead = [&](int u) {
+                const int j = u / NP;
+                const int bh = blk_head(j);
+                const int pos = blk_pos(j) + 128 * (u - j * NP) + r0 + lt;
+                n0 = global_row(perm_k, bh, pos);
+                n1 = global_row(perm_k, bh, pos + 32);
+            };
+            if (nblk > 0) ahead(0);
+            for (int u = 0; u < nblk * NP; ++u) {
+                const int a0 = n0, a1 = n1, j = u / NP, p = u - j * NP;
+                if (u + 1 < nblk * NP) ahead(u + 1);
+                if (j >= 1 && !lwait(&bars.v_empty[p], (j - 1) & 1, 72)) break;
+                const uint32_t dst = sV + p * 16384u;
+#pragma unroll 4
+                for (int i = 0; i < 64; i += 4) {
+                    const int rn = __shfl_sync(0xffffffffu, i < 32 ? a0 : a1,
+                                               (i + sub) & 31);
+                    cp_async16(dst + panel_offset(r0 + i + sub, ch, nk),
+                               vx + (size_t)rn * d + 64 * (int)crank +
+                                   ch * 8);
                 }
+                cp_async_mbar_arrive(&bars.v_full[p]);
             }
             cp_async_wait<0>();
         }
@@ -330,124 +363,119 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             }
         } else if (lane_id == 0 && nblk > 0) {
             // ------------------------------------------------- MMA issue
-            // Event driven as in the one-CTA kernel, over units (block,
-            // pass): the oldest block's second feature part first, then
-            // P V (with the first feature part after the last pass), then
-            // the next scores. Pass 1's scores reuse the S columns and wait
-            // for pass 0's P V product.
+            // Event driven, each slot at a stage of its own: 0 scores and
+            // projections, 1 P V of pass 0 and, right behind it, the scores
+            // of pass 1 (2; products run in the order of their issue, so
+            // they overwrite P only after its product has read it), 3 P V
+            // of pass 1, 4 the features' product. A new head's planes and
+            // summaries replace the old ones only after head_done: its
+            // first scores wait until every product of the blocks before
+            // is issued.
             const uint32_t id_sp = idesc_bf16(256, nk + 64, false, false);
             const uint32_t id_s = idesc_bf16(256, nk, false, false);
             const uint32_t id_o = idesc_bf16(256, d, false, true);
-            const int r0 = min(r, nk);
-            const bool two_parts = r > nk;
-            const int nunits = nblk * NP;
-            int us = 0, up = 0, i2 = 0, blocks_pv = 0, hc = 0;
+            int j = 0, stage = 0;    // this round's slot (j & 1)
+            int jo = 1, stageo = 0;  // the other slot
+            int done = 0, hc = 0;  // blocks finished, heads begun
+            auto scores = [&](int s, int p) {
+                fence_proxy_async_smem();  // cp.async data -> MMA
+                tc_fence_after();
+                const uint32_t so = tm + 256u * s;
+                const uint32_t kb = kbuf(p);
+                const int kr = krows(p);
+                for (int kk = 0; kk < d / 16; ++kk)
+                    // pass 0: scores and projections (N = 192); pass 1:
+                    // scores only
+                    mma_pair_ss(so,
+                                smem_desc(sQ + s * tileQ +
+                                              (kk >> 2) * 128 * 128 +
+                                              (kk & 3) * 32,
+                                          16, 1024),
+                                smem_desc(kb + (kk >> 2) * kr * 128 +
+                                              (kk & 3) * 32,
+                                          16, 1024),
+                                p == 0 ? id_sp : id_s, kk > 0);
+                mma_commit_pair(&bars.s_full[s]);
+                mma_commit_pair(&bars.k_empty[p]);
+                if (p == NP - 1) mma_commit_pair(&bars.q_empty[s]);
+            };
+            auto values = [&](int s, int p) {  // O (+)= P V
+                fence_proxy_async_smem();
+                tc_fence_after();
+                const uint32_t so = tm + 256u * s, vb = sV + p * 16384u;
+                for (int kk = 0; kk < nk / 16; ++kk)
+                    mma_pair_ts(so + nk, so + quarter_col(kk, 0),
+                                smem_desc(vb + kk * 2048, (uint32_t)nk * 128,
+                                          1024),
+                                id_o, p > 0 || kk > 0);
+                mma_commit_pair(&bars.v_empty[p]);
+                if (p == NP - 1) mma_commit_pair(&bars.pv_done[s]);
+            };
             unsigned long long t_last = global_ns();
-            while ((two_parts ? i2 : blocks_pv) < nblk) {
+            uint32_t idle = 0;  // the clock is read every 256 idle rounds
+            while (done < nblk) {
                 bool did = false;
-                if (two_parts && i2 < blocks_pv) {
-                    const int s = i2 & 1;
-                    const uint32_t so = tm + 256u * s;
-                    if (mbar_test(&bars.p2_full[s], (i2 >> 1) & 1)) {
-                        tc_fence_after();
-                        for (int kk = 0; kk < (r - nk) / 16; ++kk)
-                            mma_pair_ts(so + nk, so + quarter_col(kk, 0),
-                                        smem_desc(sB + (uint32_t)nk * 128 +
-                                                      kk * 2048,
-                                                  (uint32_t)r * 128, 1024),
-                                        id_o, 1);
-                        mma_commit_pair(&bars.o_full[s]);
-                        if (last_of_head(i2)) mma_commit_pair(&bars.head_done);
-                        ++i2;
-                        did = true;
-                    }
-                }
-                if (up < us) {
-                    const int j = up / NP, p = up - j * NP, s = j & 1;
-                    const int su = (j >> 1) * NP + p;  // unit within slot
-                    const uint32_t so = tm + 256u * s;
-                    if (mbar_test(&bars.p_full[s], su & 1) &&
-                        mbar_test(&bars.v_full[p], j & 1)) {
-                        fence_proxy_async_smem();  // cp.async data -> MMA
-                        tc_fence_after();
-                        const uint32_t vb = sV + p * 16384u;
-                        for (int kk = 0; kk < nk / 16; ++kk)  // O (+)= P V
-                            mma_pair_ts(so + nk, so + quarter_col(kk, 0),
-                                        smem_desc(vb + kk * 2048,
-                                                  (uint32_t)nk * 128, 1024),
-                                        id_o, p > 0 || kk > 0);
-                        mma_commit_pair(&bars.v_empty[p]);
-                        if (p < NP - 1) {
-                            mma_commit_pair(&bars.pv0_done[s]);
-                        } else {
-                            for (int kk = 0; kk < r0 / 16; ++kk)  // + Phi' B
-                                mma_pair_ts(so + nk, so + quarter_col(kk, 32),
-                                            smem_desc(sB + kk * 2048,
-                                                      (uint32_t)r * 128,
-                                                      1024),
-                                            id_o, 1);
-                            if (two_parts) {
-                                mma_commit_pair(&bars.pv_done[s]);
-                            } else {
-                                mma_commit_pair(&bars.o_full[s]);
-                                if (last_of_head(j))
-                                    mma_commit_pair(&bars.head_done);
-                            }
-                            ++blocks_pv;
+                if (j < nblk) {
+                    const int s = j & 1, k = j >> 1;
+                    bool go = false;
+                    if (stage == 0) {
+                        const bool nh = new_head(j);
+                        go = !(nh && done < j) &&
+                             mbar_test(&bars.k_full[0], j & 1) &&
+                             mbar_test(&bars.q_full[s], k & 1) &&
+                             (j < 2 ||
+                              mbar_test(&bars.tmem_empty[s], (k - 1) & 1)) &&
+                             (!nh || mbar_test(&bars.wb_full, hc & 1));
+                        if (go) {
+                            if (nh) ++hc;
+                            scores(s, 0);
                         }
-                        ++up;
-                        did = true;
-                    }
-                }
-                // a new head's planes and summaries replace the old ones
-                // only after head_done: its first scores wait until every
-                // MMA of the previous head is issued
-                const int js = us / NP, ps = us - js * NP;
-                const bool nh = ps == 0 && new_head(js);
-                if (us < nunits &&
-                    !(nh && js > 0 && (two_parts ? i2 : blocks_pv) < js)) {
-                    const int s = js & 1;
-                    const uint32_t so = tm + 256u * s;
-                    bool ready = mbar_test(&bars.k_full[ps], js & 1);
-                    if (ready && ps == 0)
-                        ready = mbar_test(&bars.q_full[s],
-                                                  (js >> 1) & 1) &&
-                                (js < 2 ||
-                                 mbar_test(&bars.tmem_empty[s],
-                                                   ((js >> 1) - 1) & 1)) &&
-                                (!nh || mbar_test(&bars.wb_full,
-                                                          hc & 1));
-                    if (ready && ps > 0)  // S columns hold P of pass ps - 1
-                        ready = mbar_test(&bars.pv0_done[s],
-                                          ((js >> 1) * (NP - 1) + ps - 1) &
-                                              1);
-                    if (ready) {
-                        if (nh) ++hc;
-                        fence_proxy_async_smem();  // cp.async data -> MMA
-                        tc_fence_after();
-                        const uint32_t kb = kbuf(ps);
-                        const int kr = krows(ps);
-                        for (int kk = 0; kk < d / 16; ++kk) {
-                            const uint32_t oq =
-                                (kk >> 2) * 128 * 128 + (kk & 3) * 32;
-                            const uint32_t okw =
-                                (kk >> 2) * kr * 128 + (kk & 3) * 32;
-                            // pass 0: scores and projections (N = 192);
-                            // pass 1: scores only
-                            mma_pair_ss(so,
-                                        smem_desc(sQ + s * tileQ + oq, 16,
-                                                  1024),
-                                        smem_desc(kb + okw, 16, 1024),
-                                        ps == 0 ? id_sp : id_s, kk > 0);
+                    } else if (stage == 1) {
+                        go = mbar_test(&bars.p_full[s], 0) &&
+                             mbar_test(&bars.v_full[0], j & 1);
+                        if (go) values(s, 0);
+                    } else if (stage == 2) {
+                        go = mbar_test(&bars.k_full[1], j & 1);
+                        if (go) scores(s, 1);
+                    } else if (stage == 3) {
+                        go = mbar_test(&bars.p_full[s], 1) &&
+                             mbar_test(&bars.v_full[1], j & 1);
+                        if (go) values(s, 1);
+                    } else {
+                        go = mbar_test(&bars.phi_full[s], k & 1);
+                        if (go) {
+                            tc_fence_after();
+                            const uint32_t so = tm + 256u * s;
+                            for (int kk = 0; kk < r / 16; ++kk)  // O += Phi' B
+                                mma_pair_ts(
+                                    so + nk,
+                                    so + (kk < 8 ? quarter_col(kk, 32)
+                                                 : quarter_col(kk - 8, 0)),
+                                    smem_desc(sB + kk * 2048,
+                                              (uint32_t)r * 128, 1024),
+                                    id_o, 1);
+                            mma_commit_pair(&bars.o_full[s]);
+                            if (last_of_head(done))
+                                mma_commit_pair(&bars.head_done);
+                            ++done;
+                            j += 2;
                         }
-                        mma_commit_pair(&bars.s_full[s]);
-                        ++us;
+                    }
+                    if (go) {
+                        stage = stage == 4 ? 0 : stage + 1;
                         did = true;
                     }
                 }
+                int x = j;  // the slots take turns
+                j = jo;
+                jo = x;
+                x = stage;
+                stage = stageo;
+                stageo = x;
                 if (did) {
-                    t_last = global_ns();
-                } else {
+                    idle = 0;
+                } else if ((++idle & 255u) == 0) {
+                    if (idle == 256) t_last = global_ns();
                     if (*abort) break;
                     if (global_ns() - t_last > kWaitLimitNs) {
                         *abort = 1;
@@ -466,9 +494,10 @@ __global__ void __launch_bounds__(kPrThreads, 1)
         // half of the pair gathered when h equals its rank), the tables of
         // the 64-bucket chunks h and h + 2 and output columns [64 h, 64 h +
         // 64).
-        const int cw = warp;
-        const int g = cw >> 3;
-        const int half = (cw >> 2) & 1;
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(
+            kPrRegsCompute));
+        const int g = warp >> 3;
+        const int half = (warp >> 2) & 1;
         const int row = (warp & 3) * 32 + lane_id;  // query row = TMEM lane
         const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
         constexpr int T = 64 / R;  // tables per 64-bucket chunk
@@ -476,194 +505,142 @@ __global__ void __launch_bounds__(kPrThreads, 1)
         const int ta1 = min((half + 2) * T, L), nt1 = min(ta1 + T, L) - ta1;
         const uint32_t cb0 = half ? 96u : 32u, cb1 = half ? 64u : 0u;
         const float sl2e = scale * kLog2e;
-        auto wwait = [=](uint64_t *bar, uint32_t par, int site) {
+        // barrier of the row's two warps; a pair's 64 threads leave a wait
+        // with one verdict (an abort seen by one warp only would strand the
+        // other there)
+        const int pid = 1 + g * 4 + (warp & 3);
+        auto pwait = [=](uint64_t *bar, uint32_t par, int site) {
             const bool ok = mbar_wait_or_abort(bar, par, abort, status, site);
-            return named_sync_and(1 + g, 256, ok);
+            return named_sync_and(pid, 64, ok);
         };
-        const int ct = (cw & 7) * 32 + lane_id;  // 0..255 within the slot
-        // a hand-off to the MMA issuer: every thread of the even CTA's slot
-        // arrives; the odd CTA's slot meets at its named barrier and one
-        // thread arrives on the even CTA's barrier
+        // a hand-off to the MMA issuer: once per warp, on the even CTA's
+        // barrier
         auto signal = [&](uint64_t *bar) {
-            if (leader) {
-                mbar_arrive(bar);
-            } else {
-                named_sync(1 + g, 256);
-                if (ct == 0) mbar_arrive_remote(bar, 0);
+            tc_fence_before();
+            __syncwarp();
+            if (lane_id == 0) {
+                if (leader)
+                    mbar_arrive(bar);
+                else
+                    mbar_arrive_remote(bar, 0);
             }
         };
-        const int crow = ct >> 4, cc = ct & 15;  // 16 chunks per row
-        // block j's queries into query buffer j & 1 (8 copies a thread)
-        auto gather_q = [&](int j) -> bool {
-            if (!wwait(&bars.idx_full[j & 1], (j >> 1) & 1, 75)) return false;
-            const int *rows = qrow[j & 1];
-            const uint32_t dst = sQ + (j & 1) * tileQ;
-            for (int rr = crow; rr < nk; rr += 16)
-                cp_async16(dst + panel_offset(rr, cc, nk),
-                           qx + (size_t)rows[rr] * d + cc * 8);
-            cp_async_mbar_arrive(&bars.q_full[j & 1]);
-            mbar_arrive(&bars.idx_empty[j & 1]);
-            return true;
-        };
-        // this CTA's 64 keys of block j's pass p into key buffer p
-        auto gather_k = [&](int j, int p) -> bool {
-            if (!wwait(&bars.idx_full[j & 1], (j >> 1) & 1, 76)) return false;
-            const int *rows = krow[j & 1][p];
-            const uint32_t dst = kbuf(p);
-            const int ld = krows(p);
-            for (int rr = crow; rr < 64; rr += 16)
-                cp_async16(dst + panel_offset(rr, cc, ld),
-                           kx + (size_t)rows[rr] * d + cc * 8);
-            cp_async_mbar_arrive(&bars.k_full[p]);
-            mbar_arrive(&bars.idx_empty[j & 1]);
-            return true;
-        };
-        bool started = true;
-        if (nblk > 0) {
-            if (g == 0)
-                started = gather_q(0) && gather_k(0, 0) && gather_k(0, 1);
-            else if (nblk > 1)
-                started = gather_q(1);
-        }
-        for (int j = g; started && j < nblk; j += 2) {
+        for (int j = g; j < nblk; j += 2) {
             const int k = j >> 1;
             const uint32_t so = tm + 256u * g + lane;
             const int bh = blk_head(j);
             const int qpos = blk_pos(j) + 128 * (int)crank + row;
             int qi = perm_q[(size_t)bh * N + qpos];  // prefetch
-            if (!wwait(&bars.s_full[g], (k * NP) & 1, 77)) break;
+            if (!pwait(&bars.s_full[g], 0, 77)) break;
+            // the A summary came by TMA: acquire its head's stage (complete
+            // already: this block's scores waited for it)
+            if ((j < 2 || blk_head(j) != blk_head(j - 2)) &&
+                !pwait(&bars.wb_full, (bh - blk_head(0)) & 1, 78))
+                break;
             tc_fence_after();
-            // this half's raw projections (pass 0 writes them where pass 0's
-            // P and the output accumulator go): the per-bit factors and Den
-            // are computed once pass 0's P is handed to its P V product
-            uint32_t pr[32];
-            const uint32_t pcol = 64u + 96u * half;  // this half's projections
-            tmem_ld16(so + pcol, *reinterpret_cast<uint32_t(*)[16]>(pr));
-            tmem_ld16(so + pcol + 16,
-                      *reinterpret_cast<uint32_t(*)[16]>(pr + 16));
-            tmem_wait_ld();
-            // pass 0: this half's 64 key columns start at 96 h
-            const uint32_t kc0 = 96u * half;
-            float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-            for (int c = 0; c < 64; c += 16) {
-                uint32_t v[16];
-                tmem_ld16(so + kc0 + c, v);
-                tmem_wait_ld();
-#pragma unroll
-                for (int jj = 0; jj < 16; ++jj)
-                    mxa[jj & 3] = fmaxf(mxa[jj & 3], __uint_as_float(v[jj]));
-            }
-            float mx = fmaxf(fmaxf(mxa[0], mxa[1]), fmaxf(mxa[2], mxa[3]));
-            xmax[g][half][row] = mx;
-            named_sync(1 + g, 256);  // every projection of the slot is read
-            mx = fmaxf(xmax[g][0][row], xmax[g][1][row]);
-            float M2 = mx * sl2e;
-            float ls[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            // P of this half into quarter 2 half (over half 0's scores, or
-            // over half 0's projections, read before the barrier above)
-            const uint32_t pc = 64u * half;
-#pragma unroll
-            for (int c = 0; c < 64; c += 32) {
-                uint32_t pk16[16];
-#pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                    uint32_t v[16];
-                    tmem_ld16(so + kc0 + c + 16 * hh, v);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int jj = 0; jj < 16; jj += 2) {
-                        const float a0 = ex2_approx(
-                            fmaf(__uint_as_float(v[jj]), sl2e, -M2));
-                        const float a1 = ex2_approx(
-                            fmaf(__uint_as_float(v[jj + 1]), sl2e, -M2));
-                        ls[(jj >> 1) & 3] += a0 + a1;
-                        pk16[8 * hh + (jj >> 1)] = pack_bf16x2(a0, a1);
-                    }
-                }
-                tmem_st16(so + pc + (c >> 1), pk16);
-            }
-            float lsum = (ls[0] + ls[1]) + (ls[2] + ls[3]);
-            xsum[g][half][row] = lsum;
-            tc_fence_before();
-            named_sync(1 + g, 256);  // every S read of the slot is done
-            tc_fence_after();
-            lsum = xsum[g][0][row] + xsum[g][1][row];
-            float sp[32];
-            uint32_t sp1[8];
-            float dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // independent chains
-            float denf = 0.0f;
-            bool pass_fail = false;
-#pragma unroll
-            for (int ps = 1; ps < NP; ++ps) {
-                // the previous pass's P goes to its P V product; this pass
-                // scores the next 128 keys into columns [0, 128)
-                tmem_wait_st();
-                tc_fence_before();
-                signal(&bars.p_full[g]);
-                // the key buffer of pass ps - 1 is free since its scores
-                // completed: the next block's keys, off the chain to the P V
-                // product just handed over
-                if (j + 1 < nblk && !gather_k(j + 1, ps - 1)) {
-                    pass_fail = true;
-                    break;
-                }
-                if (ps == 1) {
-                    // per-bit factors of this half's tables (sp[0, 16):
-                    // chunk half, sp[16, 32): chunk half + 2) and partial
-                    // Den, while pass 0's P V product and pass 1's scores
-                    // run. The A summary came by TMA: acquire its head's
-                    // stage (complete already: the scores waited for it)
-                    if ((j < 2 || blk_head(j) != blk_head(j - 2)) &&
-                        !wwait(&bars.wb_full,
-                               (blk_head(j) - blk_head(0)) & 1, 78)) {
-                        pass_fail = true;
-                        break;
-                    }
-                    race_factors16(pr, nt0 * G, beta, sp);
-                    chunk_den<G, T>(sp, nt0, Asm + ta0 * R, dacc);
-                    if (nt1 > 0) {
-                        race_factors16(pr + 16, nt1 * G, beta, sp + 16);
-                        chunk_den<G, T>(sp + 16, nt1, Asm + ta1 * R, dacc);
-                        // the second chunk's factors wait for the P V
-                        // product: kept as fp16 pairs (factors lie in
-                        // (0.11, 0.89); relative rounding 2^-11, below the
-                        // bf16 rounding of the features they make)
-#pragma unroll
-                        for (int q = 0; q < 8; ++q)
-                            sp1[q] = pack_f16x2(sp[16 + 2 * q],
-                                                sp[17 + 2 * q]);
-                    }
-                    xden[g][half][row] =
-                        (dacc[0] + dacc[1]) + (dacc[2] + dacc[3]);
-                }
-                if (!wwait(&bars.s_full[g], (k * NP + ps) & 1, 79)) {
-                    pass_fail = true;
-                    break;
-                }
-                tc_fence_after();
-                float mxb[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            // row maximum of both halves (an array per pass: pass 1 writes
+            // its own while the other half may still read pass 0's)
+            auto row_max = [&](int ps, const float (&m)[4]) {
+                xmax[ps][g][half][row] =
+                    fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+                named_sync(pid, 64);
+                return fmaxf(xmax[ps][g][0][row], xmax[ps][g][1][row]);
+            };
+            // maximum over this half's 64 scores at column c0
+            auto max64 = [&](uint32_t c0, float (&m)[4]) {
 #pragma unroll
                 for (int c = 0; c < 64; c += 16) {
                     uint32_t v[16];
-                    tmem_ld16(so + pc + c, v);
+                    tmem_ld16(so + c0 + c, v);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int jj = 0; jj < 16; ++jj)
-                        mxb[jj & 3] = fmaxf(mxb[jj & 3], __uint_as_float(v[jj]));
+                    for (int q = 0; q < 16; q += 2)
+                        m[(q >> 1) & 3] =
+                            max3(m[(q >> 1) & 3], __uint_as_float(v[q]),
+                                 __uint_as_float(v[q + 1]));
                 }
-                xmax[g][half][row] =
-                    fmaxf(fmaxf(mxb[0], mxb[1]), fmaxf(mxb[2], mxb[3]));
-                named_sync(1 + g, 256);
-                const float M2b =
-                    fmaxf(xmax[g][0][row], xmax[g][1][row]) * sl2e;
-                if (ps == 1)
-                    denf = (xden[g][0][row] + xden[g][1][row]) *
-                           (1.0f / (float)L);
+            };
+            // P of this half's 64 scores at column c0, into quarter 2 half
+            // (behind scores already read); returns its row sum
+            const uint32_t pc = 64u * half;
+            auto exp64 = [&](uint32_t c0, float M) -> float {
+                const float2 sl2 = make_float2(sl2e, sl2e),
+                             mn = make_float2(-M, -M);
+                float2 ls[2] = {make_float2(0.0f, 0.0f),
+                                make_float2(0.0f, 0.0f)};
+#pragma unroll
+                for (int c = 0; c < 64; c += 32) {
+                    uint32_t v[32], pw[16];
+                    tmem_ld32(so + c0 + c, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < 32; q += 2) {
+                        const float2 z =
+                            fma2(make_float2(__uint_as_float(v[q]),
+                                             __uint_as_float(v[q + 1])),
+                                 sl2, mn);
+                        const float2 e =
+                            make_float2(ex2_approx(z.x), ex2_approx(z.y));
+                        ls[(q >> 1) & 1] = add2(ls[(q >> 1) & 1], e);
+                        pw[q >> 1] = pack_bf16x2(e.x, e.y);
+                    }
+                    tmem_st16(so + pc + (c >> 1), pw);
+                }
+                return (ls[0].x + ls[1].x) + (ls[0].y + ls[1].y);
+            };
+            // pass 0. This half's raw projections are read first (P and the
+            // output accumulator go over them), its 64 scores start at 96 h
+            uint32_t pr[32];
+            const uint32_t pcol = 64u + 96u * half;
+            tmem_ld16(so + pcol, *reinterpret_cast<uint32_t(*)[16]>(pr));
+            tmem_ld16(so + pcol + 16,
+                      *reinterpret_cast<uint32_t(*)[16]>(pr + 16));
+            const uint32_t kc0 = 96u * half;
+            float mxa[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+            max64(kc0, mxa);
+            float M2 = row_max(0, mxa) * sl2e;
+            float lsum = exp64(kc0, M2);  // this half's
+            tmem_wait_st();
+            signal(&bars.p_full[g]);
+            // per-bit factors of this half's tables (sp[0, 16): chunk half,
+            // sp[16, 32): chunk half + 2) and its part of Den, while pass
+            // 0's P V product and pass 1's scores run. The second chunk's
+            // factors wait for the last P V product: kept as fp16 pairs
+            // (factors lie in (0.11, 0.89); relative rounding 2^-11, below
+            // the bf16 rounding of the features they make)
+            qi = (qi < 0 || qi >= N) ? 0 : qi;
+            const size_t tok = (size_t)bh * N + qi;
+            const float lam = lambda_tok ? lambda_tok[tok] : lambda;
+            const float gs = gates ? gates[2 * tok] : 1.0f;
+            const float gl = gates ? gates[2 * tok + 1] : 1.0f;
+            float sp[16];
+            uint32_t sp1[8];
+            float den;
+            {
+                float dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // independent chains
+                if (nt1 > 0) {
+                    float s1[16];
+                    race_factors<16>(pr + 16, beta, s1);
+                    chunk_den<G, T>(s1, nt1, Asm + ta1 * R, dacc);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        sp1[q] = pack_f16x2(s1[2 * q], s1[2 * q + 1]);
+                }
+                race_factors<16>(pr, beta, sp);
+                chunk_den<G, T>(sp, nt0, Asm + ta0 * R, dacc);
+                den = (dacc[0] + dacc[1]) + (dacc[2] + dacc[3]);
+            }
+            // pass 1
+            if (!pwait(&bars.s_full[g], 1, 79)) break;
+            tc_fence_after();
+            {
+                float mxb[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+                max64(pc, mxb);
+                const float M2b = row_max(1, mxb) * sl2e;
                 // online softmax: keep the running reference unless the
                 // row's max grew by more than 2^8; then rescale the
                 // accumulator (the previous P V product is complete: these
-                // scores waited for it) and the running sum
+                // scores were issued behind it) and the running sum
                 const bool need = M2b > M2 + 8.0f;
                 const float f = need ? ex2_approx(M2 - M2b) : 1.0f;
                 if (__any_sync(0xffffffffu, need)) {
@@ -682,41 +659,20 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                     lsum *= f;
                     M2 = M2b;
                 }
-                float lb[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-#pragma unroll
-                for (int c = 0; c < 64; c += 32) {
-                    uint32_t pk16[16];
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t v[16];
-                        tmem_ld16(so + pc + c + 16 * hh, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int jj = 0; jj < 16; jj += 2) {
-                            const float a0 = ex2_approx(
-                                fmaf(__uint_as_float(v[jj]), sl2e, -M2));
-                            const float a1 = ex2_approx(
-                                fmaf(__uint_as_float(v[jj + 1]), sl2e, -M2));
-                            lb[(jj >> 1) & 3] += a0 + a1;
-                            pk16[8 * hh + (jj >> 1)] = pack_bf16x2(a0, a1);
-                        }
-                    }
-                    tmem_st16(so + pc + (c >> 1), pk16);
-                }
-                xsum[g][half][row] = (lb[0] + lb[1]) + (lb[2] + lb[3]);
-                tc_fence_before();
-                named_sync(1 + g, 256);
-                tc_fence_after();
-                lsum += xsum[g][0][row] + xsum[g][1][row];
+                lsum += exp64(pc, M2);
             }
-            if (pass_fail) break;
+            tmem_wait_st();
+            signal(&bars.p_full[g]);
             // fusion scalars (Eq. (5) in log-sum-exp form, Eq. (6))
-            qi = (qi < 0 || qi >= N) ? 0 : qi;
-            const size_t tok = (size_t)bh * N + qi;
+            xsum[g][half][row] = make_float2(lsum, den);
+            named_sync(pid, 64);
+            {
+                const float2 o = xsum[g][half ^ 1][row];
+                lsum += o.x;
+                den += o.y;
+            }
+            const float denf = den * (1.0f / (float)L);
             const float log_ds = M2 * kLn2 + __logf(lsum);
-            const float lam = lambda_tok ? lambda_tok[tok] : lambda;
-            const float gs = gates ? gates[2 * tok] : 1.0f;
-            const float gl = gates ? gates[2 * tok + 1] : 1.0f;
             const float msp =
                 fusion_multiplier_fast(log_ds, lam, denf, eps, mode);
             const float c1 =
@@ -725,17 +681,9 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             const float ratio =
                 __fdividef(gl, (float)L * (denf + eps) * c1e);
             if (nt0 > 0) write_phi_chunk<G, T>(sp, nt0, ratio, so + cb0);
-            tmem_wait_st();
-            tc_fence_before();
-            signal(&bars.p_full[g]);
-            // the last pass's key buffer and the query buffer are free since
-            // the last scores completed: the next block's keys, the queries
-            // of the block after next
-            if ((j + 1 < nblk && !gather_k(j + 1, NP - 1)) ||
-                (j + 2 < nblk && !gather_q(j + 2)))
-                break;
             if (r > nk) {
-                if (!wwait(&bars.pv_done[g], k & 1, 80)) break;
+                // over P: its product is complete
+                if (!pwait(&bars.pv_done[g], k & 1, 80)) break;
                 tc_fence_after();
                 if (nt1 > 0) {
                     float f1[16];
@@ -744,22 +692,20 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                         unpack_f16x2(sp1[q], f1[2 * q], f1[2 * q + 1]);
                     write_phi_chunk<G, T>(f1, nt1, ratio, so + cb1);
                 }
-                tmem_wait_st();
-                tc_fence_before();
-                signal(&bars.p2_full[g]);
             }
-            if (!wwait(&bars.o_full[g], k & 1, 81)) break;
+            tmem_wait_st();
+            signal(&bars.phi_full[g]);
+            if (!pwait(&bars.o_full[g], k & 1, 81)) break;
             tc_fence_after();
-            // O = c1 acc, this half's 64 columns, straight from the
-            // registers: fp32, or bf16 in 32-byte stores (a whole sector
-            // each) when O is 32-byte aligned
-            const bool o_a32 = ((uintptr_t)ox & 31u) == 0;
+            // O = c1 acc, this half's 64 columns: bf16 through this warp's
+            // 2 KB, 16 rows at a time, out in 128-byte rows; fp32 from the
+            // registers
+            if constexpr (O32) {
 #pragma unroll
-            for (int c = 0; c < 64; c += 16) {
-                uint32_t v[16];
-                tmem_ld16(so + nk + half * 64 + c, v);
-                tmem_wait_ld();
-                if constexpr (O32) {
+                for (int c = 0; c < 64; c += 16) {
+                    uint32_t v[16];
+                    tmem_ld16(so + nk + half * 64 + c, v);
+                    tmem_wait_ld();
                     float4 *dst = reinterpret_cast<float4 *>(
                         o32 + tok * (size_t)d + half * 64 + c);
 #pragma unroll
@@ -768,31 +714,58 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                                              c1e * __uint_as_float(v[4 * q + 1]),
                                              c1e * __uint_as_float(v[4 * q + 2]),
                                              c1e * __uint_as_float(v[4 * q + 3]));
-                } else {
-                    uint32_t ob[8];
+                }
+                signal(&bars.tmem_empty[g]);
+            } else {
+                uint32_t ob[32];
 #pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        ob[q] = pack_bf16x2(c1e * __uint_as_float(v[2 * q]),
-                                            c1e * __uint_as_float(v[2 * q + 1]));
-                    uint16_t *dst = ox + tok * (size_t)d + half * 64 + c;
-                    if (o_a32) {
-                        st_global_v8(dst, ob);
-                    } else {
-                        uint4 *d4 = reinterpret_cast<uint4 *>(dst);
-                        d4[0] = make_uint4(ob[0], ob[1], ob[2], ob[3]);
-                        d4[1] = make_uint4(ob[4], ob[5], ob[6], ob[7]);
+                for (int c = 0; c < 64; c += 32) {
+                    uint32_t v[32];
+                    tmem_ld32(so + nk + half * 64 + c, v);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) {
+                        const float2 x = mul2(
+                            make_float2(c1e, c1e),
+                            make_float2(__uint_as_float(v[2 * q]),
+                                        __uint_as_float(v[2 * q + 1])));
+                        ob[c / 2 + q] = pack_bf16x2(x.x, x.y);
                     }
                 }
+                signal(&bars.tmem_empty[g]);
+                const uint32_t ow = sO + 2048u * warp;
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    if ((lane_id >> 4) == hh) {
+#pragma unroll
+                        for (int q = 0; q < 8; ++q)
+                            st_shared_v4(ow + (lane_id & 15) * 128 +
+                                             ((q ^ (lane_id & 7)) << 4),
+                                         ob[4 * q], ob[4 * q + 1],
+                                         ob[4 * q + 2], ob[4 * q + 3]);
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const int rl = 4 * i + (lane_id >> 3);
+                        const int to = __shfl_sync(0xffffffffu, (int)tok,
+                                                   16 * hh + rl);
+                        const uint4 val = ld_shared_v4(
+                            ow + rl * 128 +
+                            (((lane_id & 7) ^ (rl & 7)) << 4));
+                        *reinterpret_cast<uint4 *>(ox + (size_t)to * d +
+                                                   half * 64 +
+                                                   (lane_id & 7) * 8) = val;
+                    }
+                    __syncwarp();
+                }
             }
-            tc_fence_before();
-            signal(&bars.tmem_empty[g]);
             if (half == 0) {
                 if (log_ds_out) log_ds_out[tok] = log_ds;
                 if (dlr_out) dlr_out[tok] = denf;
                 if (m_out) m_out[tok] = msp;
             }
         }
-        cp_async_wait<0>();
     }
     tc_fence_before();
     __syncthreads();
@@ -813,7 +786,8 @@ size_t pair_smem(const Plan &P) {
     const size_t r = (size_t)P.r;
     return 1024 + 2 * (size_t)kPrNK * kPrD * 2 +
            (size_t)(kPrKRows0 + kPrKRows1) * kPrD * 2 + kPrNP * 16384 +
-           (r * 128 + 1023) / 1024 * 1024 + (r * 4 + 1023) / 1024 * 1024;
+           (r * 128 + 1023) / 1024 * 1024 + (r * 4 + 1023) / 1024 * 1024 +
+           16 * 2048;
 }
 
 cudaError_t launch_block_attn_pair(

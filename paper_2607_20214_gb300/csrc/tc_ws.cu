@@ -478,13 +478,13 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             const int qpos = p0 + row;
             const bool qvalid = qpos < N;
             int qi = perm_q[(size_t)bh * N + min(qpos, N - 1)];  // prefetch
+            if (!pwait(&bars.s_full[g], (k * NPASS) & 1, 51)) break;
+            tc_fence_after();
             // the A summary (read below) came by TMA: acquire its head's
-            // stage (complete already when S of this tile is)
+            // stage (complete already: S of this tile waited for it)
             if (bh != last_bh && !pwait(&bars.wb_full, (bh - bh0) & 1, 55))
                 break;
             last_bh = bh;
-            if (!pwait(&bars.s_full[g], (k * NPASS) & 1, 51)) break;
-            tc_fence_after();
             // SEL: this row's selected candidates among this half's 64 keys
             // of pass ps (bit k of the 64-bit word: key kbeg + k)
             const size_t selrow = (size_t)bh * N + (size_t)min(qpos, N - 1);
