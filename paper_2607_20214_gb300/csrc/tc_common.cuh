@@ -280,6 +280,22 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t start, uint32_t lbo,
     return d;
 }
 
+// The descriptor of the same operand `bytes` further on (a multiple of 16;
+// the sum stays below the 256 KB that the address field spans).
+__device__ __forceinline__ uint64_t desc_at(uint64_t desc, uint32_t bytes) {
+    return desc + (bytes >> 4);
+}
+
+// True in one lane of the (converged) warp, the same one on every call.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t e;
+    asm volatile(
+        "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(e));
+    return e != 0;
+}
+
 // Instruction descriptor, kind::f16 with bf16 A/B and fp32 accumulation.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn,
                                                   bool b_mn) {

@@ -319,49 +319,46 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             // first, then counts once more on the even CTA's copy. A phase
             // cannot complete twice before it is relayed: the next one needs
             // MMAs that wait for this relay.
-            if (lane_id == 0) {
-                uint64_t *bar[kPrRelayed] = {
-                    &bars.q_full[0], &bars.q_full[1], &bars.k_full[0],
-                    &bars.k_full[1], &bars.v_full[0], &bars.v_full[1],
-                    &bars.wb_full};
-                const int in0 = (nblk + 1) / 2, in1 = nblk / 2;  // per slot
-                int heads = 0;
-                for (int j = 0; j < nblk; ++j) heads += new_head(j) ? 1 : 0;
-                const int want[kPrRelayed] = {in0,  in1,  nblk, nblk,
-                                              nblk, nblk, heads};
-                int done[kPrRelayed];
-                int left = 0;
-                for (int i = 0; i < kPrRelayed; ++i) {
-                    done[i] = 0;
-                    left += want[i];
+            // One lane per barrier.
+            static_assert(kPrRelayed == 2 + 2 * kPrNP + 1, "lane order below");
+            uint64_t *bar = &bars.wb_full;
+            int want = 0, done = 0;
+            if (lane_id < 2) {
+                bar = &bars.q_full[lane_id];
+                want = (nblk + 1 - lane_id) / 2;
+            } else if (lane_id < 2 + NP) {
+                bar = &bars.k_full[lane_id - 2];
+                want = nblk;
+            } else if (lane_id < 2 + 2 * NP) {
+                bar = &bars.v_full[lane_id - 2 - NP];
+                want = nblk;
+            } else if (lane_id == 2 + 2 * NP) {
+                for (int j = 0; j < nblk; ++j) want += new_head(j) ? 1 : 0;
+            }
+            unsigned long long t_last = global_ns();
+            uint32_t idle = 0;  // the clock is read every 256 idle rounds
+            while (__any_sync(0xffffffffu, done < want)) {
+                const bool hit =
+                    done < want && mbar_test(bar, (uint32_t)done & 1u);
+                if (hit) {
+                    // this CTA's cp.async data -> the pair's MMAs
+                    fence_proxy_async_smem();
+                    mbar_arrive_remote(bar, 0);
+                    ++done;
                 }
-                unsigned long long t_last = global_ns();
-                while (left > 0) {
-                    bool did = false;
-                    for (int i = 0; i < kPrRelayed; ++i) {
-                        if (done[i] < want[i] &&
-                            mbar_test(bar[i], (uint32_t)done[i] & 1u)) {
-                            // this CTA's cp.async data -> the pair's MMAs
-                            fence_proxy_async_smem();
-                            mbar_arrive_remote(bar[i], 0);
-                            ++done[i];
-                            --left;
-                            did = true;
-                        }
+                if (__any_sync(0xffffffffu, hit)) {
+                    idle = 0;
+                } else if ((++idle & 255u) == 0) {
+                    if (idle == 256) t_last = global_ns();
+                    const bool late = global_ns() - t_last > kWaitLimitNs;
+                    if (late) {
+                        *abort = 1;
+                        record_timeout(status, 73);
                     }
-                    if (did) {
-                        t_last = global_ns();
-                    } else {
-                        if (*abort) break;
-                        if (global_ns() - t_last > kWaitLimitNs) {
-                            *abort = 1;
-                            record_timeout(status, 73);
-                            break;
-                        }
-                    }
+                    if (__any_sync(0xffffffffu, late || *abort)) break;
                 }
             }
-        } else if (lane_id == 0 && nblk > 0) {
+        } else if (nblk > 0) {
             // ------------------------------------------------- MMA issue
             // Event driven, each slot at a stage of its own: 0 scores and
             // projections, 1 P V of pass 0 and, right behind it, the scores
@@ -377,39 +374,63 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             int j = 0, stage = 0;    // this round's slot (j & 1)
             int jo = 1, stageo = 0;  // the other slot
             int done = 0, hc = 0;  // blocks finished, heads begun
+            // The whole warp runs the loop, so that its state and the
+            // operands' descriptors are warp-uniform; one lane issues.
+            const bool el = elect_one();
+            auto test = [&](uint64_t *bar, uint32_t par) -> bool {
+                return __all_sync(0xffffffffu, mbar_test(bar, par));
+            };
+            const uint64_t dQ = smem_desc(sQ, 16, 1024),
+                           dK0 = smem_desc(sK0, 16, 1024),
+                           dK1 = smem_desc(sK1, 16, 1024),
+                           dV = smem_desc(sV, (uint32_t)nk * 128, 1024),
+                           dB = smem_desc(sB, (uint32_t)r * 128, 1024);
             auto scores = [&](int s, int p) {
                 fence_proxy_async_smem();  // cp.async data -> MMA
                 tc_fence_after();
                 const uint32_t so = tm + 256u * s;
-                const uint32_t kb = kbuf(p);
-                const int kr = krows(p);
-                for (int kk = 0; kk < d / 16; ++kk)
+                const uint64_t a = desc_at(dQ, s * tileQ);
+                if (el) {
                     // pass 0: scores and projections (N = 192); pass 1:
                     // scores only
-                    mma_pair_ss(so,
-                                smem_desc(sQ + s * tileQ +
-                                              (kk >> 2) * 128 * 128 +
-                                              (kk & 3) * 32,
-                                          16, 1024),
-                                smem_desc(kb + (kk >> 2) * kr * 128 +
-                                              (kk & 3) * 32,
-                                          16, 1024),
-                                p == 0 ? id_sp : id_s, kk > 0);
-                mma_commit_pair(&bars.s_full[s]);
-                mma_commit_pair(&bars.k_empty[p]);
-                if (p == NP - 1) mma_commit_pair(&bars.q_empty[s]);
+                    if (p == 0) {
+#pragma unroll
+                        for (int kk = 0; kk < d / 16; ++kk)
+                            mma_pair_ss(
+                                so,
+                                desc_at(a, (kk >> 2) * 16384 + (kk & 3) * 32),
+                                desc_at(dK0, (kk >> 2) * kPrKRows0 * 128 +
+                                                 (kk & 3) * 32),
+                                id_sp, kk > 0);
+                    } else {
+#pragma unroll
+                        for (int kk = 0; kk < d / 16; ++kk)
+                            mma_pair_ss(
+                                so,
+                                desc_at(a, (kk >> 2) * 16384 + (kk & 3) * 32),
+                                desc_at(dK1, (kk >> 2) * kPrKRows1 * 128 +
+                                                 (kk & 3) * 32),
+                                id_s, kk > 0);
+                    }
+                    mma_commit_pair(&bars.s_full[s]);
+                    mma_commit_pair(&bars.k_empty[p]);
+                    if (p == NP - 1) mma_commit_pair(&bars.q_empty[s]);
+                }
             };
             auto values = [&](int s, int p) {  // O (+)= P V
                 fence_proxy_async_smem();
                 tc_fence_after();
-                const uint32_t so = tm + 256u * s, vb = sV + p * 16384u;
-                for (int kk = 0; kk < nk / 16; ++kk)
-                    mma_pair_ts(so + nk, so + quarter_col(kk, 0),
-                                smem_desc(vb + kk * 2048, (uint32_t)nk * 128,
-                                          1024),
-                                id_o, p > 0 || kk > 0);
-                mma_commit_pair(&bars.v_empty[p]);
-                if (p == NP - 1) mma_commit_pair(&bars.pv_done[s]);
+                const uint32_t so = tm + 256u * s;
+                const uint64_t b = desc_at(dV, p * 16384u);
+                if (el) {
+#pragma unroll
+                    for (int kk = 0; kk < nk / 16; ++kk)
+                        mma_pair_ts(so + nk, so + quarter_col(kk, 0),
+                                    desc_at(b, kk * 2048), id_o,
+                                    p > 0 || kk > 0);
+                    mma_commit_pair(&bars.v_empty[p]);
+                    if (p == NP - 1) mma_commit_pair(&bars.pv_done[s]);
+                }
             };
             unsigned long long t_last = global_ns();
             uint32_t idle = 0;  // the clock is read every 256 idle rounds
@@ -421,42 +442,45 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                     if (stage == 0) {
                         const bool nh = new_head(j);
                         go = !(nh && done < j) &&
-                             mbar_test(&bars.k_full[0], j & 1) &&
-                             mbar_test(&bars.q_full[s], k & 1) &&
+                             test(&bars.k_full[0], j & 1) &&
+                             test(&bars.q_full[s], k & 1) &&
                              (j < 2 ||
-                              mbar_test(&bars.tmem_empty[s], (k - 1) & 1)) &&
-                             (!nh || mbar_test(&bars.wb_full, hc & 1));
+                              test(&bars.tmem_empty[s], (k - 1) & 1)) &&
+                             (!nh || test(&bars.wb_full, hc & 1));
                         if (go) {
                             if (nh) ++hc;
                             scores(s, 0);
                         }
                     } else if (stage == 1) {
-                        go = mbar_test(&bars.p_full[s], 0) &&
-                             mbar_test(&bars.v_full[0], j & 1);
+                        go = test(&bars.p_full[s], 0) &&
+                             test(&bars.v_full[0], j & 1);
                         if (go) values(s, 0);
                     } else if (stage == 2) {
-                        go = mbar_test(&bars.k_full[1], j & 1);
+                        go = test(&bars.k_full[1], j & 1);
                         if (go) scores(s, 1);
                     } else if (stage == 3) {
-                        go = mbar_test(&bars.p_full[s], 1) &&
-                             mbar_test(&bars.v_full[1], j & 1);
+                        go = test(&bars.p_full[s], 1) &&
+                             test(&bars.v_full[1], j & 1);
                         if (go) values(s, 1);
                     } else {
-                        go = mbar_test(&bars.phi_full[s], k & 1);
+                        go = test(&bars.phi_full[s], k & 1);
                         if (go) {
                             tc_fence_after();
                             const uint32_t so = tm + 256u * s;
-                            for (int kk = 0; kk < r / 16; ++kk)  // O += Phi' B
-                                mma_pair_ts(
-                                    so + nk,
-                                    so + (kk < 8 ? quarter_col(kk, 32)
-                                                 : quarter_col(kk - 8, 0)),
-                                    smem_desc(sB + kk * 2048,
-                                              (uint32_t)r * 128, 1024),
-                                    id_o, 1);
-                            mma_commit_pair(&bars.o_full[s]);
-                            if (last_of_head(done))
-                                mma_commit_pair(&bars.head_done);
+                            if (el) {
+#pragma unroll
+                                for (int kk = 0; kk < 16; ++kk)
+                                    if (16 * kk < r)  // O += Phi' B
+                                        mma_pair_ts(
+                                            so + nk,
+                                            so + (kk < 8
+                                                      ? quarter_col(kk, 32)
+                                                      : quarter_col(kk - 8, 0)),
+                                            desc_at(dB, kk * 2048), id_o, 1);
+                                mma_commit_pair(&bars.o_full[s]);
+                                if (last_of_head(done))
+                                    mma_commit_pair(&bars.head_done);
+                            }
                             ++done;
                             j += 2;
                         }
@@ -476,12 +500,12 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                     idle = 0;
                 } else if ((++idle & 255u) == 0) {
                     if (idle == 256) t_last = global_ns();
-                    if (*abort) break;
-                    if (global_ns() - t_last > kWaitLimitNs) {
+                    const bool late = global_ns() - t_last > kWaitLimitNs;
+                    if (late) {
                         *abort = 1;
                         record_timeout(status, 74);
-                        break;
                     }
+                    if (__any_sync(0xffffffffu, late || *abort)) break;
                 }
             }
         }
