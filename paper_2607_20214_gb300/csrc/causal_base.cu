@@ -155,13 +155,24 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                          load(bars.v_full, bars.v_empty, sV, &tmV, row, 153);
                 }
             }
-        } else if (warp == 8 && lane_id == 0) {
+        } else if (warp == 8) {
             // ---------------------------------------------------- MMA issue
             // Whenever a slot's P is ready: its P V product, and right behind
             // it the scores of its next key tile over the same columns. The
             // products of one thread run in the order they are issued, so
             // the scores need no wait for the product before them (with one,
             // 518 us).
+            // The whole warp runs the loop, so that its state and the
+            // operands' descriptors are warp-uniform; one lane issues.
+            const bool el = elect_one();
+            auto test = [&](uint64_t *bar, uint32_t par) -> bool {
+                return __all_sync(0xffffffffu, mbar_test(bar, par));
+            };
+            auto wait = [&](uint64_t *bar, uint32_t par, int site) -> bool {
+                return __all_sync(0xffffffffu,
+                                  mbar_wait_or_abort(bar, par, abort, status,
+                                                     site));
+            };
             const uint32_t id_s = idesc_bf16(128, 128, false, false);
             const uint32_t id_o = idesc_bf16(128, D, false, true);
             const uint64_t dQ = smem_desc(sQ, 16, 1024);
@@ -173,16 +184,15 @@ __global__ void __launch_bounds__(kCbThreads, 1)
             int go0 = 0, go1 = 0;      // items finished per slot
             bool ok = true;
             for (int it = 0; ok; ++it) {
-                ok = mbar_wait_or_abort(&bars.item_full[it & 1], (it >> 1) & 1,
-                                        abort, status, 154);
+                ok = wait(&bars.item_full[it & 1], (it >> 1) & 1, 154);
                 if (!ok) break;
                 const int item = item_s[it & 1];
-                mbar_arrive(&bars.item_empty[it & 1]);
+                __syncwarp();
+                if (el) mbar_arrive(&bars.item_empty[it & 1]);
                 if (item < 0) break;
                 const CbItem w(item, N, n_leaf, segs);
                 const int n0 = w.n[0], n1 = w.n[1];
-                ok = mbar_wait_or_abort(&bars.q_full, it & 1, abort, status,
-                                        155);
+                ok = wait(&bars.q_full, it & 1, 155);
                 if (!ok) break;
                 int us0 = 0, us1 = 0, up0 = 0, up1 = 0;
                 // the scores of slot s's next key tile
@@ -190,22 +200,24 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                                   int n_o) {
                     constexpr int s = decltype(slot)::value;
                     const int st = (c0 + us) & 1;
-                    if (!mbar_wait_or_abort(&bars.k_full[st],
-                                            ((c0 + us) >> 1) & 1, abort,
-                                            status, 160))
+                    if (!wait(&bars.k_full[st], ((c0 + us) >> 1) & 1, 160))
                         return false;
                     tc_fence_after();
                     const uint64_t q = dQ + s * kTile, k = dK + st * kTile;
+                    if (el) {
 #pragma unroll
-                    for (int x = 0; x < D / 16; ++x) {
-                        const uint32_t o = (x >> 2) * 1024 + (x & 3) * 2;
-                        mma_ss(tm + 128u * s, q + o, k + o, id_s, x > 0);
+                        for (int x = 0; x < D / 16; ++x) {
+                            const uint32_t o = (x >> 2) * 1024 + (x & 3) * 2;
+                            mma_ss(tm + 128u * s, q + o, k + o, id_s, x > 0);
+                        }
+                        mma_commit(&bars.s_full[s]);
+                        // both slots have used the tile
+                        if (us >= n_o || us_o > us)
+                            mma_commit(&bars.k_empty[st]);
+                        if (us + 1 == n && us_o == n_o)
+                            mma_commit(&bars.q_empty);
                     }
-                    mma_commit(&bars.s_full[s]);
-                    // both slots have used the tile
-                    if (us >= n_o || us_o > us) mma_commit(&bars.k_empty[st]);
                     ++us;
-                    if (us == n && us_o == n_o) mma_commit(&bars.q_empty);
                     return true;
                 };
                 auto step = [&](auto slot, int &us, int &up, int &gp, int go,
@@ -213,20 +225,23 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                     constexpr int s = decltype(slot)::value;
                     constexpr uint32_t cS = 128u * s, cO = cS + 256u;
                     const int st = (c0 + up) & 1;
-                    if (up == us || !mbar_test(&bars.p_full[s], gp & 1) ||
-                        !mbar_test(&bars.v_full[st], ((c0 + up) >> 1) & 1) ||
+                    if (up == us || !test(&bars.p_full[s], gp & 1) ||
+                        !test(&bars.v_full[st], ((c0 + up) >> 1) & 1) ||
                         (up == 0 && go > 0 &&
-                         !mbar_test(&bars.o_empty[s], (go - 1) & 1)))
+                         !test(&bars.o_empty[s], (go - 1) & 1)))
                         return false;
                     tc_fence_after();
                     const uint64_t v = dV + st * kTile;
                     const uint32_t more = up > 0;
+                    if (el) {
 #pragma unroll
-                    for (int x = 0; x < 8; ++x)
-                        mma_ts(tm + cO, tm + cS + 8 * x, v + 128 * x, id_o,
-                               x > 0 ? 1u : more);
-                    mma_commit(&bars.o_done[s]);
-                    if (up >= n_o || up_o > up) mma_commit(&bars.v_empty[st]);
+                        for (int x = 0; x < 8; ++x)
+                            mma_ts(tm + cO, tm + cS + 8 * x, v + 128 * x, id_o,
+                                   x > 0 ? 1u : more);
+                        mma_commit(&bars.o_done[s]);
+                        if (up >= n_o || up_o > up)
+                            mma_commit(&bars.v_empty[st]);
+                    }
                     ++up;
                     ++gp;
                     if (us < n) ok = scores(slot, us, n, us_o, n_o);
@@ -246,17 +261,13 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                     if (a || b) {
                         idle = 0;
                     } else if ((++idle & 255u) == 0) {
-                        if (*abort) {
-                            ok = false;
-                            break;
-                        }
                         if (idle == 256u) t_last = global_ns();
-                        if (global_ns() - t_last > kWaitLimitNs) {
+                        const bool late = global_ns() - t_last > kWaitLimitNs;
+                        if (late) {
                             *abort = 1;
                             record_timeout(status, 156);
-                            ok = false;
-                            break;
                         }
+                        ok = !__any_sync(0xffffffffu, late || *abort);
                     }
                 }
                 c0 += max(n0, n1);

@@ -175,7 +175,15 @@ __global__ void __launch_bounds__(kKwThreads, 2)
         __syncwarp();
     } else if (warp == 1) {
         // ----------------------------------------------------------- MMA issue
-        if (lane_id == 0 && ntiles > 0) {
+        if (ntiles > 0) {
+            // the whole warp runs the loop (its state and the operands'
+            // descriptors are warp-uniform); one lane issues
+            const bool el = elect_one();
+            auto wait = [&](uint64_t *bar, uint32_t par, int site) -> bool {
+                return __all_sync(0xffffffffu,
+                                  mbar_wait_or_abort(bar, par, abort, status,
+                                                     site));
+            };
             const uint32_t id_proj = idesc_bf16(128, Lg_pad, false, false);
             const uint32_t id_b = idesc_bf16(128, d + 16, true, true);
             const int last0 = last_mtile(0), last1 = last_mtile(1);
@@ -183,22 +191,26 @@ __global__ void __launch_bounds__(kKwThreads, 2)
                 const int kb = it % nkb;
                 const uint32_t sK = kb ? sK1 : sK0;
                 const uint32_t dst = t + colP + 64u * (it & 1);
-                for (int k = 0; k < d / 16; ++k) {
-                    uint32_t oa = (k >> 2) * 128 * 128 + (k & 3) * 32;
-                    uint32_t ow = (k >> 2) * Lg_pad * 128 + (k & 3) * 32;
-                    mma_ss(dst, smem_desc(sK + oa, 16, 1024),
-                           smem_desc(sW + ow, 16, 1024), id_proj, k > 0);
-                }
+                const uint64_t a = smem_desc(sK, 16, 1024),
+                               b = smem_desc(sW, 16, 1024);
+                if (!el) return;
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    if (16 * k < d)
+                        mma_ss(dst,
+                               desc_at(a, (k >> 2) * 16384 + (k & 3) * 32),
+                               desc_at(b, (uint32_t)(k >> 2) * Lg_pad * 128 +
+                                              (k & 3) * 32),
+                               id_proj, k > 0);
                 mma_commit(&bars.proj_full[it & 1]);
                 mma_commit(&bars.k_empty[kb]);
             };
             // projections run two tiles ahead (both TMEM buffers); each
             // iteration issues the summary MMAs of tile i, then the
             // projection of tile i + 2
-            bool ok = mbar_wait_or_abort(&bars.w_full, 0, abort, status, 60);
+            bool ok = wait(&bars.w_full, 0, 60);
             for (int it = 0; it < 2 && it < ntiles && ok; ++it) {
-                ok = mbar_wait_or_abort(&bars.k_full[it % nkb], (it / nkb) & 1,
-                                        abort, status, 63);
+                ok = wait(&bars.k_full[it % nkb], (it / nkb) & 1, 63);
                 if (ok) {
                     tc_fence_after();
                     proj(it);
@@ -206,44 +218,42 @@ __global__ void __launch_bounds__(kKwThreads, 2)
             }
             for (int i = 0; i < ntiles && ok; ++i) {
                 const int b = i & 1;
-                ok = mbar_wait_or_abort(&bars.v_full[b], (i >> 1) & 1, abort,
-                                        status, 66);
+                ok = wait(&bars.v_full[b], (i >> 1) & 1, 66);
                 const uint32_t sV = b ? sV1 : sV0;
                 const uint32_t vst = b ? vs1 : 16384u;
                 bool got0 = false, got1 = false;
                 for (int m = 0; m < nM && ok; ++m) {
                     if (tile_needs(m, 0) && !got0)
-                        got0 = ok = mbar_wait_or_abort(&bars.phi_full[0], i & 1,
-                                                       abort, status, 65);
+                        got0 = ok = wait(&bars.phi_full[0], i & 1, 65);
                     if (ok && tile_needs(m, 1) && !got1)
-                        got1 = ok = mbar_wait_or_abort(&bars.phi_full[1], i & 1,
-                                                       abort, status, 65);
+                        got1 = ok = wait(&bars.phi_full[1], i & 1, 65);
                     if (!ok) break;
                     tc_fence_after();
-                    for (int k = 0; k < 8; ++k) {  // 128 keys, 16 per step
-                        uint64_t a = smem_desc(sPhi + 2 * m * 16384 + k * 2048,
-                                               16384, 1024);
-                        uint32_t acc = (i > 0 || k > 0) ? 1u : 0u;
-                        mma_ss(t + m * accN, a,
-                               smem_desc(sV + k * 2048, vst, 1024), id_b,
-                               acc);
+                    const uint64_t da = smem_desc(sPhi + 2 * m * 16384, 16384,
+                                                  1024),
+                                   db = smem_desc(sV, vst, 1024);
+                    const uint32_t more = i > 0;
+                    if (el) {
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)  // 128 keys, 16 per step
+                            mma_ss(t + m * accN, desc_at(da, k * 2048),
+                                   desc_at(db, k * 2048), id_b,
+                                   k > 0 ? 1u : more);
+                        if (m == last0) mma_commit(&bars.phi_empty[0]);
+                        if (m == last1) mma_commit(&bars.phi_empty[1]);
                     }
-                    if (m == last0) mma_commit(&bars.phi_empty[0]);
-                    if (m == last1) mma_commit(&bars.phi_empty[1]);
                 }
                 if (!ok) break;
-                mma_commit(&bars.v_empty[b]);
+                if (el) mma_commit(&bars.v_empty[b]);
                 if (i + 2 < ntiles) {
                     // the features of tile i have read projection buffer b
-                    ok = mbar_wait_or_abort(&bars.k_full[(i + 2) % nkb],
-                                            ((i + 2) / nkb) & 1, abort,
-                                            status, 64);
+                    ok = wait(&bars.k_full[(i + 2) % nkb], ((i + 2) / nkb) & 1, 64);
                     if (!ok) break;
                     tc_fence_after();
                     proj(i + 2);
                 }
             }
-            if (ok) mma_commit(&bars.done);
+            if (ok && el) mma_commit(&bars.done);
         }
         __syncwarp();
     } else {
@@ -464,25 +474,36 @@ __global__ void __launch_bounds__(kKtThreads, 1)
         __syncwarp();
     } else if (warp == 1) {
         // ----------------------------------------------------------- MMA issue
-        if (lane_id == 0 && ntiles > 0) {
+        if (ntiles > 0) {
+            // the whole warp runs the loop (its state and the operands'
+            // descriptors are warp-uniform); one lane issues
+            const bool el = elect_one();
+            auto wait = [&](uint64_t *bar, uint32_t par, int site) -> bool {
+                return __all_sync(0xffffffffu,
+                                  mbar_wait_or_abort(bar, par, abort, status,
+                                                     site));
+            };
             const uint32_t id_proj = idesc_bf16(128, Lg_pad, false, false);
             const uint32_t id_b = idesc_bf16(128, r, true, true);
             auto proj = [=](int it) {
                 const uint32_t sK = sK0 + (it & 1) * tileB;
                 const uint32_t dst = t + colP + 64u * (it & 1);
-                for (int k = 0; k < d / 16; ++k) {
-                    uint32_t oa = (k >> 2) * 128 * 128 + (k & 3) * 32;
-                    uint32_t ow = (k >> 2) * Lg_pad * 128 + (k & 3) * 32;
-                    mma_ss(dst, smem_desc(sK + oa, 16, 1024),
-                           smem_desc(sW + ow, 16, 1024), id_proj, k > 0);
-                }
+                const uint64_t a = smem_desc(sK, 16, 1024),
+                               b = smem_desc(sW, 16, 1024);
+                if (!el) return;
+#pragma unroll
+                for (int k = 0; k < d / 16; ++k)
+                    mma_ss(dst, desc_at(a, (k >> 2) * 16384 + (k & 3) * 32),
+                           desc_at(b, (uint32_t)(k >> 2) * Lg_pad * 128 +
+                                          (k & 3) * 32),
+                           id_proj, k > 0);
                 mma_commit(&bars.proj_full[it & 1]);
                 mma_commit(&bars.k_empty[it & 1]);
             };
             // projections run two tiles ahead (both TMEM buffers)
-            bool ok = mbar_wait_or_abort(&bars.w_full, 0, abort, status, 60);
+            bool ok = wait(&bars.w_full, 0, 60);
             for (int it = 0; it < 2 && it < ntiles && ok; ++it) {
-                ok = mbar_wait_or_abort(&bars.k_full[it], 0, abort, status, 63);
+                ok = wait(&bars.k_full[it], 0, 63);
                 if (ok) {
                     tc_fence_after();
                     proj(it);
@@ -490,34 +511,36 @@ __global__ void __launch_bounds__(kKtThreads, 1)
             }
             for (int i = 0; i < ntiles && ok; ++i) {
                 const int b = i & 1;
-                ok = mbar_wait_or_abort(&bars.v_full[b], (i >> 1) & 1, abort,
-                                        status, 66);
+                ok = wait(&bars.v_full[b], (i >> 1) & 1, 66);
                 for (int kh = 0; kh < 2 && ok; ++kh) {
-                    ok = mbar_wait_or_abort(&bars.phi_full[kh], i & 1, abort,
-                                            status, 65);
+                    ok = wait(&bars.phi_full[kh], i & 1, 65);
                     if (!ok) break;
                     tc_fence_after();
-                    for (int k = 4 * kh; k < 4 * kh + 4; ++k)  // 16 keys each
-                        mma_ss(t,
-                               smem_desc(sV0 + b * tileB + k * 2048, 16384,
-                                         1024),
-                               smem_desc(sPhi + k * 2048, 16384, 1024), id_b,
-                               (i > 0 || k > 0) ? 1u : 0u);
-                    mma_commit(&bars.phi_empty[kh]);
+                    const uint64_t da = smem_desc(sV0 + b * tileB + kh * 8192,
+                                                  16384, 1024),
+                                   db = smem_desc(sPhi + kh * 8192, 16384,
+                                                  1024);
+                    const uint32_t more = i > 0 || kh > 0;
+                    if (el) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)  // 16 keys each
+                            mma_ss(t, desc_at(da, k * 2048),
+                                   desc_at(db, k * 2048), id_b,
+                                   k > 0 ? 1u : more);
+                        mma_commit(&bars.phi_empty[kh]);
+                    }
                 }
                 if (!ok) break;
-                mma_commit(&bars.v_empty[b]);
+                if (el) mma_commit(&bars.v_empty[b]);
                 if (i + 2 < ntiles) {
                     // the features of tile i have read projection buffer b
-                    ok = mbar_wait_or_abort(&bars.k_full[b],
-                                            ((i + 2) >> 1) & 1, abort, status,
-                                            64);
+                    ok = wait(&bars.k_full[b], ((i + 2) >> 1) & 1, 64);
                     if (!ok) break;
                     tc_fence_after();
                     proj(i + 2);
                 }
             }
-            if (ok) mma_commit(&bars.done);
+            if (ok && el) mma_commit(&bars.done);
         }
         __syncwarp();
     } else if (warp >= 10) {

@@ -318,7 +318,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 __syncwarp();
                 ++hc;
             }
-        } else if (lane_id == 0 && ntiles > 0) {
+        } else if (ntiles > 0) {
             // ------------------------------------------------------ MMA issue
             // Event driven: each round issues whichever MMA group is ready,
             // the oldest tile's first (Phi'B, then P V, then the next
@@ -329,6 +329,17 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             const uint32_t id_sp = idesc_bf16(128, NR, false, false);
             const uint32_t id_s = idesc_bf16(128, nk, false, false);
             const uint32_t id_o = idesc_bf16(128, d, false, true);
+            // The whole warp runs the loop, so that its state and the
+            // operands' descriptors are warp-uniform; one lane issues. (One
+            // thread alone took about 2 K clocks to issue a group.)
+            const bool el = elect_one();
+            auto test = [&](uint64_t *bar, uint32_t par) -> bool {
+                return __all_sync(0xffffffffu, mbar_test(bar, par));
+            };
+            const uint64_t dQ = smem_desc(sQ, 16, 1024),
+                           dKW = smem_desc(sKW, 16, 1024),
+                           dV = smem_desc(sV0, (uint32_t)nk * 128, 1024),
+                           dB = smem_desc(sB, (uint32_t)r * 128, 1024);
             int us = 0, up = 0, i2 = 0;  // next unit for S, unit for P V, tile
                                          // for Phi'B
             int tiles_pv = 0;            // tiles whose last P V is issued
@@ -345,18 +356,21 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 if (i2 < tiles_pv) {
                     const int s = i2 & 1;
                     const uint32_t so = tm + 256u * s;
-                    if (mbar_test(&bars.phi_full[s], (i2 >> 1) & 1)) {
+                    if (test(&bars.phi_full[s], (i2 >> 1) & 1)) {
                         tc_fence_after();
-                        for (int kk = 0; kk < r / 16; ++kk)  // O += Phi' B
-                            mma_ts(so + nk,
-                                   so + (kk < 8 ? quarter_col(kk, 32)
-                                                : quarter_col(kk - 8, 0)),
-                                   smem_desc(sB + kk * 2048,
-                                             (uint32_t)r * 128, 1024),
-                                   id_o, 1);
-                        mma_commit(&bars.o_full[s]);
-                        if (i2 == ntiles - 1 || p2 == tph - 1)
-                            mma_commit(&bars.head_done);
+                        if (el) {
+#pragma unroll
+                            for (int kk = 0; kk < 16; ++kk)
+                                if (16 * kk < r)  // O += Phi' B
+                                    mma_ts(so + nk,
+                                           so + (kk < 8
+                                                     ? quarter_col(kk, 32)
+                                                     : quarter_col(kk - 8, 0)),
+                                           desc_at(dB, kk * 2048), id_o, 1);
+                            mma_commit(&bars.o_full[s]);
+                            if (i2 == ntiles - 1 || p2 == tph - 1)
+                                mma_commit(&bars.head_done);
+                        }
                         ++i2;
                         p2 = adv(p2);
                         did = true;
@@ -368,18 +382,20 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                     const int su = (t >> 1) * NPASS + pass;  // unit in slot
                     const int vb = up % VS;
                     const uint32_t so = tm + 256u * s;
-                    if (mbar_test(&bars.p_full[s], su & 1) &&
-                        mbar_test(&bars.v_full[vb], up / VS & 1)) {
+                    if (test(&bars.p_full[s], su & 1) &&
+                        test(&bars.v_full[vb], up / VS & 1)) {
                         fence_proxy_async_smem();  // cp.async data -> MMA
                         tc_fence_after();
-                        const uint32_t sV = sV0 + vb * tileB;
-                        for (int kk = 0; kk < nk / 16; ++kk)  // O (+)= P V
-                            mma_ts(so + nk, so + quarter_col(kk, 0),
-                                   smem_desc(sV + kk * 2048, (uint32_t)nk * 128,
-                                             1024),
-                                   id_o, pass > 0 || kk > 0);
-                        mma_commit(&bars.pv_done[s]);
-                        if (NPASS > 1) mma_commit(&bars.v_empty[vb]);
+                        const uint64_t bv = desc_at(dV, vb * tileB);
+                        if (el) {
+#pragma unroll
+                            for (int kk = 0; kk < nk / 16; ++kk)  // O (+)= P V
+                                mma_ts(so + nk, so + quarter_col(kk, 0),
+                                       desc_at(bv, kk * 2048), id_o,
+                                       pass > 0 || kk > 0);
+                            mma_commit(&bars.pv_done[s]);
+                            if (NPASS > 1) mma_commit(&bars.v_empty[vb]);
+                        }
                         if (pass == NPASS - 1) ++tiles_pv;
                         ++up;
                         did = true;
@@ -393,32 +409,38 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 if (us < nunits && !(nh && ts > 0 && i2 < ts)) {
                     const int s = ts & 1, qb = us % QS;
                     const uint32_t so = tm + 256u * s;
-                    bool ready = mbar_test(&bars.qk_full[qb], us / QS & 1);
+                    bool ready = test(&bars.qk_full[qb], us / QS & 1);
                     if (ready && spass == 0)
-                        ready = (ts < 2 || mbar_test(&bars.tmem_empty[s],
+                        ready = (ts < 2 || test(&bars.tmem_empty[s],
                                                      ((ts >> 1) - 1) & 1)) &&
-                                (!nh || mbar_test(&bars.wb_full, hc & 1));
+                                (!nh || test(&bars.wb_full, hc & 1));
                     if (ready && spass > 0)  // S columns hold P of pass - 1
-                        ready = mbar_test(
+                        ready = test(
                             &bars.pv_done[s],
                             ((ts >> 1) * NPASS + spass - 1) & 1);
                     if (ready) {
                         if (nh) ++hc;
                         fence_proxy_async_smem();  // cp.async data -> MMA
                         tc_fence_after();
-                        for (int kk = 0; kk < d / 16; ++kk) {
-                            uint32_t oq = (kk >> 2) * 128 * 128 + (kk & 3) * 32;
-                            uint32_t okw = (kk >> 2) * NR * 128 + (kk & 3) * 32;
-                            // pass 0: scores and projections (N = NR);
-                            // later passes: scores only
-                            mma_ss(so,
-                                   smem_desc(sQ + qb * tileB + oq, 16, 1024),
-                                   smem_desc(sKW + qb * tileKW + okw, 16,
-                                             1024),
-                                   spass == 0 ? id_sp : id_s, kk > 0);
+                        const uint64_t qd = desc_at(dQ, qb * tileB),
+                                       kd = desc_at(dKW, qb * tileKW);
+                        // pass 0: scores and projections (N = NR); later
+                        // passes: scores only
+                        const uint32_t id = spass == 0 ? id_sp : id_s;
+                        if (el) {
+#pragma unroll
+                            for (int kk = 0; kk < 8; ++kk)
+                                if (16 * kk < d)
+                                    mma_ss(so,
+                                           desc_at(qd, (kk >> 2) * 16384 +
+                                                           (kk & 3) * 32),
+                                           desc_at(kd, (uint32_t)(kk >> 2) *
+                                                               NR * 128 +
+                                                           (kk & 3) * 32),
+                                           id, kk > 0);
+                            mma_commit(&bars.s_full[s]);
+                            mma_commit(&bars.qk_empty[qb]);
                         }
-                        mma_commit(&bars.s_full[s]);
-                        mma_commit(&bars.qk_empty[qb]);
                         ++us;
                         if (spass == NPASS - 1) ps = adv(ps);
                         did = true;
@@ -427,13 +449,13 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 if (did) {
                     idle = 0;
                 } else if ((++idle & 255u) == 0) {
-                    if (*abort) break;
                     if (idle == 256u) t_last = global_ns();
-                    if (global_ns() - t_last > kWaitLimitNs) {
+                    const bool late = global_ns() - t_last > kWaitLimitNs;
+                    if (late) {
                         *abort = 1;
                         record_timeout(status, 41);
-                        break;
                     }
+                    if (__any_sync(0xffffffffu, late || *abort)) break;
                 }
             }
         }
