@@ -704,9 +704,21 @@ __global__ void __launch_bounds__(kCaThreads, 1)
 //   MMA  Num += P V
 //   CUDA O_lr = Num / L / (Den / L + eps), then Eq. (5)-(6) with the
 //        sparse branch's (O_s, log d_s).
-// TMEM: U_Q [0, 64), U_K [64, 128), S [128, 256), Num [256, 256 + D).
+// TMEM: U_Q [0, 64), U_K [64, 128), then S [0, 128) over them (the
+// projections of every group are in registers by then), Num [128, 128 + D).
+//
+// What bounds it: the chain of loads, products and CUDA steps of a chunk;
+// HBM would take 155 us at the size below. So two CTAs share an SM: one
+// operand buffer X serves the planes, sB_n group by group, V and half of the
+// sparse result in turn, which leaves 98 KB of shared memory and 256 TMEM
+// columns per CTA. With everything loaded at the start (193 KB, one CTA per
+// SM): 292 us at B2 H16 N16384 d128 L16; now RACE_US.
 template <int D, int L>
-__global__ void __launch_bounds__(kCaThreads, 1)
+constexpr int kRaceX =  // bytes of operand buffer X
+    D * 2 * (L * 4 > 128 ? L * 4 : 128);
+
+template <int D, int L>
+__global__ void __launch_bounds__(kCaThreads, 2)
     k_causal_race_tc(const uint16_t *__restrict__ qx,
                      const uint16_t *__restrict__ kx,
                      const uint16_t *__restrict__ vx,
@@ -743,10 +755,9 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     const uint32_t base = align1k(smem_u32(smem_raw));
     const uint32_t sQ = base;            // Q, then phi_Q of a group, then P
     const uint32_t sK = sQ + 32768;      // K, then phi_K of a group
-    const uint32_t sB = sK + 32768;      // sB_n [r x D]
-    const uint32_t sV = sB + (uint32_t)r * D * 2;
-    const uint32_t sW = sV + kTileB;     // [Lg_pad x D]
-    const uint32_t sAo = sW + (uint32_t)Lg_pad * D * 2;  // fp32 sA_n [r]
+    const uint32_t sX = sK + 32768;      // W [Lg_pad x D], sB_n of a group
+                                         // [RB x D], V [128 x D], RO
+    const uint32_t sAo = sX + align1k((uint32_t)kRaceX<D, L>);  // sA_n [r]
     const float *sAf =
         reinterpret_cast<const float *>(smem_raw + (sAo - smem_u32(smem_raw)));
 
@@ -755,14 +766,13 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     const int h = bh % H;
     const size_t row0 = (size_t)bh * N + (size_t)n * 128;
 
-    if (warp == 0) tmem_alloc(&tbase, 512);
+    if (warp == 0) tmem_alloc(&tbase, 256);
     if (tid == 0) {
         mbar_init(&mma_bar, 1);
         abort_flag = 0;
         fence_mbar_init();
     }
-    // two copy groups: what the projections and features need (Q, K,
-    // planes, sA_n), then what the products after them need (V, sB_n)
+    // what the projections and features need: Q, K, planes, sA_n
     for (int i = tid; i < 128 * (D / 8); i += kCaThreads) {
         const int rr = i / (D / 8), c = i % (D / 8);
         const size_t o = (row0 + rr) * D + c * 8;
@@ -771,24 +781,41 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     }
     for (int i = tid; i < Lg_pad * (D / 8); i += kCaThreads) {
         const int rr = i / (D / 8), c = i % (D / 8);
-        cp_async16(sW + panel_offset(rr, c, Lg_pad),
+        cp_async16(sX + panel_offset(rr, c, Lg_pad),
                    w_bf16 + ((size_t)h * Lg_pad + rr) * D + c * 8);
     }
     const size_t cidx = (size_t)bh * nc + n;
     for (int i = tid; i < r / 4; i += kCaThreads)
         cp_async16(sAo + 16 * i, sAg + cidx * r + 4 * i);
     cp_async_commit();
-    for (int i = tid; i < 128 * (D / 8); i += kCaThreads) {
-        const int rr = i / (D / 8), c = i % (D / 8);
-        cp_async16(sV + panel_offset(rr, c, 128), vx + (row0 + rr) * D + c * 8);
-    }
-    for (int i = tid; i < r * (D / 8); i += kCaThreads) {
-        const int rr = i / (D / 8), c = i % (D / 8);
-        cp_async16(sB + panel_offset(rr, c, r),
-                   sBh + (cidx * r + rr) * D + c * 8);
-    }
-    cp_async_commit();
-    cp_async_wait<1>();
+    // sB_n of group g, V, and 32 columns of each half's sparse result (fp32
+    // rows of 256 bytes at `dst`, 16-byte chunk c of row i at c ^ (i & 7))
+    auto load_b = [&](int g) {
+        for (int i = tid; i < RB * (D / 8); i += kCaThreads) {
+            const int rr = i / (D / 8), c = i % (D / 8);
+            cp_async16(sX + panel_offset(rr, c, RB),
+                       sBh + (cidx * r + g * RB + rr) * D + c * 8);
+        }
+        cp_async_commit();
+    };
+    auto load_v = [&] {
+        for (int i = tid; i < 128 * (D / 8); i += kCaThreads) {
+            const int rr = i / (D / 8), c = i % (D / 8);
+            cp_async16(sX + panel_offset(rr, c, 128),
+                       vx + (row0 + rr) * D + c * 8);
+        }
+        cp_async_commit();
+    };
+    auto load_ro = [&](uint32_t dst, int c0) {
+        for (int i = tid; i < 128 * 16; i += kCaThreads) {
+            const int rr = i / 16, c = i % 16;
+            cp_async16(dst + rr * 256 + ((c ^ (rr & 7)) << 4),
+                       RO + (row0 + rr) * D + (c >> 3) * DH + c0 +
+                           (c & 7) * 4);
+        }
+        cp_async_commit();
+    };
+    cp_async_wait<0>();
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -812,25 +839,31 @@ __global__ void __launch_bounds__(kCaThreads, 1)
         for (int k = 0; k < D / 16; ++k) {
             const uint32_t oa = (k >> 2) * 16384 + (k & 3) * 32;
             const uint64_t bw =
-                smem_desc(sW + (k >> 2) * Lg_pad * 128 + (k & 3) * 32, 16,
+                smem_desc(sX + (k >> 2) * Lg_pad * 128 + (k & 3) * 32, 16,
                           1024);
             mma_ss(tm, smem_desc(sQ + oa, 16, 1024), bw, id, k > 0);
             mma_ss(tm + 64, smem_desc(sK + oa, 16, 1024), bw, id, k > 0);
         }
     }
     ok = mma_done(130);
+    load_b(0);  // the planes are consumed
+    // every group's projections (S goes over them): group g's are the TMEM
+    // columns [32 g, 32 g + RB / 4); with 128 buckets per group each half's
+    // 16 columns load alone, with 64 the two halves share one load
+    uint32_t uq[NG][16], uk[NG][16];
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        const uint32_t c0 = 32 * g + (RB == 128 ? 16 * half : 0);
+        tmem_ld16(tm + lane + c0, uq[g]);
+        tmem_ld16(tm + lane + 64 + c0, uk[g]);
+    }
+    tmem_wait_ld();
 
     float den_inter = 0.0f;
-    for (int g = 0; g < NG && ok; ++g) {
-        // features of this thread's tables in group g (the group's
-        // projections are TMEM columns [32 g, 32 g + RB / 4); with 128
-        // buckets per group each half's 16 columns load alone, with 64 the
-        // two halves share one 16-column load)
-        uint32_t uq[16], uk[16];
-        const uint32_t c0 = 32 * g + (RB == 128 ? 16 * half : 0);
-        tmem_ld16(tm + lane + c0, uq);
-        tmem_ld16(tm + lane + 64 + c0, uk);
-        tmem_wait_ld();
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+        if (!ok) break;
+        // features of this thread's tables in group g
         auto pick = [&](const uint32_t(&u)[16], int i) -> float {
             if (RB == 128) return __uint_as_float(u[i]);
             return __uint_as_float(half ? u[(8 + i) & 15] : u[i]);
@@ -845,11 +878,11 @@ __global__ void __launch_bounds__(kCaThreads, 1)
             for (int bb = 0; bb < G; ++bb) {
                 spq[bb] = fmaf(0.5f,
                                tanh_approx(beta * tanh_approx(
-                                                      pick(uq, t * G + bb))),
+                                                      pick(uq[g], t * G + bb))),
                                0.5f);
                 spk[bb] = fmaf(0.5f,
                                tanh_approx(beta * tanh_approx(
-                                                      pick(uk, t * G + bb))),
+                                                      pick(uk[g], t * G + bb))),
                                0.5f);
             }
             float pq[R], pk[R];
@@ -864,7 +897,7 @@ __global__ void __launch_bounds__(kCaThreads, 1)
             st_shared_bf16x8(sK + panel_offset(row, col / 8, 128), pk);
             st_shared_bf16x8(sK + panel_offset(row, col / 8 + 1, 128), pk + 8);
         }
-        if (g == 0) cp_async_wait<0>();  // V and sB_n
+        cp_async_wait<0>();  // sB_n of the group
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
@@ -875,28 +908,21 @@ __global__ void __launch_bounds__(kCaThreads, 1)
 #pragma unroll
             for (int k = 0; k < RB / 16; ++k) {
                 const uint32_t oa = (k >> 2) * 16384 + (k & 3) * 32;
-                mma_ss(tm + 128, smem_desc(sQ + oa, 16, 1024),
+                mma_ss(tm, smem_desc(sQ + oa, 16, 1024),
                        smem_desc(sK + oa, 16, 1024), id_s, (g > 0 || k > 0));
-                mma_ss(tm + 256, smem_desc(sQ + oa, 16, 1024),
-                       smem_desc(sB + (uint32_t)(g * RB + 16 * k) * 128,
-                                 (uint32_t)r * 128, 1024),
+                mma_ss(tm + 128, smem_desc(sQ + oa, 16, 1024),
+                       smem_desc(sX + (uint32_t)(16 * k) * 128,
+                                 (uint32_t)RB * 128, 1024),
                        id_n, (g > 0 || k > 0));
             }
         }
         ok = mma_done(131);
+        if (ok && g + 1 < NG) load_b(g + 1);
     }
 
-    // the sparse result of the chunk's rows into the consumed sB_n space
-    // (fp32 rows, 16-byte chunk c of row i at c ^ (i & 7)), read back by
-    // the epilogue; with r < 256 the epilogue reads it from global memory
-    constexpr bool kStageRO = r >= 256;
-    if (kStageRO && ok) {
-        for (int i = tid; i < 128 * (D / 4); i += kCaThreads) {
-            const int rr = i / (D / 4), c = i % (D / 4);
-            cp_async16(sB + rr * (D * 4) + ((c ^ (rr & 7)) << 4),
-                       RO + (row0 + rr) * D + c * 4);
-        }
-        cp_async_commit();
+    if (ok) {
+        load_v();         // over sB_n, consumed
+        load_ro(sK, 0);   // over phi_K, consumed
     }
 
     // ---- P = tril(S): row i keeps keys j <= i of the chunk
@@ -904,11 +930,11 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     if (ok) {
         float s[64];
         uint32_t v[32];
-        tmem_ld32(tm + lane + 128 + 64 * half, v);
+        tmem_ld32(tm + lane + 64 * half, v);
         tmem_wait_ld();
 #pragma unroll
         for (int j = 0; j < 32; ++j) s[j] = __uint_as_float(v[j]);
-        tmem_ld32(tm + lane + 128 + 64 * half + 32, v);
+        tmem_ld32(tm + lane + 64 * half + 32, v);
         tmem_wait_ld();
 #pragma unroll
         for (int j = 0; j < 32; ++j) s[32 + j] = __uint_as_float(v[j]);
@@ -921,6 +947,7 @@ __global__ void __launch_bounds__(kCaThreads, 1)
         for (int q = 0; q < 8; ++q)
             st_shared_bf16x8(sQ + panel_offset(row, 8 * half + q, 128),
                              s + 8 * q);
+        cp_async_wait<1>();  // V
         fence_proxy_async_smem();
         tc_fence_before();
     }
@@ -931,15 +958,11 @@ __global__ void __launch_bounds__(kCaThreads, 1)
         const uint32_t id = idesc_bf16(128, D, false, true);
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-            mma_ss(tm + 256,
+            mma_ss(tm + 128,
                    smem_desc(sQ + (k >> 2) * 16384 + (k & 3) * 32, 16, 1024),
-                   smem_desc(sV + k * 2048, 16384, 1024), id, 1u);
+                   smem_desc(sX + k * 2048, 16384, 1024), id, 1u);
     }
     if (ok) ok = mma_done(132);
-    if (kStageRO) {
-        cp_async_wait<0>();
-        __syncthreads();
-    }
 
     if (ok) {
         const float invL = 1.0f / (float)L;
@@ -952,29 +975,30 @@ __global__ void __launch_bounds__(kCaThreads, 1)
         const float gl = gates ? gates[2 * tok + 1] : 1.0f;
         const float mm = fusion_multiplier(log_ds, lam, den, eps, mode);
         const float cs = gs * mm, cl = gl * invL * rl;
-        const float4 *os =
-            reinterpret_cast<const float4 *>(RO + tok * D + half * DH);
         uint16_t *o = ox + tok * D + half * DH;
 #pragma unroll
         for (int c = 0; c < DH; c += 32) {
+            // this round's RO columns; the next round's over V, consumed
+            if (c + 32 < DH) {
+                load_ro(sX, c + 32);
+                cp_async_wait<1>();
+            } else {
+                cp_async_wait<0>();
+            }
+            __syncthreads();
+            const unsigned char *rb = smem_raw +
+                                      ((c ? sX : sK) - smem_u32(smem_raw)) +
+                                      row * 256;
             uint32_t v[32];
-            tmem_ld32(tm + lane + 256 + half * DH + c, v);
+            tmem_ld32(tm + lane + 128 + half * DH + c, v);
             tmem_wait_ld();
 #pragma unroll
             for (int j = 0; j < 32; j += 8) {
-                float4 s0, s1;
-                if (kStageRO) {
-                    const int c0 = (half * DH + c + j) / 4;  // 16-byte chunk
-                    const unsigned char *rb =
-                        smem_raw + (sB - smem_u32(smem_raw)) + row * (D * 4);
-                    s0 = *reinterpret_cast<const float4 *>(
-                        rb + ((c0 ^ (row & 7)) << 4));
-                    s1 = *reinterpret_cast<const float4 *>(
-                        rb + (((c0 + 1) ^ (row & 7)) << 4));
-                } else {
-                    s0 = os[(c + j) / 4];
-                    s1 = os[(c + j) / 4 + 1];
-                }
+                const int ch = 8 * half + j / 4;  // 16-byte chunk
+                const float4 s0 = *reinterpret_cast<const float4 *>(
+                    rb + ((ch ^ (row & 7)) << 4));
+                const float4 s1 = *reinterpret_cast<const float4 *>(
+                    rb + (((ch + 1) ^ (row & 7)) << 4));
                 const float sv[8] = {s0.x, s0.y, s0.z, s0.w,
                                      s1.x, s1.y, s1.z, s1.w};
                 float y[8];
@@ -1002,9 +1026,10 @@ __global__ void __launch_bounds__(kCaThreads, 1)
             if (m_out) m_out[tok] = mm;
         }
     }
+    cp_async_wait<0>();
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    if (warp == 0) tmem_dealloc(tm, 256);
 }
 
 }  // namespace
@@ -1024,9 +1049,7 @@ bool causal_tc_supported(const Plan &P, int n_leaf) {
 size_t causal_attn_smem(int d) { return 1024 + (size_t)3 * 128 * d * 2; }
 
 size_t causal_race_smem(const Plan &P) {
-    const size_t lg_pad = ((size_t)P.L * 4 + 15) / 16 * 16;
-    return 1024 + 65536 + (size_t)P.r * P.d * 2 + (size_t)128 * P.d * 2 +
-           lg_pad * P.d * 2 + (size_t)P.r * 4;
+    return 1024 + 65536 + (size_t)128 * P.d * 2 + (size_t)P.r * 4;
 }
 
 cudaError_t launch_seg_sort(const Plan &P, int Lv, const uint32_t *keyrank,
@@ -1123,9 +1146,9 @@ cudaError_t launch_causal_race(const Plan &P, const void *q, const void *k,
                                void *o, float *log_ds, float *dlr, float *m,
                                DeviceStatus *status, cudaStream_t st) {
     const int blocks = P.BH * (P.N / 128);
-    // one CTA per SM (it holds all 512 TMEM columns)
+    // at most two CTAs per SM (each holds 256 TMEM columns)
     size_t smem = causal_race_smem(P);
-    if (smem < kSmemPerSM / 2 + 1024) smem = kSmemPerSM / 2 + 1024;
+    if (smem < kSmemPerSM / 3 + 1024) smem = kSmemPerSM / 3 + 1024;
     auto launch = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
