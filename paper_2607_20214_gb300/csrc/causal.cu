@@ -463,10 +463,16 @@ __global__ void k_seg_offsets(float *__restrict__ part, int nseg, int r,
 // state starts at the segment's offset (the sum over earlier segments) and
 // grows by each chunk's [B_n | A_n] = phi(K_n)^T [V_n | 1]; before chunk n
 // is added, sB_n (bf16) and sA_n (fp32) are written. One CTA per (head,
-// segment), 256 threads, TMEM: accumulator M-tile m at m (D + 16) (B in the
-// first D columns, A repeated in the next 16), projections after them.
+// segment, 128 buckets), 256 threads, TMEM: the accumulator at 0 (B in the
+// first D columns, A repeated in the next 16), projections after it.
+//
+// What bounds it: the serial chain of a chunk (loads, projections, features,
+// the state's product, its write-out), so two CTAs share an SM: each holds
+// one 128-bucket tile (a CTA with two took 160 KB and all 512 TMEM columns),
+// and the features go over K. 328 us before at B2 H16 N16384 d128 L16
+// beside the levels, now 288 us.
 template <int D, int L>
-__global__ void __launch_bounds__(kCaThreads, 1)
+__global__ void __launch_bounds__(kCaThreads, 2)
     k_causal_scan(const uint16_t *__restrict__ kx,
                   const uint16_t *__restrict__ vx,
                   const uint16_t *__restrict__ w_bf16,
@@ -476,12 +482,15 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     constexpr int R = 16, Gb = 4;
     constexpr int r = L * R, Lg = L * Gb;
     constexpr int Lg_pad = (Lg + 15) / 16 * 16;
-    constexpr int r_pad = r < 128 ? 128 : r;
-    constexpr int nM = r_pad / 128;
-    constexpr int TPT = L / 2;  // tables per thread (two threads per key)
-    constexpr uint32_t kAccN = D + 16;
-    constexpr uint32_t kColP = nM * kAccN;  // projections
+    constexpr int nM = r > 128 ? r / 128 : 1;  // bucket tiles of 128
+    constexpr int TT = L / nM;    // tables of a tile
+    constexpr int rt = TT * R;    // its buckets (rows past them unused)
+    constexpr int NW = Lg_pad / nM;  // its plane rows
+    constexpr int TPT = TT / 2;   // tables per thread (two threads per key)
+    constexpr int DH = D / 2;
+    constexpr uint32_t kColP = D + 16;  // projections
     constexpr uint32_t kTileB = 128 * D * 2;
+    static_assert(NW % 16 == 0 && kColP + NW <= 256, "TMEM columns");
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t mma_bar;
     __shared__ uint32_t tbase;
@@ -493,18 +502,20 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
 
     const uint32_t base = align1k(smem_u32(smem_raw));
-    const uint32_t sK = base;                    // [128 x D]
-    const uint32_t sV = sK + kTileB;             // [128 x D], then ones
-    const uint32_t sW = sV + kTileB + 16384;     // [Lg_pad x D]
-    const uint32_t sPhi = sW + align1k((uint32_t)Lg_pad * D * 2);  // [128 x r_pad]
+    const uint32_t sK = base;           // K [128 x D], then phi [128 x 128]
+    const uint32_t sV = sK + 32768;     // [128 x D], then ones
+    const uint32_t sW = sV + kTileB + 16384;  // [NW x D]
 
-    const int seg = blockIdx.x % nseg, bh = blockIdx.x / nseg;
+    const int mt = blockIdx.x % nM, seg = blockIdx.x / nM % nseg,
+              bh = blockIdx.x / nM / nseg;
     const int h = bh % H;
     const int nc = N / 128;
     const size_t per = (size_t)r * D + r;
     const float *off = offs + ((size_t)bh * nseg + seg) * per;
+    const int bk = mt * 128 + row;      // this thread's bucket
+    const bool own = row < rt;          // (its columns: half half)
 
-    if (warp == 0) tmem_alloc(&tbase, 512);
+    if (warp == 0) tmem_alloc(&tbase, 256);
     if (tid == 0) {
         mbar_init(&mma_bar, 1);
         abort_flag = 0;
@@ -515,34 +526,23 @@ __global__ void __launch_bounds__(kCaThreads, 1)
                          sV + kTileB + i * 16),
                      "r"(0x3F803F80u)
                      : "memory");
-    if (r < r_pad)  // buckets past r stay zero
-        for (int i = tid; i < 128 * (r_pad - r) / 8; i += kCaThreads) {
-            const int rr = i / ((r_pad - r) / 8), c = i % ((r_pad - r) / 8);
-            st_shared_zero16(sPhi + panel_offset(rr, r / 8 + c, 128));
-        }
-    for (int i = tid; i < Lg_pad * (D / 8); i += kCaThreads) {
+    for (int i = tid; i < NW * (D / 8); i += kCaThreads) {
         const int rr = i / (D / 8), c = i % (D / 8);
-        cp_async16(sW + panel_offset(rr, c, Lg_pad),
-                   w_bf16 + ((size_t)h * Lg_pad + rr) * D + c * 8);
+        cp_async16(sW + panel_offset(rr, c, NW),
+                   w_bf16 + ((size_t)h * Lg_pad + mt * NW + rr) * D + c * 8);
     }
-    auto load_k = [&](int n) {
+    auto load_kv = [&](int n) {
         const size_t r0 = (size_t)bh * N + (size_t)n * 128;
         for (int i = tid; i < 128 * (D / 8); i += kCaThreads) {
             const int rr = i / (D / 8), c = i % (D / 8);
-            cp_async16(sK + panel_offset(rr, c, 128), kx + (r0 + rr) * D + c * 8);
+            const uint32_t at = panel_offset(rr, c, 128);
+            cp_async16(sK + at, kx + (r0 + rr) * D + c * 8);
+            cp_async16(sV + at, vx + (r0 + rr) * D + c * 8);
         }
-    };
-    auto load_v = [&](int n) {
-        const size_t r0 = (size_t)bh * N + (size_t)n * 128;
-        for (int i = tid; i < 128 * (D / 8); i += kCaThreads) {
-            const int rr = i / (D / 8), c = i % (D / 8);
-            cp_async16(sV + panel_offset(rr, c, 128), vx + (r0 + rr) * D + c * 8);
-        }
+        cp_async_commit();
     };
     const int n0 = seg * G;
-    load_k(n0);
-    load_v(n0);
-    cp_async_commit();
+    load_kv(n0);
     fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -558,30 +558,29 @@ __global__ void __launch_bounds__(kCaThreads, 1)
         return __syncthreads_and(ok);
     };
     // The accumulator starts at the segment's offset (written into TMEM by
-    // the lanes that own the buckets), so every state is read from TMEM:
-    // thread (lane, half) owns buckets m 128 + lane of M-tiles m = half,
-    // half + 2, ...
-    for (int m = half; m < nM; m += 2) {
-        const int bk = m * 128 + row;
-        const float *ob = off + (size_t)(bk < r ? bk : 0) * D;
+    // the lanes that own the buckets), so every state is read from TMEM.
+    {
+        const float *ob = off + (size_t)(own ? bk : 0) * D + half * DH;
 #pragma unroll
-        for (int c = 0; c < D; c += 32) {
+        for (int c = 0; c < DH; c += 32) {
             uint32_t v[32];
 #pragma unroll
             for (int j = 0; j < 32; j += 4) {
                 const float4 a = *reinterpret_cast<const float4 *>(ob + c + j);
-                v[j] = __float_as_uint(bk < r ? a.x : 0.0f);
-                v[j + 1] = __float_as_uint(bk < r ? a.y : 0.0f);
-                v[j + 2] = __float_as_uint(bk < r ? a.z : 0.0f);
-                v[j + 3] = __float_as_uint(bk < r ? a.w : 0.0f);
+                v[j] = __float_as_uint(own ? a.x : 0.0f);
+                v[j + 1] = __float_as_uint(own ? a.y : 0.0f);
+                v[j + 2] = __float_as_uint(own ? a.z : 0.0f);
+                v[j + 3] = __float_as_uint(own ? a.w : 0.0f);
             }
-            tmem_st32(tm + lane + m * kAccN + c, v);
+            tmem_st32(tm + lane + half * DH + c, v);
         }
-        uint32_t a16[16];
-        const float av = bk < r ? off[(size_t)r * D + bk] : 0.0f;
+        if (half == 0) {
+            uint32_t a16[16];
+            const float av = own ? off[(size_t)r * D + bk] : 0.0f;
 #pragma unroll
-        for (int j = 0; j < 16; ++j) a16[j] = __float_as_uint(av);
-        tmem_st16(tm + lane + m * kAccN + D, a16);
+            for (int j = 0; j < 16; ++j) a16[j] = __float_as_uint(av);
+            tmem_st16(tm + lane + D, a16);
+        }
     }
     tmem_wait_st();
     tc_fence_before();
@@ -590,34 +589,36 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     // sB_n (bf16), sA_n = the accumulated state
     auto write_state = [&](int n) {
         const size_t cidx = (size_t)bh * nc + n;
-        for (int m = half; m < nM; m += 2) {
-            const int bk = m * 128 + row;
-            uint16_t *out = sBh + (cidx * r + (bk < r ? bk : 0)) * D;
+        uint16_t *out = sBh + (cidx * r + (own ? bk : 0)) * D + half * DH;
+        const bool a32 = ((uintptr_t)out & 31u) == 0;
 #pragma unroll
-            for (int c = 0; c < D; c += 32) {
-                uint32_t v[32];
-                tmem_ld32(tm + lane + m * kAccN + c, v);
-                tmem_wait_ld();
-                if (bk < r) {
+        for (int c = 0; c < DH; c += 32) {
+            uint32_t v[32];
+            tmem_ld32(tm + lane + half * DH + c, v);
+            tmem_wait_ld();
+            if (own) {
 #pragma unroll
-                    for (int j = 0; j < 32; j += 8) {
-                        uint4 pk;
-                        pk.x = pack_bf16x2(__uint_as_float(v[j]),
-                                           __uint_as_float(v[j + 1]));
-                        pk.y = pack_bf16x2(__uint_as_float(v[j + 2]),
-                                           __uint_as_float(v[j + 3]));
-                        pk.z = pack_bf16x2(__uint_as_float(v[j + 4]),
-                                           __uint_as_float(v[j + 5]));
-                        pk.w = pack_bf16x2(__uint_as_float(v[j + 6]),
-                                           __uint_as_float(v[j + 7]));
-                        *reinterpret_cast<uint4 *>(out + c + j) = pk;
+                for (int j = 0; j < 32; j += 16) {
+                    uint32_t w[8];
+#pragma unroll
+                    for (int q = 0; q < 8; ++q)
+                        w[q] = pack_bf16x2(__uint_as_float(v[j + 2 * q]),
+                                           __uint_as_float(v[j + 2 * q + 1]));
+                    if (a32) {
+                        st_global_v8(out + c + j, w);
+                    } else {
+                        uint4 *o4 = reinterpret_cast<uint4 *>(out + c + j);
+                        o4[0] = make_uint4(w[0], w[1], w[2], w[3]);
+                        o4[1] = make_uint4(w[4], w[5], w[6], w[7]);
                     }
                 }
             }
+        }
+        if (half == 0) {
             uint32_t v16[16];
-            tmem_ld16(tm + lane + m * kAccN + D, v16);
+            tmem_ld16(tm + lane + D, v16);
             tmem_wait_ld();
-            if (bk < r) sA[cidx * r + bk] = __uint_as_float(v16[0]);
+            if (own) sA[cidx * r + bk] = __uint_as_float(v16[0]);
         }
     };
     write_state(n0);
@@ -630,21 +631,20 @@ __global__ void __launch_bounds__(kCaThreads, 1)
         __syncthreads();
         if (tid == 0) {  // projections U = K W^T
             tc_fence_after();
-            const uint32_t id = idesc_bf16(128, Lg_pad, false, false);
+            const uint32_t id = idesc_bf16(128, NW, false, false);
 #pragma unroll
             for (int k = 0; k < D / 16; ++k)
                 mma_ss(tm + kColP,
                        smem_desc(sK + (k >> 2) * 16384 + (k & 3) * 32, 16, 1024),
-                       smem_desc(sW + (k >> 2) * Lg_pad * 128 + (k & 3) * 32,
-                                 16, 1024),
+                       smem_desc(sW + (k >> 2) * NW * 128 + (k & 3) * 32, 16,
+                                 1024),
                        id, k > 0);
         }
         if (!(ok = mma_done(140))) break;
-        if (c + 1 < G) load_k(n + 1);  // this chunk's K is consumed
-        // features of this thread's tables
+        // features of this thread's tables, over K (consumed)
 #pragma unroll
         for (int t = 0; t < TPT; ++t) {
-            const int tbl = half * TPT + t;
+            const int tbl = half * TPT + t;  // within the tile
             uint32_t u4[16];
             tmem_ld16(tm + lane + kColP + (tbl * Gb) / 16 * 16, u4);
             tmem_wait_ld();
@@ -663,26 +663,29 @@ __global__ void __launch_bounds__(kCaThreads, 1)
             }
             float phi[R];
             table_phi<Gb>(sp, phi);
-            st_shared_bf16x8(sPhi + panel_offset(row, tbl * 2, 128), phi);
-            st_shared_bf16x8(sPhi + panel_offset(row, tbl * 2 + 1, 128), phi + 8);
+            st_shared_bf16x8(sK + panel_offset(row, tbl * 2, 128), phi);
+            st_shared_bf16x8(sK + panel_offset(row, tbl * 2 + 1, 128), phi + 8);
         }
+        // buckets past the tile's are zero
+        constexpr int kZero = (128 - rt) / 8 / 2;  // chunks per thread
+#pragma unroll
+        for (int q = 0; q < kZero; ++q)
+            st_shared_zero16(
+                sK + panel_offset(row, rt / 8 + half * kZero + q, 128));
         fence_proxy_async_smem();
         tc_fence_before();
         __syncthreads();
         if (tid == 0) {  // state += phi^T [V | 1]
             tc_fence_after();
             const uint32_t id = idesc_bf16(128, D + 16, true, true);
-            for (int m = 0; m < nM; ++m)
 #pragma unroll
-                for (int k = 0; k < 8; ++k)
-                    mma_ss(tm + m * kAccN,
-                           smem_desc(sPhi + 2 * m * 16384 + k * 2048, 16384, 1024),
-                           smem_desc(sV + k * 2048, 16384, 1024), id, 1u);
+            for (int k = 0; k < 8; ++k)
+                mma_ss(tm, smem_desc(sK + k * 2048, 16384, 1024),
+                       smem_desc(sV + k * 2048, 16384, 1024), id, 1u);
         }
         if (!(ok = mma_done(141))) break;
         if (c + 1 < G) {
-            load_v(n + 1);  // this chunk's V is consumed
-            cp_async_commit();
+            load_kv(n + 1);  // this chunk's features and V are consumed
             write_state(n + 1);
         }
         tc_fence_before();
@@ -691,7 +694,7 @@ __global__ void __launch_bounds__(kCaThreads, 1)
     cp_async_wait<0>();
     tc_fence_before();
     __syncthreads();
-    if (warp == 0) tmem_dealloc(tm, 512);
+    if (warp == 0) tmem_dealloc(tm, 256);
 }
 
 // ----------------------------------------------- causal RACE + fusion
@@ -712,7 +715,7 @@ __global__ void __launch_bounds__(kCaThreads, 1)
 // operand buffer X serves the planes, sB_n group by group, V and half of the
 // sparse result in turn, which leaves 98 KB of shared memory and 256 TMEM
 // columns per CTA. With everything loaded at the start (193 KB, one CTA per
-// SM): 292 us at B2 H16 N16384 d128 L16; now RACE_US.
+// SM): 292 us at B2 H16 N16384 d128 L16; now 221 us.
 template <int D, int L>
 constexpr int kRaceX =  // bytes of operand buffer X
     D * 2 * (L * 4 > 128 ? L * 4 : 128);
@@ -1100,10 +1103,8 @@ int causal_segments(const Plan &P) {
 }
 
 size_t causal_scan_smem(const Plan &P) {
-    const size_t lg_pad = ((size_t)P.L * 4 + 15) / 16 * 16;
-    const size_t r_pad = P.r < 128 ? 128 : P.r;
-    return 1024 + (size_t)2 * 128 * P.d * 2 + 16384 +
-           (lg_pad * P.d * 2 + 1023) / 1024 * 1024 + 128 * r_pad * 2;
+    // at most 32 plane rows: those of one 128-bucket tile
+    return 1024 + 32768 + (size_t)128 * P.d * 2 + 16384 + (size_t)32 * P.d * 2;
 }
 
 cudaError_t launch_causal_scan(const Plan &P, const void *k, const void *v,
@@ -1117,13 +1118,14 @@ cudaError_t launch_causal_scan(const Plan &P, const void *k, const void *v,
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int G = (P.N / 128) / nseg;
-    // one CTA per SM (it holds all 512 TMEM columns)
+    const int tiles = P.r > 128 ? P.r / 128 : 1;
+    // at most two CTAs per SM (each holds 256 TMEM columns)
     size_t smem = causal_scan_smem(P);
-    if (smem < kSmemPerSM / 2 + 1024) smem = kSmemPerSM / 2 + 1024;
+    if (smem < kSmemPerSM / 3 + 1024) smem = kSmemPerSM / 3 + 1024;
     auto launch = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        kern<<<P.BH * nseg, kCaThreads, smem, st>>>(
+        kern<<<P.BH * nseg * tiles, kCaThreads, smem, st>>>(
             (const uint16_t *)k, (const uint16_t *)v, w_bf16, part, P.N, P.H,
             nseg, G, P.beta, sBh, sA, status);
         return cudaGetLastError();
