@@ -400,32 +400,62 @@ __global__ void __launch_bounds__(kCaThreads, 2)
         // ---- O = sum e^z V / (sum e^z + eps), log d (natural log)
         const float logd = (mrun + log2f(lrun)) * kLn2;
         const float inv = 1.0f / (lrun + eps * ex2_approx(-mrun));
+        // MergeLSE(running = diag, this = off): the row's weights and this
+        // level's O through shared memory (Q and K are consumed), so that
+        // the running rows are read and written whole, 512 contiguous bytes
+        // an instruction. With each thread updating its half row from
+        // registers, 32 rows an instruction, the two levels at B2 H16
+        // N16384 d128 took 190 us each beside the prefix states; now 130 us (and the
+        // prefix states 228 beside them, from 288).
         const size_t tok = hN + qrow_s[row];
-        float *o = RO + tok * D + half * DH;
-        float ld_new = logd;
-        float of[DH];
-#pragma unroll
-        for (int j = 0; j < DH / 2; ++j) f2unpack(o_acc[j], of[2 * j], of[2 * j + 1]);
-        // MergeLSE(running = diag, this = off)
         const float ld1 = RL[tok];
         const float mu = fmaxf(ld1, logd);
         const float w1 = __expf(ld1 - mu), w2 = __expf(logd - mu);
         const float ssum = w1 + w2;
         const float r = 1.0f / (ssum + eps);
-        const float c1 = w1 * r, c2 = w2 * inv * r;
+        if (half == 0) {
+            xm[0][row] = w1 * r;
+            xl[0][row] = w2 * inv * r;
+        }
+        // 16-byte chunk c of row i at chunk c ^ (i & 7) of its D * 4 bytes
 #pragma unroll
         for (int j = 0; j < DH; j += 4) {
-            float4 a = *reinterpret_cast<float4 *>(o + j);
-            a.x = c1 * a.x + c2 * of[j];
-            a.y = c1 * a.y + c2 * of[j + 1];
-            a.z = c1 * a.z + c2 * of[j + 2];
-            a.w = c1 * a.w + c2 * of[j + 3];
-            *reinterpret_cast<float4 *>(o + j) = a;
+            float x[4];
+            f2unpack(o_acc[j / 2], x[0], x[1]);
+            f2unpack(o_acc[j / 2 + 1], x[2], x[3]);
+            st_shared_v4(sQ + row * (D * 4) +
+                             (((half * DH + j) / 4 ^ (row & 7)) << 4),
+                         __float_as_uint(x[0]), __float_as_uint(x[1]),
+                         __float_as_uint(x[2]), __float_as_uint(x[3]));
         }
-        ld_new = mu + __logf(ssum + eps);
-        __syncthreads();  // qrow_s is rewritten by the next item; both
-                          // halves read RL before it changes
-        if (half == 0) RL[tok] = ld_new;
+        __syncthreads();  // both halves have read RL, too
+        if (half == 0) RL[tok] = mu + __logf(ssum + eps);
+        constexpr int CPR = D / 4;         // chunks of a row
+        constexpr int RPI = 32 / CPR;      // rows per instruction
+        constexpr int NI = 16 / RPI;       // instructions: 16 rows a warp
+        const int cl = lane_id % CPR, rl = warp * 16 + lane_id / CPR;
+#pragma unroll
+        for (int i0 = 0; i0 < NI; i0 += 8) {
+            float4 a[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                a[i] = reinterpret_cast<const float4 *>(
+                    RO + (hN + qrow_s[rl + (i0 + i) * RPI]) * D)[cl];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const int ri = rl + (i0 + i) * RPI;
+                const float c1 = xm[0][ri], c2 = xl[0][ri];
+                const uint4 w =
+                    ld_shared_v4(sQ + ri * (D * 4) + ((cl ^ (ri & 7)) << 4));
+                a[i].x = c1 * a[i].x + c2 * __uint_as_float(w.x);
+                a[i].y = c1 * a[i].y + c2 * __uint_as_float(w.y);
+                a[i].z = c1 * a[i].z + c2 * __uint_as_float(w.z);
+                a[i].w = c1 * a[i].w + c2 * __uint_as_float(w.w);
+                reinterpret_cast<float4 *>(
+                    RO + (hN + qrow_s[ri]) * D)[cl] = a[i];
+            }
+        }
+        __syncthreads();  // the next item rewrites qrow_s and every buffer
     }
     cp_async_wait<0>();
     tc_fence_before();
@@ -470,7 +500,7 @@ __global__ void k_seg_offsets(float *__restrict__ part, int nseg, int r,
 // the state's product, its write-out), so two CTAs share an SM: each holds
 // one 128-bucket tile (a CTA with two took 160 KB and all 512 TMEM columns),
 // and the features go over K. 328 us before at B2 H16 N16384 d128 L16
-// beside the levels, now 288 us.
+// beside the levels, now 228 us (288 before the levels' rows were merged whole).
 template <int D, int L>
 __global__ void __launch_bounds__(kCaThreads, 2)
     k_causal_scan(const uint16_t *__restrict__ kx,
