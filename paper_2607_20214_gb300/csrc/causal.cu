@@ -405,8 +405,8 @@ __global__ void __launch_bounds__(kCaThreads, 2)
         // the running rows are read and written whole, 512 contiguous bytes
         // an instruction. With each thread updating its half row from
         // registers, 32 rows an instruction, the two levels at B2 H16
-        // N16384 d128 took 190 us each beside the prefix states; now 130 us (and the
-        // prefix states 228 beside them, from 288).
+        // N16384 d128 took 190 us each beside the prefix states; now 130 us
+        // (and the prefix states 228 beside them, from 288).
         const size_t tok = hN + qrow_s[row];
         const float ld1 = RL[tok];
         const float mu = fmaxf(ld1, logd);
@@ -500,7 +500,8 @@ __global__ void k_seg_offsets(float *__restrict__ part, int nseg, int r,
 // the state's product, its write-out), so two CTAs share an SM: each holds
 // one 128-bucket tile (a CTA with two took 160 KB and all 512 TMEM columns),
 // and the features go over K. 328 us before at B2 H16 N16384 d128 L16
-// beside the levels, now 228 us (288 before the levels' rows were merged whole).
+// beside the levels; now 228 us (288 before the levels' rows were merged
+// whole).
 template <int D, int L>
 __global__ void __launch_bounds__(kCaThreads, 2)
     k_causal_scan(const uint16_t *__restrict__ kx,
@@ -745,7 +746,8 @@ __global__ void __launch_bounds__(kCaThreads, 2)
 // operand buffer X serves the planes, sB_n group by group, V and half of the
 // sparse result in turn, which leaves 98 KB of shared memory and 256 TMEM
 // columns per CTA. With everything loaded at the start (193 KB, one CTA per
-// SM): 292 us at B2 H16 N16384 d128 L16; now 205 us (221 with O in 16-byte stores).
+// SM): 292 us at B2 H16 N16384 d128 L16; now 205 us (221 with O in 16-byte
+// stores).
 template <int D, int L>
 constexpr int kRaceX =  // bytes of operand buffer X
     D * 2 * (L * 4 > 128 ? L * 4 : 128);

@@ -31,7 +31,10 @@
 // that chain: gathers have warps of their own, the two slots' products are
 // issued independently of each other, the second pass's scores go out right
 // behind the first P V product, P is handed over before the features and
-// the fusion scalars are computed, and all features go to one product.
+// the fusion scalars are computed, and all features go to one product: c4
+// (B1 H32 N65536 d128 L16) 697 -> 646 us; products issued by a converged warp
+// from descriptors made once, and a lane per relayed barrier: 584 us (0.54 of
+// the measured HBM bandwidth).
 //
 // TMEM columns of a slot (same layout in both CTAs): pass 0 scores keys
 // [0, 64) at [0, 64), the projections of row half 0's tables at [64, 96),

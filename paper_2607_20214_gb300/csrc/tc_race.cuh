@@ -221,10 +221,40 @@ __device__ __forceinline__ void write_phi_tmem(const float (&sp)[32], int l0,
     }
 }
 
+// sum_r phi_r A_r of one gamma = 4 table from its per-bit factors, bit by
+// bit from the highest: A[i] <- q A[i] + p A[i + half], all terms positive as
+// in table_dot4. Fewer operations (7 + 7 in pairs against 8 single and 12 in
+// pairs) in a longer chain: c3's block kernel took 133 us with table_dot4 and
+// 128 with this, but c2's 37 and 39, c5's 106 and 110, and c4's 584 with both.
+// A: 16 floats, 16-byte aligned, in shared memory.
+__device__ __forceinline__ float table_den4(const float *sp, const float *A) {
+    float4 a[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        a[j] = *reinterpret_cast<const float4 *>(A + 4 * j);
+    const float2 p3 = make_float2(sp[3], sp[3]),
+                 p2 = make_float2(sp[2], sp[2]),
+                 p1 = make_float2(sp[1], sp[1]);
+    const float2 q3 = make_float2(1.0f - sp[3], 1.0f - sp[3]),
+                 q2 = make_float2(1.0f - sp[2], 1.0f - sp[2]),
+                 q1 = make_float2(1.0f - sp[1], 1.0f - sp[1]);
+    auto lo = [](const float4 &x) { return make_float2(x.x, x.y); };
+    auto hi = [](const float4 &x) { return make_float2(x.z, x.w); };
+    const float2 c0 = fma2(p3, lo(a[2]), mul2(q3, lo(a[0]))),
+                 c1 = fma2(p3, hi(a[2]), mul2(q3, hi(a[0]))),
+                 c2 = fma2(p3, lo(a[3]), mul2(q3, lo(a[1]))),
+                 c3 = fma2(p3, hi(a[3]), mul2(q3, hi(a[1])));
+    const float2 b0 = fma2(p2, c2, mul2(q2, c0)),
+                 b1 = fma2(p2, c3, mul2(q2, c1));
+    const float2 t = fma2(p1, b1, mul2(q1, b0));
+    return fmaf(sp[0], t.y, (1.0f - sp[0]) * t.x);
+}
+
 // sum over tables t < nt of phi_t . A_t for the tables of one 64-bucket
 // chunk (at most TT of them; per-bit factors sp[t * G ..], A of the chunk's
-// first table at A). Four independent partial sums in acc.
-template <int G, int TT>
+// first table at A). Four independent partial sums in acc. FOLD: which of the
+// two forms gamma = 4 takes.
+template <int G, int TT, bool FOLD = false>
 __device__ __forceinline__ void chunk_den(const float *sp, int nt,
                                           const float *A, float (&acc)[4]) {
     constexpr int R = 1 << G;
@@ -232,9 +262,13 @@ __device__ __forceinline__ void chunk_den(const float *sp, int nt,
     for (int t = 0; t < TT; ++t) {
         if (t < nt) {
             if constexpr (G == 4) {
-                float u[4], w[4];
-                table_uw4(&sp[t * G], 1.0f, u, w);
-                acc[t & 3] += table_dot4(u, w, A + t * R);
+                if constexpr (FOLD) {
+                    acc[t & 3] += table_den4(&sp[t * G], A + t * R);
+                } else {
+                    float u[4], w[4];
+                    table_uw4(&sp[t * G], 1.0f, u, w);
+                    acc[t & 3] += table_dot4(u, w, A + t * R);
+                }
             } else {
                 float phi[R];
                 table_phi<G>(&sp[t * G], phi);

@@ -17,7 +17,7 @@
 //               64-bucket chunks h and h + 2. The two warps exchange row
 //               maxima and sums over a barrier of their 64 threads; nothing
 //               else synchronises the slot.
-//   warp 16     allocates tensor memory and issues every MMA (lane 0).
+//   warp 16     allocates tensor memory and issues every MMA (one lane of it).
 //   warp 17     per head, TMA loads of the bf16 RACE planes (under the key
 //               rows), the bf16 B summary and the fp32 A summary.
 //   warps 18-19 V rows; warps 20-23 Q and K rows: cp.async gathers, whole
@@ -31,12 +31,14 @@
 //
 // What bounds it: a slot's own chain of these steps, about 17 K clocks per
 // tile at d = 128 (clock traces: the next tile's scores are there when the
-// slot asks for them; two slots give a tile per 8.5 K clocks, where the
+// slot asks for them; two slots gave a tile per 8.5 K clocks, where the
 // copies need 6 K). Every step taken off the chain shows in the time: copies
 // by warps of their own, features under the P V product, barriers of 64
-// threads only. c3: 163 -> 143 us; c2: 45 -> 42; c5: 138 -> 129; c3 top-k (two
-// passes): 313 -> 263. Left on it at c3 (time without the step): Den 22 us,
-// features 15, stores 7, bit factors 5.
+// threads only (c3: 163 -> 143 us; c2: 45 -> 42; c5: 138 -> 129; c3 top-k, four
+// passes: 313 -> 263), products issued by a converged warp from descriptors
+// made once (c3: 137 -> 133; c2: 41 -> 37; c5: 126 -> 106; top-k: 263 -> 229),
+// Den folded bit by bit (c3: 133 -> 127). When c3 took 143 us, Den made up 22
+// of it, the features 15, the stores 7, the bit factors 5.
 #include "device_common.cuh"
 #include "tc_common.cuh"
 #include "tc_race.cuh"
@@ -571,11 +573,13 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 constexpr int n1 = T * G <= 16 ? 16 : 32;
                 race_factors<n1>(pr, beta, sp);
                 float dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // independent chains
-                chunk_den<G, T>(sp, nt0, Asm + ta0 * R, dacc);
+                constexpr bool fold = QS == 1;  // see table_den4
+                chunk_den<G, T, fold>(sp, nt0, Asm + ta0 * R, dacc);
                 if constexpr (T * G <= 16) {
                     if (nt1 > 0) {
                         race_factors<16>(pr + 16, beta, sp + 16);
-                        chunk_den<G, T>(sp + 16, nt1, Asm + ta1 * R, dacc);
+                        chunk_den<G, T, fold>(sp + 16, nt1, Asm + ta1 * R,
+                                              dacc);
                     }
                 }
                 den = (dacc[0] + dacc[1]) + (dacc[2] + dacc[3]);
@@ -991,8 +995,8 @@ cudaError_t launch_block_attn_ws(
     // r = 128); at d = 128 one fits. Key blocks of 32 and 64 take half and a
     // quarter of the softmax work of the masked path. Both together, B4 H12
     // N4096 d64 b64 r128: 63 -> 45 us; B8 H12 N8192: 215 -> 138 us; B3 H5
-    // N4800 d128 b64 (KB alone): 35 -> 27 us. (42, 129 and 25 us since the
-    // copies have warps of their own.)
+    // N4800 d128 b64 (KB alone): 35 -> 27 us. (37, 106 and 23 us since the
+    // copies and the products' issue do not bound them.)
     if (P.gamma == 4 && P.sel == 0 && passes == 1) {
         auto pick = [&](auto o32) {
             constexpr bool F = decltype(o32)::value;
