@@ -14,30 +14,6 @@ __device__ __forceinline__ uint32_t align1k(uint32_t x) {
     return (x + 1023u) & ~1023u;
 }
 
-// RACE planes of one head as bf16 rows [Lg_pad x d] in the panel layout;
-// rows >= Lg are zero.
-// With row0 / prows: the planes are rows [row0, row0 + Lg_pad) of a panel
-// layout of prows rows (planes stacked under a key tile).
-__device__ inline void load_planes_bf16(uint32_t dst, const float *w, int Lg,
-                                 int Lg_pad, int d, int tid, int nthreads,
-                                 int row0 = 0, int prows = 0) {
-    const int chunks = d >> 3;
-    if (prows == 0) prows = Lg_pad;
-    for (int i = tid; i < Lg_pad * chunks; i += nthreads) {
-        int row = i / chunks, c = i - row * chunks;
-        uint32_t addr = dst + panel_offset(row0 + row, c, prows);
-        if (row < Lg) {
-            const float4 *src =
-                reinterpret_cast<const float4 *>(w + (size_t)row * d + c * 8);
-            float4 a = src[0], b = src[1];
-            float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-            st_shared_bf16x8(addr, v);
-        } else {
-            st_shared_zero16(addr);
-        }
-    }
-}
-
 // Two threads share each row (warps w and w + 4 read the same TMEM lanes).
 // The RACE tables of a row are split between them at table `split`, chosen
 // so that each half's buckets start on a 32-bucket boundary (whole TMEM
@@ -68,21 +44,6 @@ __device__ __forceinline__ void race_bits32(uint32_t taddr, int ncols,
     }
 }
 
-// The per-bit factors of 16 projections already loaded from TMEM (fp32
-// bits in pr): sp[j] for j < 16, entries past `ncols` set to 1/2.
-__device__ __forceinline__ void race_factors16(const uint32_t *pr, int ncols,
-                                               float beta, float *sp) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-        if (j < ncols) {
-            float t = tanh_approx(beta * tanh_approx(__uint_as_float(pr[j])));
-            sp[j] = fmaf(0.5f, t, 0.5f);
-        } else {
-            sp[j] = 0.5f;
-        }
-    }
-}
-
 // The per-bit factors of n projections already loaded from TMEM (fp32 bits
 // in pr). Columns past the last table give values that nothing reads.
 template <int n>
@@ -93,16 +54,6 @@ __device__ __forceinline__ void race_factors(const uint32_t *pr, float beta,
         sp[j] = fmaf(0.5f,
                      tanh_approx(beta * tanh_approx(__uint_as_float(pr[j]))),
                      0.5f);
-}
-
-// race_bits32 over 16 projection columns: sp[j] for j < 16, entries past
-// `ncols` set to 1/2. The TMEM load is waited for inside.
-__device__ __forceinline__ void race_bits16(uint32_t taddr, int ncols,
-                                           float beta, float *sp) {
-    uint32_t pr[16];
-    tmem_ld16(taddr, pr);
-    tmem_wait_ld();
-    race_factors16(pr, ncols, beta, sp);
 }
 
 // Features of table l from its G per-bit factors: phi[r] = prod_b (bit b of
@@ -179,45 +130,6 @@ __device__ __forceinline__ void table_pack4(const float (&u)[4],
         const float2 b = mul2(make_float2(u[2], u[3]), wj);
         out[2 * j] = pack_bf16x2(a.x, a.y);
         out[2 * j + 1] = pack_bf16x2(b.x, b.y);
-    }
-}
-
-// Writes the pre-scaled features phi * scale of tables [l0, l1) of this
-// thread's query row, for buckets [lo, hi), as packed bf16 pairs into TMEM
-// with bucket lo at `taddr`. l0 * R and lo are multiples of 32 and hi of 16;
-// buckets go out in groups of 32 (16 columns), the last half group padded
-// with zeros.
-template <int G>
-__device__ __forceinline__ void write_phi_tmem(const float (&sp)[32], int l0,
-                                               int l1, int r, float scale,
-                                               int lo, int hi,
-                                               uint32_t taddr) {
-    constexpr int R = 1 << G;
-    uint32_t buf[16];
-#pragma unroll
-    for (int lt = 0; lt < 32 / G; ++lt) {
-        if (l0 + lt < l1) {
-            float phi[R];
-            table_phi<G>(&sp[lt * G], phi, scale);
-#pragma unroll
-            for (int q = 0; q < R; q += 2) {
-                const int prel = lt * R + q;     // even, relative to l0 * R
-                const int slot = (prel >> 1) & 15;
-                buf[slot] = pack_bf16x2(phi[q], phi[q + 1]);
-                const int p = l0 * R + prel;      // absolute bucket
-                const bool last = p + 2 == r;
-                if (slot == 15 || last) {
-                    if (last) {
-#pragma unroll
-                        for (int z = 0; z < 16; ++z)
-                            if (z > slot) buf[z] = 0u;
-                    }
-                    const int g = p - 2 * slot;  // first bucket of the group
-                    if (g >= lo && g < hi)
-                        tmem_st16(taddr + ((g - lo) >> 1), buf);
-                }
-            }
-        }
     }
 }
 
