@@ -34,7 +34,7 @@
 // slot asks for them; two slots gave a tile per 8.5 K clocks, where the
 // copies need 6 K). Every step taken off the chain shows in the time: copies
 // by warps of their own, features under the P V product, barriers of 64
-// threads only (c3: 163 -> 143 us; c2: 45 -> 42; c5: 138 -> 129; c3 top-k, four
+// threads only (c3: 163 -> 143 us; c2: 45 -> 42; c5: 138 -> 129; c3 top-k, two
 // passes: 313 -> 263), products issued by a converged warp from descriptors
 // made once (c3: 137 -> 133; c2: 41 -> 37; c5: 126 -> 106; top-k: 263 -> 229),
 // Den folded bit by bit (c3: 133 -> 127). When c3 took 143 us, Den made up 22
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             // out right behind its previous P V product (which reads P from
             // the S columns): products run in the order of their issue.
             // Waiting for that product's completion took 229 us against 226
-            // at c3 with four passes (top-k); two tiles' passes in turn, with
+            // at c3 with two passes (top-k); two tiles' passes in turn, with
             // a second query buffer, 259.
             const uint32_t id_sp = idesc_bf16(128, NR, false, false);
             const uint32_t id_s = idesc_bf16(128, nk, false, false);
