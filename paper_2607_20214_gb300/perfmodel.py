@@ -186,14 +186,16 @@ def kernel_work(wl: Workload, kernel: str) -> dict:
         simt = True
     elif kernel.startswith("topk_select"):
         # block sums (Q and K read through the sort orders), block scores,
-        # and per query the canonical fp32 chains over the c b candidate
-        # keys (each query block stages its candidates once): reads Q once
-        # and the candidate keys c times, writes the bitmask
+        # and per query the scores of the c b candidate keys (each query
+        # block stages its candidates once): reads Q once and the candidate
+        # keys c times, writes the bitmask. The scores are products on the
+        # tensor cores for bf16 with d_h of 64 or 128 and b a multiple of
+        # 128, canonical fp32 chains otherwise.
         c = getattr(wl, "topk_blocks", 1)
         by = H * (2 * N * d * e + N * d * e + c * N * d * e + N * c * wl.block
                   // 8)
         fl = H * (2 * N * c * wl.block * d + 2 * (N // wl.block) ** 2 * d)
-        simt = True
+        simt = simt or d not in (64, 128) or wl.block % 128 != 0
     elif kernel.startswith("sort_hash"):
         by = H * 2 * N * d * e
         fl = H * 4 * N * d * wl.sort_bits
