@@ -110,6 +110,7 @@ __global__ void __launch_bounds__(kBtThreads, 1)
                    float *__restrict__ dv, float *__restrict__ d_gates,
                    float *__restrict__ d_lambda, float *__restrict__ part,
                    int S_seg, DeviceStatus *status) {
+    wait_for_stream();
     constexpr int R = 16, G = 4;
     constexpr int r = L * R, Lg = L * G;
     constexpr int Lg_pad = (Lg + 15) / 16 * 16;
@@ -721,6 +722,7 @@ __global__ void __launch_bounds__(kBtThreads, 1)
                   const float *__restrict__ part, int S_seg, int blk_grid,
                   int N, int H, float beta, int tiles_per_head,
                   long total_tiles, DeviceStatus *status) {
+    wait_for_stream();
     constexpr int R = 16, G = 4;
     constexpr int r = L * R, Lg = L * G;
     constexpr int Lg_pad = (Lg + 15) / 16 * 16;
@@ -1124,13 +1126,13 @@ cudaError_t launch_bwd_block_tc(const Plan &P, const void *q, const void *k,
     auto launch = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        kern<<<grid, kBtThreads, smem, st>>>(
+        return launch_after(
+            kern, dim3(grid), kBtThreads, smem, st,
             (const uint16_t *)q, (const uint16_t *)k, (const uint16_t *)v,
             (const uint16_t *)d_o, w_bf16, Bh, A, perm_q, perm_k, lambda_tok,
             gates, P.N, P.H, P.beta, P.eps, P.scale, P.lambda, P.fusion_mode,
             tiles_per_head, total, dq, dk, dv, d_gates, d_lambda, part, S_seg,
             status);
-        return cudaGetLastError();
     };
     return P.L == 8 ? launch(k_bwd_block_tc<8>) : launch(k_bwd_block_tc<4>);
 }
@@ -1171,11 +1173,9 @@ cudaError_t launch_bwd_keys_tc(const Plan &P, const void *k, const void *v,
     auto launch = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        kern<<<grid, kBtThreads, smem, st>>>(tmK, tmV, tmDK, tmDV, w_bf16,
-                                             part, S_seg, blk_grid, P.N, P.H,
-                                             P.beta, tiles_per_head, total,
-                                             status);
-        return cudaGetLastError();
+        return launch_after(kern, dim3(grid), kBtThreads, smem, st, tmK, tmV,
+                            tmDK, tmDV, w_bf16, part, S_seg, blk_grid, P.N,
+                            P.H, P.beta, tiles_per_head, total, status);
     };
     return P.L == 8 ? launch(k_bwd_keys_tc<8>) : launch(k_bwd_keys_tc<4>);
 }

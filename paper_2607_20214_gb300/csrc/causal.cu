@@ -52,6 +52,7 @@ constexpr size_t kSmemPerSM = 233472;  // 228 KB of shared memory per SM
 __global__ void __launch_bounds__(kSegThreads)
     k_seg_sort(const uint32_t *__restrict__ keyrank, int N, int bins,
                int32_t *__restrict__ perms) {
+    wait_for_stream();
     __shared__ int cnt[256];
     __shared__ int wc[kSegWarps][256];
     const int s = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
@@ -151,9 +152,11 @@ __global__ void __launch_bounds__(kCaThreads, 2)
                      const uint16_t *__restrict__ kx,
                      const uint16_t *__restrict__ vx,
                      const int32_t *__restrict__ permq,
-                     const int32_t *__restrict__ permk, int N, int m, int b, int items, int *__restrict__ next_item,
+                     const int32_t *__restrict__ permk, int N, int m, int b,
+                     int items, int *__restrict__ next_item,
                      float scale, float eps, float *__restrict__ RO,
                      float *__restrict__ RL, DeviceStatus *status) {
+    wait_for_stream();
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t mma_bar;
     __shared__ uint32_t tbase;
@@ -1101,8 +1104,8 @@ cudaError_t launch_seg_sort(const Plan &P, int Lv, const uint32_t *keyrank,
                             int32_t *perms, cudaStream_t st) {
     if (Lv == 0) return cudaSuccess;
     dim3 grid((1u << Lv) - 1, P.BH, 2);
-    k_seg_sort<<<grid, kSegThreads, 0, st>>>(keyrank, P.N, P.bins, perms);
-    return cudaGetLastError();
+    return launch_after(k_seg_sort, grid, kSegThreads, 0, st, keyrank, P.N,
+                        P.bins, perms);
 }
 
 // SortLSH blocks of level `level` (1 = top), whose halves hold
@@ -1125,11 +1128,10 @@ cudaError_t launch_causal_attn(const Plan &P, int level, const void *q,
     auto launch = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        kern<<<grid, kCaThreads, smem, st>>>(
-            (const uint16_t *)q, (const uint16_t *)k, (const uint16_t *)v, pq,
-            pk, P.N, m, P.b, items, next_item, P.scale, P.eps, RO, RL,
-            status);
-        return cudaGetLastError();
+        return launch_after(kern, dim3(grid), kCaThreads, smem, st,
+                            (const uint16_t *)q, (const uint16_t *)k,
+                            (const uint16_t *)v, pq, pk, P.N, m, P.b, items,
+                            next_item, P.scale, P.eps, RO, RL, status);
     };
     return P.d == 128 ? launch(k_causal_attn_tc<128>)
                       : launch(k_causal_attn_tc<64>);

@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                   int segs, int items, int *__restrict__ next_item,
                   float scale, float eps, float *__restrict__ RO,
                   float *__restrict__ RL, DeviceStatus *status) {
+    wait_for_stream();
     extern __shared__ unsigned char smem_raw[];
     __shared__ CbBars bars;
     __shared__ uint32_t tbase;
@@ -446,10 +447,9 @@ cudaError_t launch_causal_base(const Plan &P, int n_leaf, const void *q,
     auto launch = [&](auto kern) {
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem);
-        kern<<<items < sms ? items : sms, kCbThreads, smem, st>>>(
-            tmQ, tmK, tmV, P.N, n_leaf, segs, items, next_item, P.scale,
-            P.eps, RO, RL, status);
-        return cudaGetLastError();
+        return launch_after(kern, dim3(items < sms ? items : sms), kCbThreads,
+                            smem, st, tmQ, tmK, tmV, P.N, n_leaf, segs, items,
+                            next_item, P.scale, P.eps, RO, RL, status);
     };
     return P.d == 128 ? launch(k_causal_base<128>) : launch(k_causal_base<64>);
 }

@@ -482,6 +482,7 @@ __global__ void __launch_bounds__(kHashTile)
                         const int *__restrict__ hist, int N, int tiles,
                         int bins, int32_t *__restrict__ perm_q,
                         int32_t *__restrict__ perm_k, DeviceStatus *status) {
+    wait_for_stream();
     __shared__ int off[kFusedScan];
     __shared__ int warp_tot[kHashTile / 32];
     const int tile = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
@@ -638,9 +639,9 @@ cudaError_t launch_sort_scatter(const Plan &P, const uint32_t *keyrank,
                                 cudaStream_t st) {
     dim3 grid(P.tiles, P.BH, 2);
     if (sort_fused(P)) {
-        k_sort_scan_scatter<<<grid, kHashTile, 0, st>>>(
-            keyrank, hist, P.N, P.tiles, P.bins, perm_q, perm_k, status);
-        return cudaGetLastError();
+        return launch_after(k_sort_scan_scatter, grid, kHashTile, 0, st,
+                            keyrank, hist, P.N, P.tiles, P.bins, perm_q,
+                            perm_k, status);
     }
     k_sort_scatter<<<grid, kHashTile, 0, st>>>(keyrank, hist, P.N, P.tiles,
                                                P.bins, perm_q, perm_k, status);
