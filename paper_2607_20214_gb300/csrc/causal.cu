@@ -1017,7 +1017,7 @@ __global__ void __launch_bounds__(kCaThreads, 2)
         const bool o_a32 = ((uintptr_t)ox & 31u) == 0;
 #pragma unroll
         for (int c = 0; c < DH; c += 32) {
-            // this round's RO columns; the next round's over V, consumed
+            // these 32 RO columns a half; the next ones go over V, consumed
             if (c + 32 < DH) {
                 load_ro(sX, c + 32);
                 cp_async_wait<1>();

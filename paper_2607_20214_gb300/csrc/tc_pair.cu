@@ -374,7 +374,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             const uint32_t id_sp = idesc_bf16(256, nk + 64, false, false);
             const uint32_t id_s = idesc_bf16(256, nk, false, false);
             const uint32_t id_o = idesc_bf16(256, d, false, true);
-            int j = 0, stage = 0;    // this round's slot (j & 1)
+            int j = 0, stage = 0;    // the slot at hand (j & 1)
             int jo = 1, stageo = 0;  // the other slot
             int done = 0, hc = 0;  // blocks finished, heads begun
             // The whole warp runs the loop, so that its state and the
