@@ -33,7 +33,7 @@
 // behind the first P V product, P is handed over before the features and
 // the fusion scalars are computed, and all features go to one product: c4
 // (B1 H32 N65536 d128 L16) 697 -> 646 us; products issued by a converged warp
-// from descriptors made once, and a lane per relayed barrier: 584 us (0.54 of
+// from descriptors made once, and a lane per relayed barrier: 587 us (0.54 of
 // the measured HBM bandwidth).
 //
 // TMEM columns of a slot (same layout in both CTAs): pass 0 scores keys
@@ -48,6 +48,7 @@
 // arrivals reach the even CTA's barriers through the relay (one remote
 // arrival per phase), the MMA completions reach both CTAs by multicast.
 #include "device_common.cuh"
+#include "pair_order.h"
 #include "tc_common.cuh"
 #include "tc_race.cuh"
 
@@ -363,25 +364,27 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             }
         } else if (nblk > 0) {
             // ------------------------------------------------- MMA issue
-            // Event driven, each slot at a stage of its own: 0 scores and
-            // projections, 1 P V of pass 0 and, right behind it, the scores
-            // of pass 1 (2; products run in the order of their issue, so
-            // they overwrite P only after its product has read it), 3 P V
-            // of pass 1, 4 the features' product. A new head's planes and
-            // summaries replace the old ones only after head_done: its
-            // first scores wait until every product of the blocks before
-            // is issued.
+            // Event driven, each slot at a stage of its own: the order is
+            // PairOrder's (pair_order.h). The scores of pass 1 go out right
+            // behind the P V product of pass 0 and overwrite its P. A new
+            // head's planes and summaries replace the old ones only after
+            // head_done: its first scores wait until every product of the
+            // blocks before is issued.
             const uint32_t id_sp = idesc_bf16(256, nk + 64, false, false);
             const uint32_t id_s = idesc_bf16(256, nk, false, false);
             const uint32_t id_o = idesc_bf16(256, d, false, true);
-            int j = 0, stage = 0;    // the slot at hand (j & 1)
-            int jo = 1, stageo = 0;  // the other slot
-            int done = 0, hc = 0;  // blocks finished, heads begun
             // The whole warp runs the loop, so that its state and the
             // operands' descriptors are warp-uniform; one lane issues.
             const bool el = elect_one();
-            auto test = [&](uint64_t *bar, uint32_t par) -> bool {
-                return __all_sync(0xffffffffu, mbar_test(bar, par));
+            auto test = [&](PairBar bar, int i, uint32_t par) -> bool {
+                uint64_t *b = bar == PairBar::k_full       ? &bars.k_full[i]
+                              : bar == PairBar::q_full     ? &bars.q_full[i]
+                              : bar == PairBar::v_full     ? &bars.v_full[i]
+                              : bar == PairBar::tmem_empty ? &bars.tmem_empty[i]
+                              : bar == PairBar::p_full     ? &bars.p_full[i]
+                              : bar == PairBar::phi_full   ? &bars.phi_full[i]
+                                                           : &bars.wb_full;
+                return __all_sync(0xffffffffu, mbar_test(b, par));
             };
             const uint64_t dQ = smem_desc(sQ, 16, 1024),
                            dK0 = smem_desc(sK0, 16, 1024),
@@ -435,70 +438,27 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                     if (p == NP - 1) mma_commit_pair(&bars.pv_done[s]);
                 }
             };
+            auto features = [&](int s, int n) {  // O += Phi' B
+                tc_fence_after();
+                const uint32_t so = tm + 256u * s;
+                if (el) {
+#pragma unroll
+                    for (int kk = 0; kk < 16; ++kk)
+                        if (16 * kk < r)
+                            mma_pair_ts(so + nk,
+                                        so + (kk < 8 ? quarter_col(kk, 32)
+                                                     : quarter_col(kk - 8, 0)),
+                                        desc_at(dB, kk * 2048), id_o, 1);
+                    mma_commit_pair(&bars.o_full[s]);
+                    if (last_of_head(n)) mma_commit_pair(&bars.head_done);
+                }
+            };
+            PairOrder order;
             unsigned long long t_last = global_ns();
             uint32_t idle = 0;  // the clock is read every 256 idle rounds
-            while (done < nblk) {
-                bool did = false;
-                if (j < nblk) {
-                    const int s = j & 1, k = j >> 1;
-                    bool go = false;
-                    if (stage == 0) {
-                        const bool nh = new_head(j);
-                        go = !(nh && done < j) &&
-                             test(&bars.k_full[0], j & 1) &&
-                             test(&bars.q_full[s], k & 1) &&
-                             (j < 2 ||
-                              test(&bars.tmem_empty[s], (k - 1) & 1)) &&
-                             (!nh || test(&bars.wb_full, hc & 1));
-                        if (go) {
-                            if (nh) ++hc;
-                            scores(s, 0);
-                        }
-                    } else if (stage == 1) {
-                        go = test(&bars.p_full[s], 0) &&
-                             test(&bars.v_full[0], j & 1);
-                        if (go) values(s, 0);
-                    } else if (stage == 2) {
-                        go = test(&bars.k_full[1], j & 1);
-                        if (go) scores(s, 1);
-                    } else if (stage == 3) {
-                        go = test(&bars.p_full[s], 1) &&
-                             test(&bars.v_full[1], j & 1);
-                        if (go) values(s, 1);
-                    } else {
-                        go = test(&bars.phi_full[s], k & 1);
-                        if (go) {
-                            tc_fence_after();
-                            const uint32_t so = tm + 256u * s;
-                            if (el) {
-#pragma unroll
-                                for (int kk = 0; kk < 16; ++kk)
-                                    if (16 * kk < r)  // O += Phi' B
-                                        mma_pair_ts(
-                                            so + nk,
-                                            so + (kk < 8
-                                                      ? quarter_col(kk, 32)
-                                                      : quarter_col(kk - 8, 0)),
-                                            desc_at(dB, kk * 2048), id_o, 1);
-                                mma_commit_pair(&bars.o_full[s]);
-                                if (last_of_head(done))
-                                    mma_commit_pair(&bars.head_done);
-                            }
-                            ++done;
-                            j += 2;
-                        }
-                    }
-                    if (go) {
-                        stage = stage == 4 ? 0 : stage + 1;
-                        did = true;
-                    }
-                }
-                int x = j;  // the slots take turns
-                j = jo;
-                jo = x;
-                x = stage;
-                stage = stageo;
-                stageo = x;
+            while (order.done < nblk) {
+                const bool did = order.round(nblk, new_head, test, scores,
+                                             values, features);
                 if (did) {
                     idle = 0;
                 } else if ((++idle & 255u) == 0) {
