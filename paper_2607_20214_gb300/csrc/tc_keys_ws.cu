@@ -377,28 +377,28 @@ __global__ void __launch_bounds__(kKwThreads, 2)
 // round: D = V^T Phi, lanes = value dimensions, N = r buckets, so that a tile
 // takes 8 MMAs of N = r where Phi^T [V | 1] takes 16 of N = 144 (which ran at
 // 80 ns each beside the copies and feature stores: shared-memory bandwidth),
-// and the feature tile is handed over per 64 keys. A = Phi^T 1 is summed by
-// four more warps, one per 64 buckets, from the bf16 features that the MMAs
-// read. Live beside the sort hash: c3 103 -> 82 us, c4 412 -> 340 us (with A as
-// MMAs of N = 16 against ones, 0.8 us per tile, 97 us at c3; summed by the
-// feature threads 141). Roles and copies as above.
+// and the feature tile is handed over per 64 keys. A = Phi^T 1 comes from MMAs
+// of N = 16 against ones in the same key steps, so that A and B are sums of the
+// same unit and its truncations cancel in Num / Den. (Summed from the same
+// features by four warps, with rounding to nearest, A is 2.4e-5 larger at
+// N = 64K and d_lr off by 1.36e-4 there instead of 1.13e-4; no faster: 80 us at
+// c3 and 317 at c4 against 80 and 323.) k_race_keys_ws took 103 and 412 us,
+// live beside the sort hash as all of these. Roles and copies as above.
 struct KtBars {
     uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2], w_full, done;
     uint64_t proj_full[2];
     uint64_t phi_full[2], phi_empty[2];  // per 64 keys
 };
 
-constexpr int kKtThreads = kKwThreads + 128;
-
 template <int NT>  // tables per row half, 4 or 8 (L <= 2 NT)
-__global__ void __launch_bounds__(kKtThreads, 1)
+__global__ void __launch_bounds__(kKwThreads, 1)
     k_race_keys_t(const __grid_constant__ CUtensorMap tmK,
                   const __grid_constant__ CUtensorMap tmV,
                   const __grid_constant__ CUtensorMap tmW, int N, int H, int L,
                   int Lg_pad, int chunk, float beta, float *__restrict__ part,
                   DeviceStatus *status) {
     constexpr int d = 128;
-    constexpr uint32_t tileB = 128u * d * 2u, colP = 256;
+    constexpr uint32_t tileB = 128u * d * 2u, colP = 256, colA = 384;
     extern __shared__ unsigned char smem_raw[];
     __shared__ KtBars bars;
     __shared__ uint32_t tbase;
@@ -411,8 +411,9 @@ __global__ void __launch_bounds__(kKtThreads, 1)
     const uint32_t sW = align1k(smem_u32(smem_raw));
     const uint32_t sK0 = sW + align1k(Lg_pad * d * 2);
     const uint32_t sV0 = sK0 + 2 * tileB;
-    const uint32_t sPhi = sV0 + 2 * tileB;
-    const int panels = (r + 63) >> 6;
+    const uint32_t sOnes = sV0 + 2 * tileB;  // [16 x 64], B operand of A
+    const uint32_t sPhi = sOnes + 2048;
+    const int nM = (r + 127) >> 7;
 
     if (warp == 1) tmem_alloc(&tbase, 512);
     if (tid == 0) {
@@ -425,11 +426,17 @@ __global__ void __launch_bounds__(kKtThreads, 1)
             mbar_init(&bars.v_empty[b], 1);
             mbar_init(&bars.proj_full[b], 1);
             mbar_init(&bars.phi_full[b], 128);
-            mbar_init(&bars.phi_empty[b], 1 + panels);
+            mbar_init(&bars.phi_empty[b], 1);
         }
         abort_flag = 0;
         fence_mbar_init();
     }
+    for (int i = tid; i < 2048 / 16; i += kKwThreads)  // bf16 ones
+        asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(
+                         sOnes + i * 16),
+                     "r"(0x3F803F80u)
+                     : "memory");
+    fence_proxy_async_smem();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -485,6 +492,8 @@ __global__ void __launch_bounds__(kKtThreads, 1)
             };
             const uint32_t id_proj = idesc_bf16(128, Lg_pad, false, false);
             const uint32_t id_b = idesc_bf16(128, r, true, true);
+            const uint32_t id_a = idesc_bf16(128, 16, true, false);
+            const uint64_t d1 = smem_desc(sOnes, 16, 1024);
             auto proj = [=](int it) {
                 const uint32_t sK = sK0 + (it & 1) * tileB;
                 const uint32_t dst = t + colP + 64u * (it & 1);
@@ -527,6 +536,14 @@ __global__ void __launch_bounds__(kKtThreads, 1)
                             mma_ss(t, desc_at(da, k * 2048),
                                    desc_at(db, k * 2048), id_b,
                                    k > 0 ? 1u : more);
+#pragma unroll
+                        for (int m = 0; m < 2; ++m)
+                            if (m < nM)
+#pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    mma_ss(t + colA + 16 * m,
+                                           desc_at(db, m * 32768 + k * 2048),
+                                           d1, id_a, k > 0 ? 1u : more);
                         mma_commit(&bars.phi_empty[kh]);
                     }
                 }
@@ -543,55 +560,6 @@ __global__ void __launch_bounds__(kKtThreads, 1)
             if (ok && el) mma_commit(&bars.done);
         }
         __syncwarp();
-    } else if (warp >= 10) {
-        // ------------------------------------------- A of buckets 64 p + ..
-        const int p = warp - 10;
-        if (p < panels) {
-            // lane: 8 buckets (16-byte chunk lane mod 8) of every fourth key
-            const int ch = lane_id & 7, sub = lane_id >> 3;
-            float2 a[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) a[q] = make_float2(0.0f, 0.0f);
-            bool ok = true;
-            for (int i = 0; i < ntiles && ok; ++i)
-                for (int kh = 0; kh < 2 && ok; ++kh) {
-                    ok = __all_sync(0xffffffffu,
-                                    mbar_wait_or_abort(&bars.phi_full[kh],
-                                                       i & 1, abort, status,
-                                                       70));
-                    if (!ok) break;
-                    const uint32_t at = sPhi + p * 16384;
-#pragma unroll 8
-                    for (int x = 0; x < 16; ++x) {
-                        const uint4 v = ld_shared_v4(
-                            at + panel_offset(64 * kh + 4 * x + sub, ch, 128));
-                        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                        for (int q = 0; q < 4; ++q)
-                            a[q] = add2(
-                                a[q],
-                                make_float2(
-                                    __uint_as_float(w[q] << 16),
-                                    __uint_as_float(w[q] & 0xffff0000u)));
-                    }
-                    __syncwarp();
-                    if (lane_id == 0) mbar_arrive(&bars.phi_empty[kh]);
-                }
-            float *outA =
-                part + ((size_t)bh * S + s) * ((size_t)r * d + r) +
-                (size_t)r * d;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-#pragma unroll
-                for (int o = 8; o < 32; o <<= 1) {
-                    a[q].x += __shfl_xor_sync(0xffffffffu, a[q].x, o);
-                    a[q].y += __shfl_xor_sync(0xffffffffu, a[q].y, o);
-                }
-                const int bucket = 64 * p + 8 * ch + 2 * q;
-                if (sub == 0 && ok && ntiles > 0 && bucket < r)
-                    *reinterpret_cast<float2 *>(outA + bucket) = a[q];
-            }
-        }
     } else {
         // ------------------------------------------------------------ features
         const int half = (warp - 2) >> 2;
@@ -657,6 +625,14 @@ __global__ void __launch_bounds__(kKtThreads, 1)
                 for (int j = 0; j < 16; ++j)
                     out[(size_t)(16 * c + j) * d + row] =
                         __uint_as_float(v[j]);
+            }
+            if (half < nM) {  // lane = bucket of tile `half`
+                uint32_t v[16];
+                tmem_ld16(t + lane + colA + 16 * half, v);
+                tmem_wait_ld();
+                const int bucket = 128 * half + row;
+                if (bucket < r)
+                    out[(size_t)r * d + bucket] = __uint_as_float(v[0]);
             }
         } else if (ntiles == 0) {
             for (int i = tid - 64; i < r * d + r; i += 256) out[i] = 0.0f;
@@ -765,12 +741,12 @@ cudaError_t launch_race_keys_ws(const Plan &P, const void *k, const void *v,
     };
     if (P.d == 128 && P.gamma == 4) {
         const size_t sm = 1024 + (size_t)lg_pad * P.d * 2 +
-                          4 * (size_t)128 * P.d * 2 +
-                          (size_t)((P.r + 63) / 64) * 16384;
+                          4 * (size_t)128 * P.d * 2 + 2048 +
+                          (size_t)((P.r + 127) / 128) * 32768;
         auto launch_t = [&](auto kern) {
             cudaFuncSetAttribute(
                 kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-            kern<<<grid, kKtThreads, sm, st>>>(tmK, tmV, tmW, P.N, P.H, P.L,
+            kern<<<grid, kKwThreads, sm, st>>>(tmK, tmV, tmW, P.N, P.H, P.L,
                                                lg_pad, P.chunk, P.beta, part,
                                                status);
             return cudaGetLastError();
