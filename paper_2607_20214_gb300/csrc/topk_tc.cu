@@ -542,6 +542,8 @@ __global__ void __launch_bounds__(kTselThreads, NC <= 256 ? 2 : 1)
 #pragma unroll
                 for (int m = 0; m < MH; ++m) out[m] |= slot[half * MH + m];
             }
+            // the next rows' lanes write the words that these have read
+            __syncwarp();
         }
         uint32_t *dst =
             selmask + ((size_t)bh * N + p0 + row) * M + half * MH;
