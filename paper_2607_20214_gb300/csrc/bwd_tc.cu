@@ -1124,8 +1124,6 @@ cudaError_t launch_bwd_block_tc(const Plan &P, const void *q, const void *k,
     const int S_seg = bwd_tc_segments(P);
     const size_t smem = bwd_tc_smem(P);
     auto launch = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
         return launch_after(
             kern, dim3(grid), kBtThreads, smem, st,
             (const uint16_t *)q, (const uint16_t *)k, (const uint16_t *)v,
@@ -1171,8 +1169,6 @@ cudaError_t launch_bwd_keys_tc(const Plan &P, const void *k, const void *v,
         e = make_tma_map_f32(&tmDV, dv, rows, kBtD, 32, kBtT);
     if (e != cudaSuccess) return e;
     auto launch = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
         return launch_after(kern, dim3(grid), kBtThreads, smem, st, tmK, tmV,
                             tmDK, tmDV, w_bf16, part, S_seg, blk_grid, P.N,
                             P.H, P.beta, tiles_per_head, total, status);

@@ -1126,8 +1126,6 @@ cudaError_t launch_causal_attn(const Plan &P, int level, const void *q,
     if (smem < kSmemPerSM / 3 + 1024) smem = kSmemPerSM / 3 + 1024;
     const int grid = items < 2 * 152 ? items : 2 * 152;
     auto launch = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
         return launch_after(kern, dim3(grid), kCaThreads, smem, st,
                             (const uint16_t *)q, (const uint16_t *)k,
                             (const uint16_t *)v, pq, pk, P.N, m, P.b, items,

@@ -445,8 +445,6 @@ cudaError_t launch_causal_base(const Plan &P, int n_leaf, const void *q,
     if (e == cudaSuccess) e = make_tma_map_bf16(&tmV, v, rows, P.d, 128);
     if (e != cudaSuccess) return e;
     auto launch = [&](auto kern) {
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem);
         return launch_after(kern, dim3(items < sms ? items : sms), kCbThreads,
                             smem, st, tmQ, tmK, tmV, P.N, n_leaf, segs, items,
                             next_item, P.scale, P.eps, RO, RL, status);

@@ -45,6 +45,13 @@ __device__ __forceinline__ void wait_for_stream() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// The error of a runtime call, no longer kept as the thread's last error,
+// where the next <<<>>> launch would find and report it.
+inline cudaError_t taken(cudaError_t e) {
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
+}
+
 // A launch whose grid may be set up while the kernel before it in the stream
 // drains (programmatic dependent launch): it runs up to wait_for_stream(),
 // then waits for that kernel's end, so the launch itself leaves the chain of
@@ -55,6 +62,11 @@ __device__ __forceinline__ void wait_for_stream() {
 template <typename... K, typename... A>
 cudaError_t launch_after(void (*kern)(K...), dim3 grid, int threads,
                          size_t smem, cudaStream_t st, A... args) {
+    if (smem > 0) {
+        const cudaError_t e = cudaFuncSetAttribute(
+            kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return taken(e);
+    }
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
@@ -65,7 +77,7 @@ cudaError_t launch_after(void (*kern)(K...), dim3 grid, int threads,
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, K(args)...);
+    return taken(cudaLaunchKernelEx(&cfg, kern, K(args)...));
 }
 
 // First fault wins; later faults keep the first record.

@@ -796,7 +796,7 @@ cudaError_t launch_block_attn_pair(
     auto launch = [&](auto kern) {
         cudaError_t err = cudaFuncSetAttribute(
             kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (err != cudaSuccess) return err;
+        if (err != cudaSuccess) return taken(err);
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -813,17 +813,17 @@ cudaError_t launch_block_attn_pair(
         int clusters = 0;
         cfg.gridDim = dim3(2 * 76);
         err = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
-        if (err != cudaSuccess) return err;
+        if (err != cudaSuccess) return taken(err);
         if (clusters < 1) return cudaErrorInvalidConfiguration;
         const long ncl = total < clusters ? total : clusters;
         cfg.gridDim = dim3((unsigned)(2 * ncl));
-        return cudaLaunchKernelEx(
+        return taken(cudaLaunchKernelEx(
             &cfg, kern, (const uint16_t *)q, (const uint16_t *)k,
             (const uint16_t *)v, tmW, tmB, perm_q, perm_k, A, lambda_tok,
             gates, P.o32 ? nullptr : (uint16_t *)o,
             P.o32 ? (float *)o : nullptr, log_d_sparse, d_lr, m_sparse, P.N,
             P.H, P.L, P.Lg_pad, P.beta, P.eps, P.scale, P.lambda,
-            P.fusion_mode, bph, total, status);
+            P.fusion_mode, bph, total, status));
     };
     return P.o32 ? launch(k_block_attn_pair<true>)
                  : launch(k_block_attn_pair<false>);
