@@ -471,10 +471,10 @@ __global__ void __launch_bounds__(kKwThreads, 1)
             };
             for (int i = 0; i <= ntiles; ++i) {
                 if (i < ntiles &&
-                    !load(i, bars.k_full, bars.k_empty, sK0, &tmK, 61))
+                    !load(i, bars.k_full, bars.k_empty, sK0, &tmK, 101))
                     break;
                 if (i > 0 &&
-                    !load(i - 1, bars.v_full, bars.v_empty, sV0, &tmV, 62))
+                    !load(i - 1, bars.v_full, bars.v_empty, sV0, &tmV, 102))
                     break;
             }
         }
@@ -510,9 +510,9 @@ __global__ void __launch_bounds__(kKwThreads, 1)
                 mma_commit(&bars.k_empty[it & 1]);
             };
             // projections run two tiles ahead (both TMEM buffers)
-            bool ok = wait(&bars.w_full, 0, 60);
+            bool ok = wait(&bars.w_full, 0, 100);
             for (int it = 0; it < 2 && it < ntiles && ok; ++it) {
-                ok = wait(&bars.k_full[it], 0, 63);
+                ok = wait(&bars.k_full[it], 0, 103);
                 if (ok) {
                     tc_fence_after();
                     proj(it);
@@ -520,9 +520,9 @@ __global__ void __launch_bounds__(kKwThreads, 1)
             }
             for (int i = 0; i < ntiles && ok; ++i) {
                 const int b = i & 1;
-                ok = wait(&bars.v_full[b], (i >> 1) & 1, 66);
+                ok = wait(&bars.v_full[b], (i >> 1) & 1, 106);
                 for (int kh = 0; kh < 2 && ok; ++kh) {
-                    ok = wait(&bars.phi_full[kh], i & 1, 65);
+                    ok = wait(&bars.phi_full[kh], i & 1, 105);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t da = smem_desc(sV0 + b * tileB + kh * 8192,
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(kKwThreads, 1)
                 if (el) mma_commit(&bars.v_empty[b]);
                 if (i + 2 < ntiles) {
                     // the features of tile i have read projection buffer b
-                    ok = wait(&bars.k_full[b], ((i + 2) >> 1) & 1, 64);
+                    ok = wait(&bars.k_full[b], ((i + 2) >> 1) & 1, 104);
                     if (!ok) break;
                     tc_fence_after();
                     proj(i + 2);
@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(kKwThreads, 1)
         bool ok = true;
         for (int i = 0; i < ntiles; ++i) {
             const int b = i & 1;
-            ok = wwait(&bars.proj_full[b], (i >> 1) & 1, 67);
+            ok = wwait(&bars.proj_full[b], (i >> 1) & 1, 107);
             if (!ok) break;
             tc_fence_after();
             float sp[NT * 4];
@@ -590,7 +590,7 @@ __global__ void __launch_bounds__(kKwThreads, 1)
                 tmem_wait_ld();
                 race_factors<16>(pr, beta, sp);
             }
-            if (i >= 1) ok = wwait(&bars.phi_empty[kh], (i - 1) & 1, 68);
+            if (i >= 1) ok = wwait(&bars.phi_empty[kh], (i - 1) & 1, 108);
             if (!ok) break;
             const float one = c0 + i * 128 + row < c1 ? 1.0f : 0.0f;
 #pragma unroll
@@ -614,7 +614,7 @@ __global__ void __launch_bounds__(kKwThreads, 1)
         // partial summaries of this chunk: lane = value dimension; the
         // halves take every other 16 buckets
         float *out = part + ((size_t)bh * S + s) * ((size_t)r * d + r);
-        if (ok && ntiles > 0) ok = wwait(&bars.done, 0, 69);
+        if (ok && ntiles > 0) ok = wwait(&bars.done, 0, 109);
         if (ok && ntiles > 0) {
             tc_fence_after();
             for (int c = half; c < L; c += 2) {

@@ -670,7 +670,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             if (nt0 > 0) write_phi_chunk<G, T>(sp, nt0, ratio, so + cb0);
             if (r > nk) {
                 // over P: its product is complete
-                if (!pwait(&bars.pv_done[g], k & 1, 80)) break;
+                if (!pwait(&bars.pv_done[g], k & 1, 110)) break;
                 tc_fence_after();
                 if (nt1 > 0) {
                     float f1[16];
@@ -682,7 +682,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             }
             tmem_wait_st();
             signal(&bars.phi_full[g]);
-            if (!pwait(&bars.o_full[g], k & 1, 81)) break;
+            if (!pwait(&bars.o_full[g], k & 1, 111)) break;
             tc_fence_after();
             // O = c1 acc, this half's 64 columns: bf16 through this warp's
             // 2 KB, 16 rows at a time, out in 128-byte rows; fp32 from the

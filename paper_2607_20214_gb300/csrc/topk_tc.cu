@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(kTselThreads, NC <= 256 ? 2 : 1)
         }
         const float qn = norms[(size_t)bh * N + p0 + row];
         const float kn = __uint_as_float(kmax_bits[par]);
-        bool ok = mbar_wait(&bar, phase, status, 70);
+        bool ok = mbar_wait(&bar, phase, status, 170);
         if (!__syncthreads_and(ok)) break;
         tc_fence_after();
         if (next < tiles) gather(next, par ^ 1);
