@@ -515,6 +515,15 @@ __global__ void k_copy_summaries(const float *__restrict__ a,
 cudaError_t launch_copy_summaries(const float *a, const float *b, size_t na,
                                   size_t nb, float *oa, float *ob,
                                   cudaStream_t st) {
+    // destinations that no 4-byte store may take are copied by the runtime
+    if (((uintptr_t)oa | (uintptr_t)ob) & 3) {
+        const cudaError_t e = taken(cudaMemcpyAsync(
+            oa, a, na * sizeof(float), cudaMemcpyDeviceToDevice, st));
+        return e != cudaSuccess
+                   ? e
+                   : taken(cudaMemcpyAsync(ob, b, nb * sizeof(float),
+                                           cudaMemcpyDeviceToDevice, st));
+    }
     const size_t want = (nb / 4 + 255) / 256;
     const int grid = (int)(want < 1 ? 1 : want > 1216 ? 1216 : want);
     k_copy_summaries<<<grid, 256, 0, st>>>(a, b, na, nb, oa, ob);
