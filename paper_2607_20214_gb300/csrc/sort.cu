@@ -621,10 +621,19 @@ cudaError_t launch_sort_hash(const Plan &P, const void *q, const void *k,
 // Calls of so few rows that their launches decide.
 bool short_call(const Plan &P) { return (long)P.BH * P.N <= 32768; }
 
-// With many tiles the repeated scans cost more than the launch they save (c2:
-// 1536 tiles, 4 us).
+// Every CTA of the fused launch repeats its head's scan, 16 counts a thread
+// at 2048, so beyond 1024 counts it is worth the launch that it saves only
+// while an SM has one such CTA. Calls of 32768 rows, fused against apart: at
+// 1024 counts 8 heads of 4096 rows, d = 128, 46.7 us (graph 39.0) against 49.5
+// (39.0); at 2048 counts 4 heads of 8192 rows 62.3 (56.4) against 49.4 (41.0),
+// 32 heads of 1024 rows with 8 bits 68.2 (61.5) against 54.8 (45.1). At 2048
+// counts with 64 CTAs (4 heads of 1024 rows, 8 bits, d = 64) 31.7 (22.6)
+// against 34.0 (22.7).
 bool sort_fused(const Plan &P) {
-    return short_call(P) && P.tiles * P.bins <= kFusedScan;
+    const int counts = P.tiles * P.bins;
+    const long ctas = 2L * P.BH * P.tiles;
+    return short_call(P) &&
+           (counts <= 1024 || (counts <= kFusedScan && ctas <= 152));
 }
 
 cudaError_t launch_sort_scan(const Plan &P, int *hist, cudaStream_t st) {
