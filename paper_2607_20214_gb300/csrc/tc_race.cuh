@@ -136,8 +136,14 @@ __device__ __forceinline__ void table_pack4(const float (&u)[4],
 // sum_r phi_r A_r of one gamma = 4 table from its per-bit factors, bit by
 // bit from the highest: A[i] <- q A[i] + p A[i + half], all terms positive as
 // in table_dot4. Fewer operations (7 + 7 in pairs against 8 single and 12 in
-// pairs) in a longer chain: c3's block kernel took 133 us with table_dot4 and
-// 128 with this, but c2's 37 and 39, c5's 106 and 110, and c4's 584 with both.
+// pairs) in a longer chain. The block kernel takes it where one query buffer
+// is in flight and no window is walked. us with table_dot4 and with this, 32
+// heads of 16384 rows, d = 128, r = 256: c3 133 and 128, top-k of one block 164
+// and 161, of two, three and four 226 and 225, 312 and 311, 390 and 391,
+// r = 128 with b = 128, 64 110 and 110, 109 and 109; but a window of three
+// blocks 244 and 255. 48 heads of 8192 rows, d = 64, b = 256: r = 128 105 and
+// 107, r = 256 126 and 124. With three query buffers c2 37 and 39, c5 106 and
+// 110; the pair kernel 584 with both.
 // A: 16 floats, 16-byte aligned, in shared memory.
 __device__ __forceinline__ float table_den4(const float *sp, const float *A) {
     float4 a[4];

@@ -573,7 +573,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                 constexpr int n1 = T * G <= 16 ? 16 : 32;
                 race_factors<n1>(pr, beta, sp);
                 float dacc[4] = {0.0f, 0.0f, 0.0f, 0.0f};  // independent chains
-                constexpr bool fold = QS == 1;  // see table_den4
+                constexpr bool fold = QS == 1 && !WIN;  // see table_den4
                 chunk_den<G, T, fold>(sp, nt0, Asm + ta0 * R, dacc);
                 if constexpr (T * G <= 16) {
                     if (nt1 > 0) {
