@@ -14,14 +14,17 @@
 // anywhere with a bracket lo <= T < hi (count(>= lo) >= k > count(>= hi));
 // the window is then [lo - 2E, hi + 2E].
 //
-// E = 2^-15 |q| max|k|: the chain's own error is at most d 2^-24 sum|q k| <=
-// 2^-17 |q| |k| at d = 128, the MMA's (8 steps of 16 products, aligned to the
-// largest and truncated at 2^-23 or finer of it) about as much again; the
-// bound keeps a factor of two over their sum (the largest |s - e| / (|q| |k|)
-// of 2^26 scores per distribution: 2^-22.3 Gaussian, 2^-20.5 with exponents
-// spread over 2^24, 2^-19.6 with two elements holding the norm). Rows whose
-// norms are not finite, overflow in their squares or are below 1e-15 (where
-// squares and products underflow) are selected by the chain alone.
+// E = 2^-15 |q| max|k| = 3.05e-5 of it. The chain's own error is at most
+// d 2^-24 sum|q k| <= 2^-17 |q| |k| at d = 128 (7.6e-6). For the MMA it is
+// assumed, as its additions are not documented, that each of the 8 steps
+// aligns 16 products and the accumulator to the largest of them, truncates
+// every term at 2^-23 of it or finer and the sum once more: at most 8 * 18 *
+// 2^-23 |q| |k| (1.72e-5). Together 2.48e-5, so E has a margin of 1.2 over what
+// is assumed; samples are well inside (the largest |s - e| / (|q| |k|) of 2^26
+// scores per distribution: 2^-22.3 Gaussian, 2^-20.5 with exponents spread
+// over 2^24, 2^-19.6 with two elements holding the norm). Rows whose norms
+// are not finite, overflow in their squares or are below 1e-15 (where squares
+// and products underflow) are selected by the chain alone.
 //
 // What bounds it: the issue slots of the search (about five passes over the
 // scores at 1.5 FP32 instructions each, one more that makes the masks). Two
@@ -43,7 +46,10 @@ using namespace tc;
 
 constexpr int kTselThreads = 256;
 constexpr int kTselList = 64;    // open candidates of 32 rows, one lane each
-constexpr int kTselLeft = 20;    // the search ends with at most so many
+// The search ends with at most so many open candidates: 10, 20 and 40 take
+// 209, 210 and 223 us at 256 candidates a row, 145, 143 and 151 at 128, 400,
+// 390 and 414 at 384, 487, 492 and 530 at 512 (B2 H16 N16384 d128).
+constexpr int kTselLeft = 20;
 constexpr int kTselRowMax = 8;   // of one row; more: the row's own pass
 constexpr int kTselSteps = 48;   // search steps before the bracket is taken
 
