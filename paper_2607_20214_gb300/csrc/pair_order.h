@@ -17,7 +17,13 @@
 // only when block j - 1's product of the same stage, which waited for the
 // phase before, has been issued. Block j - 1 waits for nothing of block j, so
 // the order cannot stall; the slots are half a block apart, so it hardly costs
-// anything (B1 H32 N65536 d128 r256: 587 us, 584 without it).
+// anything (B1 H32 N65536 d128 r256: 585 us, 584 without it).
+//
+// The scores of pass 1 go over P of pass 0, so they wait until the product
+// that reads it is complete (pv0_done, of the slot: the value buffer's own
+// barrier may be two phases on by then). Products of different accumulators are
+// not documented to run in the order of their issue; relying on it would gain
+// 2 us of the 587.
 #pragma once
 
 #ifdef __CUDACC__
@@ -29,8 +35,8 @@
 namespace elsaa {
 
 // barriers that the issuer tests: per pass (k_full, v_full), per slot, or one
-enum class PairBar { k_full, q_full, v_full, tmem_empty, p_full, phi_full,
-                     wb_full };
+enum class PairBar { k_full, q_full, v_full, pv0_done, tmem_empty, p_full,
+                     phi_full, wb_full };
 
 struct PairOrder {
     int j = 0, stage = 0;    // the slot at hand (j & 1)
@@ -75,7 +81,8 @@ struct PairOrder {
                     ++values0;
                 }
             } else if (stage == 2) {
-                go = issued1 == j && test(PairBar::k_full, 1, j & 1);
+                go = issued1 == j && test(PairBar::k_full, 1, j & 1) &&
+                     test(PairBar::pv0_done, s, k & 1);
                 if (go) {
                     scores(s, 1);
                     ++issued1;

@@ -29,9 +29,9 @@
 // about a third of the issue slots and the products about a quarter of the
 // tensor pipe's), so everything that another slot or pass can cover is off
 // that chain: gathers have warps of their own, the two slots' products are
-// issued independently of each other, the second pass's scores go out right
-// behind the first P V product, P is handed over before the features and
-// the fusion scalars are computed, and all features go to one product: c4
+// issued as they become ready (block by block at each stage: pair_order.h),
+// P is handed over before the features and the fusion scalars are computed,
+// and all features go to one product: c4
 // (B1 H32 N65536 d128 L16) 697 -> 646 us; products issued by a converged warp
 // from descriptors made once, and a lane per relayed barrier: 587 us (0.54 of
 // the measured HBM bandwidth).
@@ -80,7 +80,7 @@ struct PrBars {
     uint64_t tmem_empty[2], p_full[2], phi_full[2];
     // MMA completions, committed to both CTAs
     uint64_t q_empty[2], k_empty[kPrNP], v_empty[kPrNP];
-    uint64_t s_full[2], pv_done[2], o_full[2], head_done;
+    uint64_t s_full[2], pv0_done[2], pv_done[2], o_full[2], head_done;
 };
 constexpr int kPrRelayed = 2 + kPrNP + kPrNP + 1;  // copy barriers
 
@@ -159,6 +159,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
             mbar_init(&bars.p_full[s], 16);
             mbar_init(&bars.phi_full[s], 16);
             mbar_init(&bars.s_full[s], 1);
+            mbar_init(&bars.pv0_done[s], 1);
             mbar_init(&bars.pv_done[s], 1);
             mbar_init(&bars.o_full[s], 1);
         }
@@ -365,11 +366,9 @@ __global__ void __launch_bounds__(kPrThreads, 1)
         } else if (nblk > 0) {
             // ------------------------------------------------- MMA issue
             // Event driven, each slot at a stage of its own: the order is
-            // PairOrder's (pair_order.h). The scores of pass 1 go out right
-            // behind the P V product of pass 0 and overwrite its P. A new
-            // head's planes and summaries replace the old ones only after
-            // head_done: its first scores wait until every product of the
-            // blocks before is issued.
+            // PairOrder's (pair_order.h). A new head's planes and summaries
+            // replace the old ones only after head_done: its first scores
+            // wait until every product of the blocks before is issued.
             const uint32_t id_sp = idesc_bf16(256, nk + 64, false, false);
             const uint32_t id_s = idesc_bf16(256, nk, false, false);
             const uint32_t id_o = idesc_bf16(256, d, false, true);
@@ -380,6 +379,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                 uint64_t *b = bar == PairBar::k_full       ? &bars.k_full[i]
                               : bar == PairBar::q_full     ? &bars.q_full[i]
                               : bar == PairBar::v_full     ? &bars.v_full[i]
+                              : bar == PairBar::pv0_done   ? &bars.pv0_done[i]
                               : bar == PairBar::tmem_empty ? &bars.tmem_empty[i]
                               : bar == PairBar::p_full     ? &bars.p_full[i]
                               : bar == PairBar::phi_full   ? &bars.phi_full[i]
@@ -435,7 +435,8 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                                     desc_at(b, kk * 2048), id_o,
                                     p > 0 || kk > 0);
                     mma_commit_pair(&bars.v_empty[p]);
-                    if (p == NP - 1) mma_commit_pair(&bars.pv_done[s]);
+                    mma_commit_pair(p == 0 ? &bars.pv0_done[s]
+                                           : &bars.pv_done[s]);
                 }
             };
             auto features = [&](int s, int n) {  // O += Phi' B
@@ -627,7 +628,7 @@ __global__ void __launch_bounds__(kPrThreads, 1)
                 // online softmax: keep the running reference unless the
                 // row's max grew by more than 2^8; then rescale the
                 // accumulator (the previous P V product is complete: these
-                // scores were issued behind it) and the running sum
+                // scores waited for it) and the running sum
                 const bool need = M2b > M2 + 8.0f;
                 const float f = need ? ex2_approx(M2 - M2b) : 1.0f;
                 if (__any_sync(0xffffffffu, need)) {

@@ -40,7 +40,7 @@ struct Run {
     std::vector<Event> events;
     Bar k_full[2], q_full[2], v_full[2], wb_full, tmem_empty[2], p_full[2],
         phi_full[2], q_empty[2], k_empty[2], v_empty[2], s_full[2],
-        pv_done[2], o_full[2], head_done;
+        pv0_done[2], pv_done[2], o_full[2], head_done;
     int k[2] = {-1, -1}, q[2] = {-1, -1}, v[2] = {-1, -1}, wb = -1;
     const char *fault = nullptr;
     long mma_free = 0;  // products end in the order of their issue
@@ -139,6 +139,7 @@ struct Run {
                 case PairBar::k_full: return k_full[i].test(par);
                 case PairBar::q_full: return q_full[i].test(par);
                 case PairBar::v_full: return v_full[i].test(par);
+                case PairBar::pv0_done: return pv0_done[i].test(par);
                 case PairBar::tmem_empty: return tmem_empty[i].test(par);
                 case PairBar::p_full: return p_full[i].test(par);
                 case PairBar::phi_full: return phi_full[i].test(par);
@@ -154,6 +155,9 @@ struct Run {
                 expect(wb == j / per_head, "planes that are not there");
                 expect(tmem_empty[s].phases >= j >> 1,
                        "scores over an output that is not read");
+            } else {
+                expect(pv0_done[s].phases == (j >> 1) + 1,
+                       "scores over a P that is still read");
             }
             product([this, s, p, j] {
                 expect(k[p] == j && q[s] == j, "operands overwritten");
@@ -170,7 +174,7 @@ struct Run {
             product([this, s, p, j] {
                 expect(v[p] == j, "values overwritten");
                 ++v_empty[p].phases;
-                if (p == 1) ++pv_done[s].phases;
+                ++(p ? pv_done : pv0_done)[s].phases;
             });
         };
         auto features = [&](int s, int n) {
