@@ -325,12 +325,13 @@ __global__ void __launch_bounds__(kWsThreads, 1)
             // Event driven: each round issues whichever MMA group is ready,
             // the oldest tile's first (Phi'B, then P V, then the next
             // scores), so one slot's epilogue never holds back the other
-            // slot's products. Units: (tile, pass); a tile's later scores go
-            // out right behind its previous P V product (which reads P from
-            // the S columns): products run in the order of their issue.
-            // Waiting for that product's completion took 229 us against 226
-            // at c3 with two passes (top-k); two tiles' passes in turn, with
-            // a second query buffer, 259.
+            // slot's products. Units: (tile, pass); a tile's later scores
+            // wait for its previous P V product, which reads P from the S
+            // columns. (Sent out right behind it they took 226 us against 233
+            // at c3 with two passes (top-k), but products of different
+            // accumulators are not documented to run in the order of their
+            // issue; two tiles' passes in turn, with a second query buffer,
+            // took 259.)
             const uint32_t id_sp = idesc_bf16(128, NR, false, false);
             const uint32_t id_s = idesc_bf16(128, nk, false, false);
             const uint32_t id_o = idesc_bf16(128, d, false, true);
@@ -421,9 +422,12 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                                                      ((ts >> 1) - 1) & 1)) &&
                                 (!nh || test(&bars.wb_full, hc & 1));
                     // the S columns hold P of the pass before: its product
-                    // is issued, and products run in the order of their
-                    // issue
-                    if (spass > 0) ready = ready && up == us;
+                    // must be complete. (That stage's barrier cannot run on:
+                    // its next phase is a later unit's product.)
+                    if (spass > 0)
+                        ready = ready && up == us &&
+                                test(&bars.v_empty[(us - 1) % VS],
+                                     (us - 1) / VS & 1);
                     if (ready) {
                         if (nh) ++hc;
                         fence_proxy_async_smem();  // cp.async data -> MMA
@@ -724,7 +728,7 @@ __global__ void __launch_bounds__(kWsThreads, 1)
                         // online softmax: keep the running reference unless
                         // the row's max grew by more than 2^8; then rescale
                         // the accumulator (the previous P V product is
-                        // complete: these scores were issued behind it) and
+                        // complete: these scores waited for it) and
                         // the running sum. From an empty start (M2 = -inf) the
                         // factor is 0.
                         const bool need = M2b > M2 + 8.0f;
