@@ -11,8 +11,8 @@
 //                   maximum nor the sum needs another thread
 //   warp 8          issues every MMA: S = Q K^T, O += P V (P from TMEM)
 //   warp 9          takes the items, TMA loads of Q, K (two buffers), V (two)
-// TMEM: S_s (then P_s over it) at 128 s, O_s at 256 + 128 s. O stays in
-// tensor memory; a softmax warp rescales it when the maximum of one of its
+// TMEM: S_s at 128 s, O_s at 256 + 128 s, P_s behind O_s at D = 64, over S_s at
+// D = 128. O stays in tensor memory; a softmax warp rescales it when the maximum of one of its
 // rows grows. (Only beyond 2^8 it was no faster, and off by up to 2.5 times as
 // much in peaked heads: the weight of the largest key is exactly 1 only
 // against its own maximum; otherwise bf16 rounds it.)
@@ -160,10 +160,15 @@ __global__ void __launch_bounds__(kCbThreads, 1)
         } else if (warp == 8) {
             // ---------------------------------------------------- MMA issue
             // Whenever a slot's P is ready: its P V product, and right behind
-            // it the scores of its next key tile over the same columns. The
-            // products of one thread run in the order they are issued, so
-            // the scores need no wait for the product before them (with one,
-            // 518 us).
+            // it the scores of its next key tile; the softmax sees these only
+            // when both are complete (a commit covers all that was issued
+            // before it). At D = 128 the scores go over P. That relies on the
+            // two products running in the order of their issue, as products
+            // of one thread do on this chip, though it is documented for
+            // products of one accumulator only; a wait for the P V product
+            // takes 539 us instead of 465 (B2 H16 N16384, 4096-row segments)
+            // and there are no other columns. At D = 64 P has columns of its
+            // own.
             // The whole warp runs the loop, so that its state and the
             // operands' descriptors are warp-uniform; one lane issues.
             const bool el = elect_one();
@@ -225,7 +230,8 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                 auto step = [&](auto slot, int &us, int &up, int &gp, int go,
                                 int n, int us_o, int up_o, int n_o) {
                     constexpr int s = decltype(slot)::value;
-                    constexpr uint32_t cS = 128u * s, cO = cS + 256u;
+                    constexpr uint32_t cO = 128u * s + 256u;
+                    constexpr uint32_t cP = D == 64 ? cO + 64 : 128u * s;
                     const int st = (c0 + up) & 1;
                     if (up == us || !test(&bars.p_full[s], gp & 1) ||
                         !test(&bars.v_full[st], ((c0 + up) >> 1) & 1) ||
@@ -238,7 +244,7 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                     if (el) {
 #pragma unroll
                         for (int x = 0; x < 8; ++x)
-                            mma_ts(tm + cO, tm + cS + 8 * x, v + 128 * x, id_o,
+                            mma_ts(tm + cO, tm + cP + 8 * x, v + 128 * x, id_o,
                                    x > 0 ? 1u : more);
                         mma_commit(&bars.o_done[s]);
                         if (up >= n_o || up_o > up)
@@ -284,6 +290,7 @@ __global__ void __launch_bounds__(kCbThreads, 1)
         const int s = warp >> 2, row = (warp & 3) * 32 + lane_id;
         const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t tS = tm + lane + 128u * s, tO = tS + 256u;
+        const uint32_t tP = D == 64 ? tO + 64 : tS;
         const float sl2 = scale * kLog2e;
         const float2 sl22 = make_float2(sl2, sl2);
         auto wwait = [=](uint64_t *bar, uint32_t par, int site) {
@@ -384,7 +391,7 @@ __global__ void __launch_bounds__(kCbThreads, 1)
                         ls[(q >> 1) & 1] = add2(ls[(q >> 1) & 1], p);
                         pw[q >> 1] = pack_bf16x2(p.x, p.y);
                     }
-                    tmem_st16(tS + c / 2, pw);
+                    tmem_st16(tP + c / 2, pw);
                 }
                 lsum += (ls[0].x + ls[1].x) + (ls[0].y + ls[1].y);
                 tmem_wait_st();
