@@ -49,7 +49,7 @@ struct __align__(sizeof(X) * CPL) RowPiece {
 // loaded whole, kU at a time; the additions stay in sorted order. The row
 // norms of 32 rows are reduced together (one shuffle per row). Bound by the
 // read of Q and K: one thread per column and two-byte loads took 132 us at
-// B2 H16 N16384 d128, this kernel 85 us (beside the RACE key side in both).
+// B2 H16 N16384 d128, this kernel 67 us (beside the RACE key side in both).
 template <typename X, int CPL>
 __global__ void __launch_bounds__(kSelThreads)
     k_topk_sums(const X *__restrict__ qx, const X *__restrict__ kx,
@@ -582,7 +582,14 @@ cudaError_t launch_topk(int stage, const Plan &P, const void *q,
         }
     }
     if (stage == 1) {
-        // eight query blocks per CTA while their scores fit 83 KB
+        // Eight query blocks per CTA while their scores fit 83 KB; two where
+        // eight would leave most SMs idle and a block has few keys' sums to
+        // read. us with one block per CTA, eight, two (d = 128, c = 2): one
+        // head of 128 blocks 10.1, 12.2, 10.2; four of 64 10.0, 12.0, 10.0;
+        // eight of 64 11.8, 12.1, 10.7; one of 512 41, 20, 27; sixteen of
+        // 64 16.9, 12.2, 12.2; eight of 128 24, 12, 16; one of 2048 485, 107,
+        // 310.
+        const bool few = T <= 128 && (long)P.BH * T <= 512;
         auto run = [&](auto kern, int G) {
             const size_t csm = (size_t)G * P.d * 4 + (size_t)G * T * 5;
             cudaFuncSetAttribute(kern,
@@ -592,7 +599,8 @@ cudaError_t launch_topk(int stage, const Plan &P, const void *q,
                 sums, T, P.d, P.tk_c, cand);
             return cudaGetLastError();
         };
-        return T <= 2048 ? run(k_topk_cand<8>, 8) : run(k_topk_cand<2>, 2);
+        return T <= 2048 && !few ? run(k_topk_cand<8>, 8)
+                                 : run(k_topk_cand<2>, 2);
     }
     if (topk_tc_supported(P))
         return launch_topk_select_tc(P, q, k, perm_q, perm_k, cand, norms,
