@@ -381,9 +381,9 @@ __global__ void __launch_bounds__(kKwThreads, 2)
 // of N = 16 against ones in the same key steps, so that A and B are sums of the
 // same unit and its truncations cancel in Num / Den. (Summed from the same
 // features by four warps, with rounding to nearest, A is 2.4e-5 larger at
-// N = 64K and d_lr off by 1.36e-4 there instead of 1.13e-4; no faster: 80 us at
-// c3 and 317 at c4 against 80 and 323.) k_race_keys_ws took 103 and 412 us,
-// live beside the sort hash as all of these. Roles and copies as above.
+// N = 64K and d_lr off by 1.36e-4 there instead of 1.13e-4; c3 took 82 us and c4
+// 340 so.) k_race_keys_ws took 103 and 412 us, this kernel takes 84 and 345, all
+// live beside the sort hash. Roles and copies as above.
 struct KtBars {
     uint64_t k_full[2], k_empty[2], v_full[2], v_empty[2], w_full, done;
     uint64_t proj_full[2];
